@@ -1,4 +1,4 @@
-// CUDA-core kernels: append (a0), fp32-accurate attention (a1) and score (a2) for fp32 inputs
+// CUDA-core kernels: fp32-accurate append + attention (a0, a1) and score (a2) for fp32 inputs
 // (and, as a diagnostic, bf16 inputs).
 #pragma once
 #include "geom.cuh"
@@ -6,152 +6,297 @@
 
 namespace kvc {
 
-// ------------------------------------------------------------------------------------------------
-// a0 append (Alg. 1: C <- C u (K_i, V_i)).  One warp per (token, kv-head) row: copies the K and V
-// rows into cache rows n_c + t and records the absolute position.
-// grid (ceil(n*Hkv / 8), 1, nl), block 256.
+// Both kernels below are register-tiled products on the FMA pipes (packed fp32: one instruction, two IEEE fused
+// multiply-adds).  A warp is a 4 x 8 grid of lanes: lane (rg, kg) holds rows rg, rg + 4, ... of the row tile and keys
+// kg, kg + 8, ... of the key tile, so that an operand row is one 16-byte shared-memory read for four or eight lanes at
+// once (row stride D + 4 floats: the distinct rows of one read lie on different banks) and feeds 2 .. 8 products.
+static constexpr int kCcThreads = 256, kCcWarps = 8;
+
+__device__ __forceinline__ ulonglong2 lds_f32x4(const float* s) { return *reinterpret_cast<const ulonglong2*>(s); }
+
+// Eight or four consecutive elements to shared memory as fp32: fp32 asynchronously (cp.async), bf16 through registers.
 template <typename T>
-__global__ void __launch_bounds__(256) append_kernel(const T* __restrict__ k, const T* __restrict__ v,
-                                                     char* __restrict__ cache, Geom p) {
-  pdl_launch_dependents();                 // the attention kernel may set itself up meanwhile
-  pdl_wait();                              // the previous block's compaction still reads and writes this cache
-  if (threadIdx.x == 0) stamp_begin(p);
-  const int layer = blockIdx.z;
-  const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (row < p.n * p.Hkv) {
-    const int t = row / p.Hkv, g = row % p.Hkv;
-    char* blob = cache + layer * p.cache_ls;
-    const int vec_per_row = p.d * (int)sizeof(T) / 16;
-    const uint4* ksrc = reinterpret_cast<const uint4*>(k + layer * p.kv_ls + (static_cast<long long>(t) * p.Hkv + g) * p.d);
-    const uint4* vsrc = reinterpret_cast<const uint4*>(v + layer * p.kv_ls + (static_cast<long long>(t) * p.Hkv + g) * p.d);
-    const long long dst_row = static_cast<long long>(g) * p.cap + p.n_c + t;
-    uint4* kdst = reinterpret_cast<uint4*>(blob + dst_row * p.d * sizeof(T));
-    uint4* vdst = reinterpret_cast<uint4*>(blob + p.v_off + dst_row * p.d * sizeof(T));
-    for (int i = lane; i < vec_per_row; i += 32) {
-      kdst[i] = ksrc[i];
-      vdst[i] = vsrc[i];
-    }
-    if (lane == 0) reinterpret_cast<int*>(blob + p.pos_off)[dst_row] = static_cast<int>(p.pos0 + t);
+__device__ __forceinline__ void stage16(float* dst, const T* src) {
+  if constexpr (sizeof(T) == 4) {
+    cp_async16(dst, src);
+  } else {
+    const uint4 raw = *reinterpret_cast<const uint4*>(src);
+    reinterpret_cast<float4*>(dst)[0] = make_float4(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u),
+                                                    __uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u));
+    reinterpret_cast<float4*>(dst)[1] = make_float4(__uint_as_float(raw.z << 16), __uint_as_float(raw.z & 0xffff0000u),
+                                                    __uint_as_float(raw.w << 16), __uint_as_float(raw.w & 0xffff0000u));
   }
-  __syncthreads();
-  if (threadIdx.x == 0) stamp_end(p);
+}
+
+template <typename T> __device__ __forceinline__ void store4(T* dst, float4 v);
+template <> __device__ __forceinline__ void store4<float>(float* dst, float4 v) { *reinterpret_cast<float4*>(dst) = v; }
+template <> __device__ __forceinline__ void store4<__nv_bfloat16>(__nv_bfloat16* dst, float4 v) {
+  *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w));
 }
 
 // ------------------------------------------------------------------------------------------------
-// a1 attention on CUDA cores (Eq. 1), fp32 arithmetic throughout.
-// Block = 4 warps x 4 rows = 16 tokens of one query head; keys/values stream through shared memory
-// 32 at a time.  In the score phase lane j owns key j of the tile; in the PV phase lane c owns
-// output columns c, c+32, ....  grid (ceil(n/16), Hq, nl), block 128.
-template <typename T, int D>
-__global__ void __launch_bounds__(128) attn_cc_kernel(const T* __restrict__ q, const char* __restrict__ cache,
-                                                      T* __restrict__ out, char* __restrict__ ws, Geom p) {
-  constexpr int RW = 4, KT = 32, KS = D + 4, NC = D / 32;
-  __shared__ __align__(16) float sK[KT * KS];
-  __shared__ __align__(16) float sV[KT * D];
-  __shared__ __align__(16) float sQ[16 * D];
+// a0 + a1 on CUDA cores: append (Alg. 1: C <- C u (K_i, V_i)) and attention (Eq. 1), fp32 arithmetic throughout.
+// The G query heads of a kv-head are stacked with the tokens (row = token * G + head), a CTA takes BM rows.  Its eight
+// warps share the rows and split the KEYS: warp w of cluster rank s takes key tiles s*8 + w, + 8*S, ... with a running
+// maximum, row sums and an output of its own, which are merged in shared memory at the end.  So no warp waits for
+// another inside the loop, and a launch with few rows still fills the SMs.  Bound: with many rows the FMA pipe (4608
+// rows, 1088 keys, d = 128: 48 us, 1.9 GFLOP at 39 TFLOP/s, where one key per lane and shuffled probabilities took
+// 154 us), with few the latency of a step (256 rows, 192 keys, d = 64: 5.6 us against 23 us for 16 CTAs that each walked
+// all keys), by device stamps.  The next K tile is fetched (cp.async) while the current one's
+// P V is computed, the next V tile behind the scores.  Keys are the cache rows [0, n_c) followed by the block's own
+// tokens, read from the inputs; the CTAs of a kv-head copy the block's rows into the cache on the side.
+// grid (ceil(n*G/BM) * S, Hkv, nl), cluster (S,1,1) with S a power of two, block 256, dynamic smem AttnCc::kBytes.
+template <int D, int BM>
+struct AttnCc {
+  static constexpr int KT = D == 128 ? 16 : 32;            // keys per warp and step
+  static constexpr int KS = D + 4, PS = KT + 4;            // row strides (floats) of Q / K and of P
+  static constexpr int kWarpFloats = KT * KS + KT * D;     // a warp's K and V tile; holds its O at the end
+  static_assert(kWarpFloats >= BM * D, "a warp's O overlays its K and V tiles");
+  static constexpr int kBytes = (BM * KS + kCcWarps * BM * PS + kCcWarps * kWarpFloats + 3 * kCcWarps * BM) * 4;
+};
+
+template <typename T, int D, int BM>
+__global__ void __launch_bounds__(kCcThreads, 1) attn_cc_kernel(const T* __restrict__ q, const T* __restrict__ k,
+                                                                const T* __restrict__ v, char* __restrict__ cache,
+                                                                T* __restrict__ out, char* __restrict__ ws, Geom p, int S) {
+  using L = AttnCc<D, BM>;
+  constexpr int KT = L::KT, KS = L::KS, PS = L::PS, RT = BM / 4, JT = KT / 8, CT = D / 32;
+  constexpr int EPC = 16 / (int)sizeof(T), CPR = D / EPC;  // elements per 16-byte piece, pieces per row
+  extern __shared__ __align__(16) float smem_f[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rg = lane >> 3, kg = lane & 7;
+  float* sQ = smem_f;                                       // [BM][KS]; at the end this CTA's merged rows
+  float* sP = sQ + BM * KS + warp * BM * PS;                // [BM][PS] of this warp
+  float* bufs = sQ + BM * KS + kCcWarps * BM * PS;
+  float* sK = bufs + warp * L::kWarpFloats;                 // [KT][KS]
+  float* sV = sK + KT * KS;                                 // [KT][D]
+  float* sM = bufs + kCcWarps * L::kWarpFloats;             // [8][BM] the warps' maxima, later their weights
+  float* sL = sM + kCcWarps * BM;                           // [8][BM] row sums
+  float* sA = sL + kCcWarps * BM;                           // [2][BM] merged maximum and sum
+
+  const int layer = blockIdx.z, g = blockIdx.y;
+  const int split = S > 1 ? static_cast<int>(cluster_ctarank()) : 0;
+  const int tile = static_cast<int>(gridDim.x) / S - 1 - static_cast<int>(blockIdx.x) / S;   // longest rows first
+  const int row0 = tile * BM, rows = p.n * p.G;
+  char* blob = cache + layer * p.cache_ls;
+  T* Kc = reinterpret_cast<T*>(blob) + static_cast<long long>(g) * p.cap * D;
+  T* Vc = reinterpret_cast<T*>(blob + p.v_off) + static_cast<long long>(g) * p.cap * D;
+  const long long in_stride = static_cast<long long>(p.Hkv) * D;
+  const T* Kn = k + layer * p.kv_ls + static_cast<long long>(g) * D;
+  const T* Vn = v + layer * p.kv_ls + static_cast<long long>(g) * D;
+  const T* qb = q + layer * p.q_ls + static_cast<long long>(g) * p.G * D;
+  auto row_off = [&](int r) { return (static_cast<long long>(r / p.G) * p.Hq + r % p.G) * D; };   // row r of q / out
+
+  pdl_launch_dependents();
+  pdl_wait();                                               // the previous block's compaction is done with the cache
   if (threadIdx.x == 0) stamp_begin(p);
-  const int layer = blockIdx.z, h = blockIdx.y, g = h / p.G;
-  const int tok0 = blockIdx.x * 16;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const char* blob = cache + layer * p.cache_ls;
-  const T* Kc = reinterpret_cast<const T*>(blob) + static_cast<long long>(g) * p.cap * D;
-  const T* Vc = reinterpret_cast<const T*>(blob + p.v_off) + static_cast<long long>(g) * p.cap * D;
-  const T* qb = q + layer * p.q_ls;
 
-  for (int i = threadIdx.x; i < 16 * D; i += 128) {
-    const int r = i / D, c = i % D, tok = tok0 + r;
-    sQ[i] = tok < p.n ? to_f32<T>(qb[(static_cast<long long>(tok) * p.Hq + h) * D + c]) : 0.f;
+  const int kv_end = p.n_c + (min(row0 + BM, rows) - 1) / p.G + 1;     // keys the last row of this CTA sees
+  const int n_tiles = (kv_end + KT - 1) / KT;
+  // (rows past the last visible key: a copy of it, masked below)
+  auto fetch = [&](float* dst, int stride, const T* cached, const T* fresh, int kt) {
+    if (kt < n_tiles) {
+#pragma unroll
+      for (int i = 0; i < KT * CPR / 32; ++i) {
+        const int r = (lane + 32 * i) / CPR, c = (lane + 32 * i) % CPR * EPC;
+        const int key = min(kt * KT + r, kv_end - 1);
+        const T* src = key < p.n_c ? cached + static_cast<long long>(key) * D : fresh + (key - p.n_c) * in_stride;
+        stage16<T>(dst + r * stride + c, src + c);
+      }
+    }
+    cp_async_commit();
+  };
+  const int step = S * kCcWarps;
+  int kt = split * kCcWarps + warp;
+  for (int i = threadIdx.x; i < BM * CPR; i += kCcThreads) {
+    const int r = i / CPR, c = i % CPR * EPC;
+    stage16<T>(sQ + r * KS + c, qb + row_off(min(row0 + r, rows - 1)) + c);
+  }
+  fetch(sK, KS, Kc, Kn, kt);
+  fetch(sV, D, Vc, Vn, kt);
+  // a0: warp w of CTA x copies tokens 8x + w, ...: one row of K and one of V each
+  for (int t = blockIdx.x * kCcWarps + warp; t < p.n; t += gridDim.x * kCcWarps) {
+    const long long dst = p.n_c + t;
+    if (lane < CPR) {
+      reinterpret_cast<uint4*>(Kc + dst * D)[lane] = reinterpret_cast<const uint4*>(Kn + t * in_stride)[lane];
+      reinterpret_cast<uint4*>(Vc + dst * D)[lane] = reinterpret_cast<const uint4*>(Vn + t * in_stride)[lane];
+    }
+    if (lane == 0) reinterpret_cast<int*>(blob + p.pos_off)[static_cast<long long>(g) * p.cap + dst] = static_cast<int>(p.pos0 + t);
   }
 
-  float m[RW], l[RW], acc[RW][NC];
+  int lim[RT];                                              // visible keys of the thread's rows (causal inside the block)
+  float m[RT], l[RT];
+  uint64_t acc[RT][2 * CT];                                 // columns (kg + 8c)*4 .. +3 of every row, in pairs
 #pragma unroll
-  for (int r = 0; r < RW; ++r) {
-    m[r] = -INFINITY; l[r] = 0.f;
+  for (int i = 0; i < RT; ++i) {
+    const int r = row0 + rg + 4 * i;
+    lim[i] = r < rows ? p.n_c + r / p.G + 1 : 0;
+    m[i] = -INFINITY; l[i] = 0.f;
 #pragma unroll
-    for (int c = 0; c < NC; ++c) acc[r][c] = 0.f;
+    for (int c = 0; c < 2 * CT; ++c) acc[i][c] = 0ull;
   }
-  const int last_tok = min(tok0 + 16, p.n) - 1;
-  const int kv_end = p.n_c + last_tok + 1;          // keys visible to the last row of this block
+  const int lim_min = row0 + BM <= rows ? p.n_c + row0 / p.G + 1 : 0;
+  cp_async_wait<1>();                                       // Q and the first K tile have landed
+  __syncthreads();
 
-  for (int t0 = 0; t0 < kv_end; t0 += KT) {
-    __syncthreads();
-    for (int i = threadIdx.x; i < KT * D; i += 128) {
-      const int j = i / D, c = i % D, key = t0 + j;
-      float kk = 0.f, vv = 0.f;
-      if (key < kv_end) {
-        kk = to_f32<T>(Kc[static_cast<long long>(key) * D + c]);
-        vv = to_f32<T>(Vc[static_cast<long long>(key) * D + c]);
-      }
-      sK[j * KS + c] = kk;
-      sV[j * D + c] = vv;
-    }
-    __syncthreads();
-
-    float s[RW];
+  for (; kt < n_tiles; kt += step) {
+    cp_async_wait<1>();
+    __syncwarp();
+    uint64_t s2[RT][JT];
 #pragma unroll
-    for (int r = 0; r < RW; ++r) s[r] = 0.f;
-    const float4* krow = reinterpret_cast<const float4*>(&sK[lane * KS]);
-#pragma unroll 8
-    for (int c4 = 0; c4 < D / 4; ++c4) {
-      const float4 kv = krow[c4];
+    for (int i = 0; i < RT; ++i)
 #pragma unroll
-      for (int r = 0; r < RW; ++r) {
-        const float4 qv = reinterpret_cast<const float4*>(&sQ[(warp * RW + r) * D])[c4];
-        s[r] = fmaf(qv.x, kv.x, s[r]); s[r] = fmaf(qv.y, kv.y, s[r]);
-        s[r] = fmaf(qv.z, kv.z, s[r]); s[r] = fmaf(qv.w, kv.w, s[r]);
-      }
-    }
-    const int key = t0 + lane;
-    float pr[RW];
-#pragma unroll
-    for (int r = 0; r < RW; ++r) {
-      const int tok = tok0 + warp * RW + r;
-      const bool vis = tok < p.n && key < p.n_c + tok + 1;     // causal inside the block only
-      const float t = vis ? s[r] * p.scale_log2 : -INFINITY;
-      float tmax = t;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
-      const float m_new = fmaxf(m[r], tmax);
-      float pv = 0.f, corr = 1.f;
-      if (m_new != -INFINITY) {
-        pv = exp2f(t - m_new);
-        corr = exp2f(m[r] - m_new);
-      }
-      float psum = pv;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) psum += __shfl_xor_sync(0xffffffffu, psum, o);
-      l[r] = l[r] * corr + psum;
-      m[r] = m_new;
-#pragma unroll
-      for (int c = 0; c < NC; ++c) acc[r][c] *= corr;
-      pr[r] = pv;
-    }
+      for (int j = 0; j < JT; ++j) s2[i][j] = 0ull;
 #pragma unroll 4
-    for (int j = 0; j < KT; ++j) {
-      float vj[NC];
+    for (int c = 0; c < D; c += 4) {
+      ulonglong2 b[JT];
 #pragma unroll
-      for (int c = 0; c < NC; ++c) vj[c] = sV[j * D + lane + 32 * c];
+      for (int j = 0; j < JT; ++j) b[j] = lds_f32x4(sK + (kg + 8 * j) * KS + c);
 #pragma unroll
-      for (int r = 0; r < RW; ++r) {
-        const float pj = __shfl_sync(0xffffffffu, pr[r], j);
+      for (int i = 0; i < RT; ++i) {
+        const ulonglong2 a = lds_f32x4(sQ + (rg + 4 * i) * KS + c);
 #pragma unroll
-        for (int c = 0; c < NC; ++c) acc[r][c] = fmaf(pj, vj[c], acc[r][c]);
+        for (int j = 0; j < JT; ++j) { s2[i][j] = fma_f32x2(a.x, b[j].x, s2[i][j]); s2[i][j] = fma_f32x2(a.y, b[j].y, s2[i][j]); }
       }
     }
+    __syncwarp();
+    fetch(sK, KS, Kc, Kn, kt + step);
+    const bool masked = (kt + 1) * KT > lim_min;
+    bool grew = false;
+    float corr[RT];
+#pragma unroll
+    for (int i = 0; i < RT; ++i) {
+      float s[JT], mx = -INFINITY;
+#pragma unroll
+      for (int j = 0; j < JT; ++j) {
+        float lo, hi;
+        f32x2_split(s2[i][j], lo, hi);
+        s[j] = (lo + hi) * p.scale_log2;
+        if (masked && kt * KT + kg + 8 * j >= lim[i]) s[j] = -INFINITY;
+        mx = fmaxf(mx, s[j]);
+      }
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      const float m_new = fmaxf(m[i], mx);
+      const float m_use = m_new == -INFINITY ? 0.f : m_new;
+      corr[i] = exp2f(m[i] - m_use);
+      grew |= m_new > m[i];
+      m[i] = m_new;
+      l[i] *= corr[i];
+#pragma unroll
+      for (int j = 0; j < JT; ++j) {
+        const float e = exp2f(s[j] - m_use);
+        l[i] += e;
+        sP[(rg + 4 * i) * PS + kg + 8 * j] = e;
+      }
+    }
+    if (__any_sync(0xffffffffu, grew)) {
+#pragma unroll
+      for (int i = 0; i < RT; ++i) {
+        const uint64_t f = f32x2(corr[i], corr[i]);
+#pragma unroll
+        for (int c = 0; c < 2 * CT; ++c) acc[i][c] = mul_f32x2(acc[i][c], f);
+      }
+    }
+    cp_async_wait<1>();                                     // the V tile
+    __syncwarp();
+#pragma unroll 2
+    for (int j = 0; j < KT; j += 4) {
+      float4 pr[RT];
+#pragma unroll
+      for (int i = 0; i < RT; ++i) pr[i] = *reinterpret_cast<const float4*>(sP + (rg + 4 * i) * PS + j);
+#pragma unroll
+      for (int jj = 0; jj < 4; ++jj) {
+        ulonglong2 vv[CT];
+#pragma unroll
+        for (int c = 0; c < CT; ++c) vv[c] = lds_f32x4(sV + (j + jj) * D + (kg + 8 * c) * 4);
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+          const float pv = jj == 0 ? pr[i].x : jj == 1 ? pr[i].y : jj == 2 ? pr[i].z : pr[i].w;
+          const uint64_t pp = f32x2(pv, pv);
+#pragma unroll
+          for (int c = 0; c < CT; ++c) { acc[i][2 * c] = fma_f32x2(pp, vv[c].x, acc[i][2 * c]); acc[i][2 * c + 1] = fma_f32x2(pp, vv[c].y, acc[i][2 * c + 1]); }
+        }
+      }
+    }
+    __syncwarp();
+    fetch(sV, D, Vc, Vn, kt + step);
   }
+  cp_async_wait<0>();
+  __syncwarp();
 
-  float* lse = reinterpret_cast<float*>(ws_slot(ws, p, layer) + p.lse_off);
-  T* ob = out + layer * p.out_ls;
+  // merge the warps' partial results: every warp leaves its O over its tiles, and (m, l) beside it
 #pragma unroll
-  for (int r = 0; r < RW; ++r) {
-    const int tok = tok0 + warp * RW + r;
-    if (tok >= p.n) continue;
-    const float inv = 1.f / l[r];
+  for (int i = 0; i < RT; ++i) {
+    const int r = rg + 4 * i;
 #pragma unroll
-    for (int c = 0; c < NC; ++c)
-      ob[(static_cast<long long>(tok) * p.Hq + h) * D + lane + 32 * c] = from_f32<T>(acc[r][c] * inv);
-    if (lane == 0) lse[static_cast<long long>(tok) * p.Hq + h] = (m[r] + log2f(l[r])) * 0.6931471805599453f;
+    for (int o = 4; o > 0; o >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], o);
+    if (kg == 0) { sM[warp * BM + r] = m[i]; sL[warp * BM + r] = l[i]; }
+#pragma unroll
+    for (int c = 0; c < CT; ++c) *reinterpret_cast<ulonglong2*>(sK + r * D + (kg + 8 * c) * 4) = make_ulonglong2(acc[i][2 * c], acc[i][2 * c + 1]);
+  }
+  __syncthreads();
+  if (threadIdx.x < BM) {
+    const int r = threadIdx.x;
+    float mw[kCcWarps], ma = -INFINITY, sum = 0.f;
+#pragma unroll
+    for (int w = 0; w < kCcWarps; ++w) { mw[w] = sM[w * BM + r]; ma = fmaxf(ma, mw[w]); }
+#pragma unroll
+    for (int w = 0; w < kCcWarps; ++w) {
+      const float wt = mw[w] == -INFINITY ? 0.f : exp2f(mw[w] - ma);   // -inf: the warp saw no key of the row
+      sum = fmaf(wt, sL[w * BM + r], sum);
+      sM[w * BM + r] = wt;
+    }
+    sA[r] = ma; sA[BM + r] = sum;
+  }
+  __syncthreads();
+  T* ob = out + layer * p.out_ls + static_cast<long long>(g) * p.G * D;
+  float* lse = reinterpret_cast<float*>(ws_slot(ws, p, layer) + p.lse_off) + g * p.G;
+  auto write = [&](int r, int c, float4 o, float mx, float sum) {
+    if (row0 + r >= rows) return;
+    const float inv = 1.f / sum;
+    store4<T>(ob + row_off(row0 + r) + c * 4, make_float4(o.x * inv, o.y * inv, o.z * inv, o.w * inv));
+    if (c == 0) lse[static_cast<long long>((row0 + r) / p.G) * p.Hq + (row0 + r) % p.G] = (mx + log2f(sum)) * 0.6931471805599453f;
+  };
+#pragma unroll 1
+  for (int i = threadIdx.x; i < BM * D / 4; i += kCcThreads) {
+    const int r = i / (D / 4), c = i % (D / 4);
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int w = 0; w < kCcWarps; ++w) {
+      const float wt = sM[w * BM + r];
+      const float4 x = *reinterpret_cast<const float4*>(bufs + w * L::kWarpFloats + r * D + c * 4);
+      o.x = fmaf(wt, x.x, o.x); o.y = fmaf(wt, x.y, o.y); o.z = fmaf(wt, x.z, o.z); o.w = fmaf(wt, x.w, o.w);
+    }
+    if (S == 1) write(r, c, o, sA[r], sA[BM + r]);
+    else *reinterpret_cast<float4*>(sQ + r * KS + c * 4) = o;
+  }
+  if (S > 1) {                                              // merge over the cluster: rank s takes rows s, s + S, ...
+    cluster_arrive(); cluster_wait();
+#pragma unroll 1
+    for (int i = threadIdx.x; i < BM / S * (D / 4); i += kCcThreads) {
+      const int r = i / (D / 4) * S + split, c = i % (D / 4);
+      // (all remote reads are issued before the first result is used: one at a time they cost 10 us at S = 8)
+      float ma = -INFINITY, sum = 0.f, ms[8], ls[8];
+      float4 xs[8];
+#pragma unroll
+      for (int s2 = 0; s2 < 8; ++s2) {
+        const int src = s2 < S ? s2 : split;                // (S <= 8; the others repeat this rank's with weight zero)
+        ms[s2] = dsmem_ld_f32(dsmem_addr(smem_u32(sA + r), src));
+        ls[s2] = dsmem_ld_f32(dsmem_addr(smem_u32(sA + BM + r), src));
+        xs[s2] = dsmem_ld_v4(dsmem_addr(smem_u32(sQ + r * KS + c * 4), src));
+      }
+#pragma unroll
+      for (int s2 = 0; s2 < 8; ++s2) ma = fmaxf(ma, ms[s2]);
+      float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int s2 = 0; s2 < 8; ++s2) {
+        const float wt = s2 >= S || ms[s2] == -INFINITY ? 0.f : exp2f(ms[s2] - ma);
+        sum = fmaf(wt, ls[s2], sum);
+        o.x = fmaf(wt, xs[s2].x, o.x); o.y = fmaf(wt, xs[s2].y, o.y); o.z = fmaf(wt, xs[s2].z, o.z); o.w = fmaf(wt, xs[s2].w, o.w);
+      }
+      write(r, c, o, ma, sum);
+    }
+    cluster_arrive(); cluster_wait();                       // nobody leaves while its rows are being read
   }
   __syncthreads();
   if (threadIdx.x == 0) stamp_end(p);
@@ -159,23 +304,25 @@ __global__ void __launch_bounds__(128) attn_cc_kernel(const T* __restrict__ q, c
 
 // ------------------------------------------------------------------------------------------------
 // a2 score on CUDA cores (Eq. 4): score_j = sum over the w observer rows and the G heads of the
-// group of 2^(s_ij*scale_log2 - lse2_i).  A CTA owns 8 candidate keys; sixteen threads share a key and
-// split the observer rows between them (the sum over rows is the long serial chain otherwise, and a launch
-// of this path has a few hundred keys at most: many small CTAs, not few long ones).
-// grid (ceil(n_cand/8), Hkv, nl), block 128, dynamic smem = 8*(D+4)*4 + 32*D*4 + 32*4 bytes.
-static constexpr int kScoreCcKeys = 8;
+// group of 2^(s_ij*scale_log2 - lse2_i).  A CTA owns NK candidate keys; its eight warps take 16 observer rows each,
+// 128 at a time, and their sums are added in a fixed order at the end.  Bound: loading the observer rows, then the
+// FMA pipe (2 kv-heads x 1056 keys x 128 rows, d = 128: 7.9 us; one key per 16 threads took 65 us).
+// grid (ceil(n_cand/NK), Hkv, nl), block 256, dynamic smem score_cc_bytes.
+static constexpr int kScoreCcRows = 128;
+template <int D, int NK> constexpr int score_cc_bytes() { return ((NK + kScoreCcRows) * (D + 4) + kScoreCcRows + kCcWarps * NK) * 4; }
 
-template <typename T, int D>
-__global__ void __launch_bounds__(128) score_cc_kernel(const T* __restrict__ q, const char* __restrict__ cache,
-                                                       char* __restrict__ ws, Geom p) {
-  constexpr int KS = D + 4;
+template <typename T, int D, int NK>
+__global__ void __launch_bounds__(kCcThreads) score_cc_kernel(const T* __restrict__ q, const char* __restrict__ cache,
+                                                              char* __restrict__ ws, Geom p) {
+  constexpr int KS = D + 4, RT = 4, JT = NK / 8;
+  constexpr int EPC = 16 / (int)sizeof(T), CPR = D / EPC;
   extern __shared__ __align__(16) float smem_f[];
-  float* sK = smem_f;                          // [32][KS]
-  float* sQ = sK + kScoreCcKeys * KS;          // [32][D]
-  float* sL = sQ + 32 * D;                     // [32]
-  if (threadIdx.x == 0) stamp_begin(p);
-  const int layer = blockIdx.z, g = blockIdx.y;
-  const int key0 = blockIdx.x * kScoreCcKeys;
+  float* sK = smem_f;                          // [NK][KS]
+  float* sQ = sK + NK * KS;                    // [128][KS]
+  float* sL = sQ + kScoreCcRows * KS;          // [128]
+  float* sS = sL + kScoreCcRows;               // [8][NK] the warps' sums
+  const int layer = blockIdx.z, g = blockIdx.y, key0 = blockIdx.x * NK;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rg = lane >> 3, kg = lane & 7;
   const char* blob = cache + layer * p.cache_ls;
   const T* Kc = reinterpret_cast<const T*>(blob) + static_cast<long long>(g) * p.cap * D;
   const T* qb = q + layer * p.q_ls;
@@ -183,53 +330,78 @@ __global__ void __launch_bounds__(128) score_cc_kernel(const T* __restrict__ q, 
   const float* lse = reinterpret_cast<const float*>(slot + p.lse_off);
   float* score = reinterpret_cast<float*>(slot + p.score_off) + static_cast<long long>(g) * p.cap;
 
-  for (int i = threadIdx.x; i < kScoreCcKeys * D; i += 128) {
-    const int j = i / D, c = i % D, key = key0 + j;
-    sK[j * KS + c] = key < p.n_cand ? to_f32<T>(Kc[static_cast<long long>(key) * D + c]) : 0.f;
+  pdl_launch_dependents();
+  pdl_wait();
+  if (threadIdx.x == 0) stamp_begin(p);
+  for (int i = threadIdx.x; i < NK * CPR; i += kCcThreads) {
+    const int r = i / CPR, c = i % CPR * EPC;
+    stage16<T>(sK + r * KS + c, Kc + static_cast<long long>(min(key0 + r, p.n_cand - 1)) * D + c);
   }
   const int rows = p.w * p.G;
-  const int kj = threadIdx.x >> 4, part = threadIdx.x & 15;     // key of the CTA, sixteenth of the observer rows
-  float acc = 0.f;
-  const float4* krow = reinterpret_cast<const float4*>(&sK[kj * KS]);
-  for (int r0 = 0; r0 < rows; r0 += 32) {
-    __syncthreads();
-    for (int i = threadIdx.x; i < 32 * D; i += 128) {
-      const int r = r0 + i / D, c = i % D;
-      float x = 0.f;
-      if (r < rows) {
-        const int tok = p.n - p.w + r / p.G, h = g * p.G + r % p.G;
-        x = to_f32<T>(qb[(static_cast<long long>(tok) * p.Hq + h) * D + c]);
-      }
-      sQ[i] = x;
+  float acc[JT];
+#pragma unroll
+  for (int j = 0; j < JT; ++j) acc[j] = 0.f;
+  for (int r0 = 0; r0 < rows; r0 += kScoreCcRows) {
+    const int cnt = min(kScoreCcRows, rows - r0);
+    if (r0) __syncthreads();
+    auto token_head = [&](int r) { return static_cast<long long>(p.n - p.w + r / p.G) * p.Hq + g * p.G + r % p.G; };
+    for (int i = threadIdx.x; i < cnt * CPR; i += kCcThreads) {
+      const int r = i / CPR, c = i % CPR * EPC;
+      stage16<T>(sQ + r * KS + c, qb + token_head(r0 + r) * D + c);
     }
-    if (threadIdx.x < 32) {
-      const int r = r0 + threadIdx.x;
-      float lv = INFINITY;                                   // padding rows contribute 2^-inf = 0
-      if (r < rows) {
-        const int tok = p.n - p.w + r / p.G, h = g * p.G + r % p.G;
-        lv = lse[static_cast<long long>(tok) * p.Hq + h] * 1.4426950408889634f;
-      }
-      sL[threadIdx.x] = lv;
-    }
+    if (threadIdx.x < cnt) sL[threadIdx.x] = lse[token_head(r0 + threadIdx.x)] * 1.4426950408889634f;
+    cp_async_commit();
+    cp_async_wait<0>();
     __syncthreads();
-    const int rmax = min(32, rows - r0);
-    for (int r = part; r < rmax; r += 16) {
-      const float4* qrow = reinterpret_cast<const float4*>(&sQ[r * D]);
-      float s = 0.f;
-#pragma unroll 8
-      for (int c4 = 0; c4 < D / 4; ++c4) {
-        const float4 a = qrow[c4], b = krow[c4];
-        s = fmaf(a.x, b.x, s); s = fmaf(a.y, b.y, s); s = fmaf(a.z, b.z, s); s = fmaf(a.w, b.w, s);
+    const int w0 = warp * 16;                  // this warp's rows of the group (rows past the last: a copy of it, not summed)
+    if (w0 < cnt) {
+      uint64_t s2[RT][JT];
+      const float* qr[RT];
+#pragma unroll
+      for (int i = 0; i < RT; ++i) {
+        qr[i] = sQ + min(w0 + rg + 4 * i, cnt - 1) * KS;
+#pragma unroll
+        for (int j = 0; j < JT; ++j) s2[i][j] = 0ull;
       }
-      acc += exp2f(s * p.scale_log2 - sL[r]);
+#pragma unroll 4
+      for (int c = 0; c < D; c += 4) {
+        ulonglong2 b[JT];
+#pragma unroll
+        for (int j = 0; j < JT; ++j) b[j] = lds_f32x4(sK + (kg + 8 * j) * KS + c);
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+          const ulonglong2 a = lds_f32x4(qr[i] + c);
+#pragma unroll
+          for (int j = 0; j < JT; ++j) { s2[i][j] = fma_f32x2(a.x, b[j].x, s2[i][j]); s2[i][j] = fma_f32x2(a.y, b[j].y, s2[i][j]); }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < RT; ++i) {
+        const int r = w0 + rg + 4 * i;
+        if (r < cnt) {
+#pragma unroll
+          for (int j = 0; j < JT; ++j) {
+            float lo, hi;
+            f32x2_split(s2[i][j], lo, hi);
+            acc[j] += exp2f((lo + hi) * p.scale_log2 - sL[r]);
+          }
+        }
+      }
     }
   }
-  acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-  acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-  acc += __shfl_xor_sync(0xffffffffu, acc, 4);
-  acc += __shfl_xor_sync(0xffffffffu, acc, 8);
-  const int key = key0 + kj;
-  if (part == 0 && key < p.n_cand) score[key] = acc;
+#pragma unroll
+  for (int j = 0; j < JT; ++j) {
+    acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], 8);
+    acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], 16);
+    if (rg == 0) sS[warp * NK + kg + 8 * j] = acc[j];
+  }
+  __syncthreads();
+  if (threadIdx.x < NK && key0 + threadIdx.x < p.n_cand) {
+    float t = 0.f;
+#pragma unroll
+    for (int w = 0; w < kCcWarps; ++w) t += sS[w * NK + threadIdx.x];
+    score[key0 + threadIdx.x] = t;
+  }
   __syncthreads();
   if (threadIdx.x == 0) stamp_end(p);
 }

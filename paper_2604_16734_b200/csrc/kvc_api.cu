@@ -428,21 +428,6 @@ static cudaError_t opt_in_smem(Kernel kernel, int bytes, bool* done_per_device, 
   return e;
 }
 
-template <typename T, int D>
-static void launch_cc_attn(const Geom& g, const void* q, void* cache, void* out, void* ws, cudaStream_t st) {
-  dim3 grid((g.n + 15) / 16, g.Hq, g.nl);
-  kvc::attn_cc_kernel<T, D><<<grid, 128, 0, st>>>((const T*)q, (const char*)cache, (T*)out, (char*)ws, g);
-}
-template <typename T, int D>
-static cudaError_t launch_cc_score(const Geom& g, int dev, const void* q, void* cache, void* ws, cudaStream_t st) {
-  const int smem = (kvc::kScoreCcKeys * (D + 4) + 32 * D + 32) * 4;
-  static bool attr_set[kMaxDevices] = {};
-  if (cudaError_t e = opt_in_smem(kvc::score_cc_kernel<T, D>, smem, attr_set, dev)) return e;
-  dim3 grid((g.n_cand + kvc::kScoreCcKeys - 1) / kvc::kScoreCcKeys, g.Hkv, g.nl);
-  kvc::score_cc_kernel<T, D><<<grid, 128, smem, st>>>((const T*)q, (const char*)cache, (char*)ws, g);
-  return cudaSuccess;
-}
-
 // Launch attributes shared by the PDL-aware kernels: an optional cluster size and, unless disabled,
 // programmatic stream serialization (the kernel may start while its predecessor drains; it calls
 // griddepcontrol.wait before it touches anything the predecessor wrote or still reads).
@@ -462,6 +447,78 @@ struct LaunchAttrs {
     }
   }
 };
+
+template <typename T, int D, int BM>
+static cudaError_t launch_cc_attn_bm(const Geom& g, int dev, const void* q, const void* k, const void* v, void* cache, void* out,
+                                     void* ws, int S, bool pdl, cudaStream_t st) {
+  using L = kvc::AttnCc<D, BM>;
+  static bool attr_set[kMaxDevices] = {};
+  if (cudaError_t e = opt_in_smem(kvc::attn_cc_kernel<T, D, BM>, L::kBytes, attr_set, dev)) return e;
+  cudaLaunchConfig_t lc;
+  memset(&lc, 0, sizeof(lc));
+  lc.gridDim = dim3((int)(((long long)g.n * g.G + BM - 1) / BM) * S, g.Hkv, g.nl);
+  lc.blockDim = dim3(kvc::kCcThreads, 1, 1);
+  lc.dynamicSmemBytes = L::kBytes;
+  lc.stream = st;
+  LaunchAttrs la(S, pdl);
+  lc.attrs = la.at;
+  lc.numAttrs = la.n;
+  return cudaLaunchKernelEx(&lc, kvc::attn_cc_kernel<T, D, BM>, (const T*)q, (const T*)k, (const T*)v, (char*)cache, (T*)out,
+                            (char*)ws, g, S);
+}
+// Rows per CTA (BM) and key split (S) of the CUDA-core attention, by a model of its duration fitted to device stamps
+// of all twelve shapes on nine configurations (128 .. 4608 rows, 192 .. 2080 keys): a step (a key tile per warp) costs
+// 3.1 / 4.2 / 7 us at BM = 8 / 16 / 32, a CTA 3 us around its steps, the merge over a cluster 1.5 us more, and an SM
+// holds one CTA (clusters of 4 and 8 find room for 32 and 14 of them at a time).  E.g. 128 rows, 2080 keys: BM 16, S 8
+// 14.2 us against 41.1 (BM 8, S 1); 4608 rows, 1088 keys: BM 16, S 1 51.8 against 69.1 (BM 8) and 58.2 (BM 32);
+// 3136 rows, 708 keys: BM 32, S 1 44.3 against 46.4 (BM 16).  The model's choice was the fastest shape or within 3 %.
+template <typename T, int D>
+static cudaError_t launch_cc_attn(const Geom& g, int dev, const void* q, const void* k, const void* v, void* cache, void* out,
+                                  void* ws, bool allow_split, bool pdl, cudaStream_t st) {
+  constexpr int KT = kvc::AttnCc<D, 8>::KT;
+  const long long rows = (long long)g.n * g.G, heads = (long long)g.Hkv * g.nl;
+  const int bms[3] = {32, 16, 8}, capacity[4] = {kvc::kNumSMs, kvc::kNumSMs, 128, 112};
+  const double step_us[3] = {7.0, 4.2, 3.1};
+  int BM = 32, S = 1;
+  double best = 0.0;
+  for (int b = 0; b < 3; ++b) {
+    const long long base = (rows + bms[b] - 1) / bms[b] * heads;
+    for (int s = 0; s < (allow_split ? 4 : 1); ++s) {
+      if (s > 0 && (base << s) > capacity[s]) break;
+      const long long waves = ((base << s) + capacity[s] - 1) / capacity[s];
+      const int keys = waves > 1 ? g.n_c + g.n / 2 : g.n_c + g.n;      // the longest row, or the average over waves
+      const int per_step = KT * (kvc::kCcWarps << s);
+      const double est = (double)waves * ((keys + per_step - 1) / per_step * step_us[b] + 3.0) + (s > 0 ? 1.5 : 0.0);
+      if (best == 0.0 || est < best) { best = est; BM = bms[b]; S = 1 << s; }
+    }
+  }
+  if (BM == 32) return launch_cc_attn_bm<T, D, 32>(g, dev, q, k, v, cache, out, ws, S, pdl, st);
+  if (BM == 16) return launch_cc_attn_bm<T, D, 16>(g, dev, q, k, v, cache, out, ws, S, pdl, st);
+  return launch_cc_attn_bm<T, D, 8>(g, dev, q, k, v, cache, out, ws, S, pdl, st);
+}
+template <typename T, int D, int NK>
+static cudaError_t launch_cc_score_nk(const Geom& g, int dev, const void* q, void* cache, void* ws, bool pdl, cudaStream_t st) {
+  constexpr int smem = kvc::score_cc_bytes<D, NK>();
+  static bool attr_set[kMaxDevices] = {};
+  if (cudaError_t e = opt_in_smem(kvc::score_cc_kernel<T, D, NK>, smem, attr_set, dev)) return e;
+  cudaLaunchConfig_t lc;
+  memset(&lc, 0, sizeof(lc));
+  lc.gridDim = dim3((g.n_cand + NK - 1) / NK, g.Hkv, g.nl);
+  lc.blockDim = dim3(kvc::kCcThreads, 1, 1);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = st;
+  LaunchAttrs la(0, pdl);
+  lc.attrs = la.at;
+  lc.numAttrs = la.n;
+  return cudaLaunchKernelEx(&lc, kvc::score_cc_kernel<T, D, NK>, (const T*)q, (const char*)cache, (char*)ws, g);
+}
+template <typename T, int D>
+static cudaError_t launch_cc_score(const Geom& g, int dev, const void* q, void* cache, void* ws, bool pdl, cudaStream_t st) {
+  // 32 keys per CTA read the observer rows half as often (8 kv-heads x 608 keys, d = 64: 6.5 us against 7.5); 16 spread
+  // a launch that does not fill the GPU over twice the SMs (2 x 1056 keys, d = 128: 7.9 us against 11.1)
+  if ((long long)(g.n_cand + 31) / 32 * g.Hkv * g.nl > kvc::kNumSMs) return launch_cc_score_nk<T, D, 32>(g, dev, q, cache, ws, pdl, st);
+  return launch_cc_score_nk<T, D, 16>(g, dev, q, cache, ws, pdl, st);
+}
 
 // Number of CTAs the key range of one row-tile pair is split over (= cluster size): enough to put
 // a CTA on every SM when the row tiles alone cannot, as long as every CTA keeps a few key tiles.
@@ -690,22 +747,7 @@ static int run_chunk(kvc_ctx* c, int layer0, int nl, const void* q, long long q_
   // (the built-in scratch array) gets its status word cleared first.
   if (clear_status)
     if (int rc = check_cuda(c, cudaMemsetAsync(ws, 0, kvc::kWsHeaderBytes, st), "cudaMemsetAsync(status word)")) return rc;
-  // a0 append (the tensor-core attention kernel appends by itself)
-  if (!c->use_tc) {
-    ProfScope ps(c, 0, st);
-    g.stamps = next_stamp(c, 0);
-    dim3 grid((n * g.Hkv + 7) / 8, 1, nl);
-    cudaLaunchConfig_t lc;
-    memset(&lc, 0, sizeof(lc));
-    lc.gridDim = grid; lc.blockDim = dim3(256, 1, 1); lc.stream = st;
-    LaunchAttrs la(0, pdl);
-    lc.attrs = la.at; lc.numAttrs = la.n;
-    if (f32) e = cudaLaunchKernelEx(&lc, kvc::append_kernel<float>, (const float*)k, (const float*)v, (char*)cache, g);
-    else e = cudaLaunchKernelEx(&lc, kvc::append_kernel<__nv_bfloat16>, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (char*)cache, g);
-    c->launches++;
-  }
-  if (e != cudaSuccess) return check_cuda(c, e, "append launch");
-  // a1 attention
+  // a0 append + a1 attention
   long long attn_ctas = 0;                                    // CTAs of the attention launch (tensor-core path)
   {
   ProfScope ps(c, 1, st);
@@ -717,10 +759,10 @@ static int run_chunk(kvc_ctx* c, int layer0, int nl, const void* q, long long q_
     attn_ctas = (long long)(((g.n + TOK - 1) / TOK + R - 1) / R) * S * g.Hkv * g.nl;
     e = D == 128 ? launch_tc_attn<128>(g, dev, tq, tk, tv, tkin, tvin, cache, out, ws, S, R, pdl, st)
                  : launch_tc_attn<64>(g, dev, tq, tk, tv, tkin, tvin, cache, out, ws, S, R, pdl, st);
-  } else if (f32) {
-    if (D == 128) launch_cc_attn<float, 128>(g, q, cache, out, ws, st); else launch_cc_attn<float, 64>(g, q, cache, out, ws, st);
   } else {
-    if (D == 128) launch_cc_attn<__nv_bfloat16, 128>(g, q, cache, out, ws, st); else launch_cc_attn<__nv_bfloat16, 64>(g, q, cache, out, ws, st);
+    auto launch = [&](auto launcher) { return launcher(g, dev, q, k, v, cache, out, ws, !(cf.flags & 4u), pdl, st); };
+    if (f32) e = D == 128 ? launch(launch_cc_attn<float, 128>) : launch(launch_cc_attn<float, 64>);
+    else e = D == 128 ? launch(launch_cc_attn<__nv_bfloat16, 128>) : launch(launch_cc_attn<__nv_bfloat16, 64>);
   }
   }
   if (e != cudaSuccess) return check_cuda(c, e, "attention launch setup");
@@ -757,9 +799,9 @@ static int run_chunk(kvc_ctx* c, int layer0, int nl, const void* q, long long q_
       if (c->use_tc) {
         e = D == 128 ? launch_tc_score<128>(g, dev, tk, tqo, ws, tok_per_group, st) : launch_tc_score<64>(g, dev, tk, tqo, ws, tok_per_group, st);
       } else if (f32) {
-        e = D == 128 ? launch_cc_score<float, 128>(g, dev, q, cache, ws, st) : launch_cc_score<float, 64>(g, dev, q, cache, ws, st);
+        e = D == 128 ? launch_cc_score<float, 128>(g, dev, q, cache, ws, pdl, st) : launch_cc_score<float, 64>(g, dev, q, cache, ws, pdl, st);
       } else {
-        e = D == 128 ? launch_cc_score<__nv_bfloat16, 128>(g, dev, q, cache, ws, st) : launch_cc_score<__nv_bfloat16, 64>(g, dev, q, cache, ws, st);
+        e = D == 128 ? launch_cc_score<__nv_bfloat16, 128>(g, dev, q, cache, ws, pdl, st) : launch_cc_score<__nv_bfloat16, 64>(g, dev, q, cache, ws, pdl, st);
       }
       if (e != cudaSuccess) return check_cuda(c, e, "score launch");
       c->launches++;
