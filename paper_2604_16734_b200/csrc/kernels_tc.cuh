@@ -16,7 +16,9 @@ static constexpr int kSubTileBytes = 128 * 128;   // 128 rows x 64 bf16 (one 128
 // kv-head.  A tile holds TOK = 128 / G tokens (TOK * G <= 128 rows).
 
 
-static constexpr int kStages = 4;                 // K/V ring slots of the attention kernel
+// K/V ring slots of the attention kernel: with one row tile per CTA the shared memory of the second Q tile and what is
+// left beside it hold two more, so that each of the two key chains has a key tile in flight beyond the one it works on.
+template <int R> __host__ __device__ constexpr int attn_stages() { return R == 1 ? 6 : 4; }
 
 // ------------------------------------------------------------------------------------------------
 // a0 + a1: append (Alg. 1) and attention (Eq. 1).  Two 128-row tiles (A, B) per CTA, software pipelined,
@@ -46,46 +48,48 @@ static constexpr int kStages = 4;                 // K/V ring slots of the atten
 // has grown by more than 2^8, so P stays below 256 and O rarely needs touching.
 //
 // Key split: with cluster size S the CTA of cluster rank s handles key tiles [s*T/S, (s+1)*T/S) of
-// its row-tile pair and ends with a partial (O, m, l).  The partials are exchanged through
-// distributed shared memory: rank s owns rows [s*128/S, (s+1)*128/S) of both tiles.  With two row tiles
-// every CTA copies its partial rows (fp32) into the owner's shared memory with remote stores, the cluster
-// synchronises, and each rank combines and writes its rows.  With one row tile the rows (with m and l
-// behind them) leave in one bulk copy per owner, which completes on a barrier of the owner.  Nothing but
-// the final result goes to HBM.
+// its row tile (one per CTA then) and ends with a partial (O, m, l).  The partials are exchanged through distributed
+// shared memory: rank s owns rows [s*128/S, (s+1)*128/S), every CTA sends the rows of another owner, (m, l) behind
+// them, in one bulk copy, and each rank combines and writes its rows.  Nothing but the final result goes to HBM.
 // Row tiles per CTA: R = 2 as described, or R = 1.  A CTA with one row tile runs it twice over: softmax group and
 // issuer t take its key tiles t, t+2, ... with S, P, O, maximum and row sum of their own (tile B's TMEM columns), and
-// the two partial results are merged at the end.  That costs about 1.1 times as much per row tile and key tile, but
-// exchanges half as much in the combine and doubles the CTA count, which lets a launch that would need S = 4 do
-// with S = 2; the host picks.
+// the two partial results are merged at the end, column half by column half straight from TMEM.  That doubles the CTA
+// count at about 1.06 times the cost per row tile and key tile.
+// What bounds a launch (device stamps, us): 1.3 until the first S (dependency wait, TMA, MMA), then 0.94 per key tile
+// with one row tile or 1.78 with two, 1.5 for the epilogue, 2.7 for the combine of a key split.  With the output through
+// shared memory, the merge from TMEM, the six-slot ring and cluster barriers that order no memory: tiled image (13 key
+// tiles, 128 CTAs) 16.4 -> 14.5, video (18 key tiles split over two, 112 CTAs) 17.5 -> 15.3; two row tiles (long video)
+// 73.3 -> 73.1.
 // grid (ceil(ceil(n/TOK)/R) * S, Hkv, nl), cluster (S,1,1), block 384,
-// dynamic smem (2 + kStages) * (D/64) * 16 KB + 1 KB.
+// dynamic smem (R + attn_stages<R>()) * (D/64) * 16 KB + 1 KB.
 static constexpr int kAttnThreads = 384;
 
 struct TcSmemAttn {
-  uint64_t q_full[2], kv_full[kStages], kv_empty[kStages], s_full[2], p_half[2][2], pv_done[2];
+  uint64_t q_full[2], kv_full[6], kv_empty[6], s_full[2], p_half[2][2], pv_done[2];
   uint64_t comb_full;        // key split: the other ranks' partial rows have landed in this CTA's shared memory
   uint32_t tmem_base;
   int wait_ctl[2];           // [0] abort flag, [1] wait limit in units of 1024 cycles (see mbar_wait)
-  alignas(16) float stat[2 * 128 * 2];   // (read and written as float2) key split: (m, l) of the rows this rank owns, [S sources][2 tiles][rows_per][2], S * rows_per = 128
 };
 
-template <int D>
+template <int D, int R>
 __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
                                                                    const __grid_constant__ CUtensorMap tm_k,
                                                                    const __grid_constant__ CUtensorMap tm_v,
                                                                    const __grid_constant__ CUtensorMap tm_kin,
                                                                    const __grid_constant__ CUtensorMap tm_vin,
+                                                                   const __grid_constant__ CUtensorMap tm_out,
                                                                    char* __restrict__ cache,
                                                                    __nv_bfloat16* __restrict__ out,
-                                                                   char* __restrict__ ws, Geom p, int S, int R) {
+                                                                   char* __restrict__ ws, Geom p, int S) {
+  constexpr int kStages = attn_stages<R>();
   constexpr int NSUB = D / 64;
   constexpr int TILE_BYTES = NSUB * kSubTileBytes;
   constexpr uint32_t TMEM_COLS = 512;
   constexpr float kRescaleThreshold = 8.f;      // log2 units
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* sQ = smem;                            // two tiles
-  uint8_t* ring = smem + 2 * TILE_BYTES;         // kStages tiles; after the key loop: the parked O tiles
+  uint8_t* sQ = smem;                            // R tiles; after the key loop: the output tiles
+  uint8_t* ring = smem + R * TILE_BYTES;         // kStages tiles; after the key loop: the partials of a key split
   __shared__ TcSmemAttn sh;
 
   const int layer = blockIdx.z, g = blockIdx.y;
@@ -102,11 +106,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
   const int T = Tc + (last_tok + 128) / 128;
   const int t_begin = split * T / S, t_end = (split + 1) * T / S;
   const int Tl = t_end - t_begin;                // key tiles of this CTA (0 is possible when S > T)
-  // A CTA with one row tile and at least two key tiles runs the tile twice over: softmax group and issuer t take the
-  // key tiles t, t+2, ... with accumulators, maxima and sums of their own (the TMEM columns of tile B are free), two
-  // key tiles are in flight as with two row tiles, and the two partial results are merged at the end.
-  const bool alt = !has_B && Tl >= 2;
-  const int n_it[2] = {alt ? (Tl + 1) / 2 : Tl, alt ? Tl / 2 : (has_B ? Tl : 0)};   // key tiles of group 0 / 1
+  // A CTA with one row tile runs it twice over: softmax group and issuer t take the key tiles t, t+2, ... with
+  // accumulators, maxima and sums of their own (the TMEM columns of tile B are free), two key tiles are in flight as
+  // with two row tiles, and the two partial results are merged at the end.  (With Tl = 1 group 1 has none; Tl = 0
+  // happens with a key split, for the first rows of a block that see less of it than the last ones.)
+  const bool alt = !has_B;
+  const int n_it0 = alt ? (Tl + 1) / 2 : Tl, n_it1 = alt ? Tl / 2 : Tl;   // key tiles of group 0 / 1
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) {
@@ -117,14 +122,14 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
     for (int i = 0; i < kStages; ++i) { mbar_init(&sh.kv_full[i], 1); mbar_init(&sh.kv_empty[i], has_B ? 2 : 1); }
     sh.wait_ctl[0] = 0; sh.wait_ctl[1] = p.wait_limit_k;
     mbar_init(&sh.comb_full, 1);
-    // key split with one row tile: every other rank of the cluster will copy its partial of this rank's rows here
-    if (S > 1 && !has_B) mbar_expect_tx(&sh.comb_full, (S - 1) * (128 / S) * (D + 4) * 4);
+    // key split: every other rank of the cluster will copy its partial of this rank's rows here
+    if (S > 1) mbar_expect_tx(&sh.comb_full, (S - 1) * (128 / S) * (D + 4) * 4);
     mbar_fence_init();
   }
   // rows of the Q tiles that TMA never writes (rows >= TOK*G) must still be finite
   {
     const int pad16 = (128 - rows) * 8;          // 16-byte units per sub-tile
-    for (int i = threadIdx.x; i < 2 * NSUB * pad16; i += blockDim.x) {
+    for (int i = threadIdx.x; i < R * NSUB * pad16; i += blockDim.x) {
       const int sub = i / pad16, rem = i % pad16;
       reinterpret_cast<uint4*>(sQ + sub * kSubTileBytes + rows * 128)[rem] = make_uint4(0, 0, 0, 0);
     }
@@ -146,7 +151,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
       // ---------------------------------------------------------------- TMA producer
       if (lane == 0) {
         tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v);
-        tma_prefetch_desc(&tm_kin); tma_prefetch_desc(&tm_vin);
+        tma_prefetch_desc(&tm_kin); tma_prefetch_desc(&tm_vin); tma_prefetch_desc(&tm_out);
       }
       // While the previous kernel drains: ask L2 for the Q tiles and the first two key / value tiles (a hint only,
       // nothing is read into the SM before the wait below), so that the first loads find them there.
@@ -191,7 +196,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
           }
         }
       }
-    } else if (warp == 9 || (warp == 10 && (has_B || alt))) {
+    } else if (warp == 9 || warp == 10) {
       // ---------------------------------------------------------------- MMA issuer of tile t
       // a0 append (Alg. 1: C <- C u (K_i, V_i)).  The block's keys and values pass through the ring as key tiles
       // anyway: the issuer of tile A stores such a tile from its ring slot into cache rows n_c + 128u .. with one
@@ -209,7 +214,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
           for (int i = u * 128 + lane; i < min(p.n, u * 128 + 128); i += 32) pos[i] = static_cast<int>(p.pos0 + i);
         }
       }
-      if (lane == 0 && Tl > 0) {
+      if (lane == 0 && (warp == 9 ? n_it0 : n_it1) > 0) {
         const int t = warp - 9;
         bool stored = false, store_waited = false;
         // item i of the ring (2j = K, 2j+1 = V of local key tile j) has landed in `slot`: store it if it is ours
@@ -270,11 +275,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
           // two row tiles nothing else sits between the two groups of MMAs: the next K tile (landed long ago) is
           // waited for here, and the commits that free the slots and publish O come after the next S has been issued
           // (they then complete with it, which nobody minds: O is read after the next S at the earliest).  In-kernel
-          // stamps put the commits and the wait at 380 of the chain's 4000 cycles.  With one row tile and two key
-          // chains every ring item feeds one chain only and the ring holds one key tile per chain: there the V slot
-          // goes back to the producer first, and the K tile is waited for when it is needed (measured: the deferred
-          // order starves the other chain and costs 13 %).
-          const bool defer = !alt;
+          // stamps put the commits and the wait at 380 of the chain's 4000 cycles.  A CTA with one row tile in a
+          // launch of two (ring of four slots) has two key chains, every ring item feeds one of them only, and the
+          // ring holds one key tile per chain: there the V slot goes back to the producer first, and the K tile is
+          // waited for when it is needed (measured: the deferred order starves the other chain and costs 13 %; with
+          // the six slots of a one-row-tile launch it gains 3 %).
+          const bool defer = !alt || R == 1;
           if (defer && jn < Tl) {
             ok = mbar_wait(&sh.kv_full[slotK], (ik / kStages) & 1, abort_flag);
             if (!ok) break;
@@ -312,14 +318,14 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
       }
     }
     __syncwarp();
-    // Key split with one row tile: softmax group 0 writes over the ring once both key chains are complete, which says
+    // One row tile: the epilogue writes over the ring and the Q tile once both key chains are complete, which says
     // nothing about the stores above; warps 9 and 10 tell it here that no store reads the ring any more.
-    if (S > 1 && !has_B && (warp == 9 || warp == 10)) named_barrier_arrive(6, 128 + 64);
-    if (lane == 0) tma_store_wait_all();        // ... and the appended rows are in the cache before the kernel ends
+    if (alt && (warp == 9 || warp == 10)) named_barrier_arrive(5, 256 + 64);
     if (S > 1) {                                             // the cluster barriers of the combine below
-      cluster_arrive(); cluster_wait();
-      cluster_arrive(); cluster_wait();
+      cluster_arrive_relaxed(); cluster_wait();
+      cluster_arrive_relaxed(); cluster_wait();
     }
+    if (lane == 0) tma_store_wait_all();        // the appended rows are in the cache before the kernel ends
   } else {
     reg_inc<216>();
     // ---------------------------------------------------------------- softmax + epilogue of tile t
@@ -331,15 +337,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
     const uint32_t lane_addr = static_cast<uint32_t>((warp & 3) * 32) << 16;
     const uint32_t tmem_S = tmem + t * 128 + lane_addr, tmem_O = tmem + 256 + t * 128 + lane_addr;
     float m_ref = -INFINITY, l = 0.f;                        // reference maximum (log2 units) and row sum
-    float wm0 = 1.f, wm1 = 0.f;                              // key split, one row tile: weights of the two key chains' O
     bool ok = true;
-    const bool writer = t == 0 || has_B;                     // this group writes results (a row tile of its own)
-    const bool active = writer || alt;                       // this group takes part in the key loop
     const int first = alt ? t : 0, step = alt ? 2 : 1;       // local key tiles of this group: first, first + step, ...
     // Turn taking (named barrier 2 + t = "group t may go", 128 waiters + 128 arrivals).  Group 0 goes first.
-    const bool turns = (has_B || alt) && Tl > 0;
+    const bool turns = Tl > 0;
     if (turns && t == 1) named_barrier_arrive(2, 256);
-    if (active) {
+    {
       for (int jj = first, it = 0; jj < Tl; jj += step, ++it) {
         const int kt = t_begin + jj;                          // key tile index
         // Waits that gave up only skip the arithmetic: the turn barrier is passed on every path, once per key
@@ -428,351 +431,212 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
         } while (0);
         if (turns && !took_turn) named_barrier(2 + t, 256);   // a wait gave up before the turn was taken: take it now
         // hand the turn over if the other group has a key tile left: its it-th (group 0 asks) or (it+1)-th (group 1)
-        if (turns && (t == 0 ? it < n_it[1] : it + 1 < n_it[0])) named_barrier_arrive(3 - t, 256);
+        if (turns && (t == 0 ? it < n_it1 : it + 1 < n_it0)) named_barrier_arrive(3 - t, 256);
       }
       // The key loop is over: the next kernel of the stream may be scheduled and set itself up while this one
       // writes its results.  (Triggered at the start instead, the waiting CTAs of the next attention launch take the
       // SMs that the compress kernel of the previous layer, ready on a side stream, could use.)
       if (threadIdx.x == 0) pdl_launch_dependents();
-      if (ok && n_it[t] > 0) ok = mbar_wait(&sh.pv_done[t], (n_it[t] - 1) & 1, abort_flag);
+    }
+    // ---- epilogue.  Output rows leave through shared memory and TMA: a thread holds one row, and 32 threads storing 16
+    // bytes each of 32 different rows cost a sector per thread and instruction.
+    const long long head_row = static_cast<long long>(g) * p.G;       // output / lse row of (token, hh): token * Hq + head_row + hh
+    auto out_chunk = [&](int tile, int c16) -> uint4* {               // 16-byte piece c16 of row r in the swizzled output tile
+      return reinterpret_cast<uint4*>(sQ + tile * TILE_BYTES + (c16 >> 3) * kSubTileBytes + r * 128 + (((c16 & 7) ^ (r & 7)) << 4));
+    };
+    if (has_B) {
+      // Two row tiles: a group owns its rows.  Normalise, round, store the tile over its Q tile (read for the last time
+      // by the MMAs that pv_done covers) and let TMA write it out (tokens past n are clipped).
+      ok = ok && mbar_wait(&sh.pv_done[t], (Tl - 1) & 1, abort_flag);
       ok = __all_sync(0xffffffffu, ok);                       // the TMEM accesses below are warp-wide
-      if (ok && n_it[t] > 0) tc_fence_after_sync();
-      if (alt && S == 1) {
-        // Merge and write out, half the columns per group: group t keeps columns [t*D/2, (t+1)*D/2) of its O in
-        // registers and parks the other half (fp32, 16-byte chunks XOR-swizzled with row & 7 against bank conflicts)
-        // and its (m, l) in shared memory over the Q tiles, which nobody reads once both groups are past their
-        // last P V; then each group combines its columns of both partial results and writes them.
-        constexpr int H = D / 2;
-        float* mrg = reinterpret_cast<float*>(smem);          // [2 groups][128][H]
-        named_barrier(5, 256);
-        if (ok) {
+      if (ok) {
+        tc_fence_after_sync();
+        const float inv = 1.f / l;
 #pragma unroll
-          for (int c = 0; c < H / 32; ++c) {
-            uint32_t o[32];
-            tmem_ld32(tmem_O + (1 - t) * H + c * 32, o);
-            tmem_wait_ld();
+        for (int c = 0; c < D / 32; ++c) {
+          uint32_t o[32];
+          tmem_ld32(tmem_O + c * 32, o);
+          tmem_wait_ld();
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
-              *reinterpret_cast<uint4*>(mrg + (t * 128 + r) * H + (((c * 8 + k) ^ (r & 7)) << 2)) = make_uint4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
+          for (int i = 0; i < 4; ++i) {
+            uint4 vv;
+            vv.x = pack_bf16x2(__uint_as_float(o[8 * i + 0]) * inv, __uint_as_float(o[8 * i + 1]) * inv);
+            vv.y = pack_bf16x2(__uint_as_float(o[8 * i + 2]) * inv, __uint_as_float(o[8 * i + 3]) * inv);
+            vv.z = pack_bf16x2(__uint_as_float(o[8 * i + 4]) * inv, __uint_as_float(o[8 * i + 5]) * inv);
+            vv.w = pack_bf16x2(__uint_as_float(o[8 * i + 6]) * inv, __uint_as_float(o[8 * i + 7]) * inv);
+            *out_chunk(t, c * 4 + i) = vv;
           }
         }
-        sh.stat[(t * 128 + r) * 2] = (ok && l > 0.f) ? m_ref : -INFINITY;   // -inf: this group saw no key of the row
-        sh.stat[(t * 128 + r) * 2 + 1] = l;
-        named_barrier(5, 256);
+        if (row_valid) {
+          float* lse = reinterpret_cast<float*>(ws_slot(ws, p, layer) + p.lse_off);
+          lse[static_cast<long long>(tok) * p.Hq + head_row + hh] = (m_ref + log2f(l)) * 0.6931471805599453f;
+        }
+        fence_proxy_async_smem();
+      }
+      named_barrier(1 + 3 * t, 128);                           // (ids 1 and 4)
+      if (r == 0 && ok) {
+        for (int sub = 0; sub < NSUB; ++sub)
+          tma_store_4d(&tm_out, sQ + t * TILE_BYTES + sub * kSubTileBytes, sub * 64, g * p.G, tok0, layer);
+        tma_store_commit();
+        tma_store_wait_read();
+      }
+    } else {
+      // One row tile, two key chains.  Both accumulators sit in TMEM on the same lanes, so no thread has to hand rows
+      // over: group t takes half the columns of both, and only (m, l) are exchanged (through the TMEM columns of S).
+      constexpr int H = D / 2;
+      if (ok && n_it0 > 0) ok = mbar_wait(&sh.pv_done[0], (n_it0 - 1) & 1, abort_flag);
+      if (ok && n_it1 > 0) ok = mbar_wait(&sh.pv_done[1], (n_it1 - 1) & 1, abort_flag);
+      ok = __all_sync(0xffffffffu, ok);
+      if (ok) {
+        tc_fence_after_sync();
+        tmem_st2(tmem_S, __float_as_uint(l > 0.f ? m_ref : -INFINITY), __float_as_uint(l));   // -inf: no key of the row seen
+        tmem_wait_st();
+        tc_fence_before_sync();
+      }
+      named_barrier(5, 256 + 64);                              // both groups are here, and no store reads the ring
+      // This CTA's shared memory may be written by the cluster: everything that used it is complete and nothing was
+      // written there through the generic proxy, so the arrival need not order memory (a release costs 0.4 us here).
+      if (S > 1) cluster_arrive_relaxed();
+      float m_all = -INFINITY, L = 0.f, w0 = 0.f, w1 = 0.f;
+      if (ok) {
+        tc_fence_after_sync();
+        uint32_t mb, lb;
+        tmem_ld2(tmem + (1 - t) * 128 + lane_addr, mb, lb);
+        tmem_wait_ld();
+        const float m_own = l > 0.f ? m_ref : -INFINITY, m_oth = __uint_as_float(mb), l_oth = __uint_as_float(lb);
+        m_all = fmaxf(m_own, m_oth);
+        const float w_own = m_own == -INFINITY ? 0.f : fast_exp2(m_own - m_all);
+        const float w_oth = m_oth == -INFINITY ? 0.f : fast_exp2(m_oth - m_all);
+        L = fmaf(w_oth, l_oth, w_own * l);
+        w0 = t == 0 ? w_own : w_oth;
+        w1 = t == 0 ? w_oth : w_own;
+      }
+      const uint32_t tO0 = tmem + 256 + lane_addr + t * H, tO1 = tO0 + 128;    // this group's columns of both chains' O
+      const bool both = n_it1 > 0;                             // (one key tile: chain 1 has no O)
+      if (S == 1) {
         if (ok) {
-          const float m1 = sh.stat[((1 - t) * 128 + r) * 2], l1 = sh.stat[((1 - t) * 128 + r) * 2 + 1];
-          const float m0 = l > 0.f ? m_ref : -INFINITY;
-          const float m_all = fmaxf(m0, m1);                   // finite: group 0 has seen key tile 0, hence a key of every row
-          const float w0 = fast_exp2(m0 - m_all), w1 = fast_exp2(m1 - m_all);
-          const float L = fmaf(w1, l1, w0 * l);
           const float inv = 1.f / L, a0 = w0 * inv, a1 = w1 * inv;
-          __nv_bfloat16* orow = out + layer * p.out_ls + (static_cast<long long>(tok) * p.Hq + g * p.G + hh) * D + t * H;
 #pragma unroll
           for (int c = 0; c < H / 32; ++c) {
-            uint32_t o[32];
-            tmem_ld32(tmem_O + t * H + c * 32, o);
+            uint32_t o[32], q[32];
+            tmem_ld32(tO0 + c * 32, o);
+            if (both) tmem_ld32(tO1 + c * 32, q);
             tmem_wait_ld();
-            if (row_valid) {
+            float f[32];
 #pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                const float4 b0 = *reinterpret_cast<const float4*>(mrg + ((1 - t) * 128 + r) * H + (((c * 8 + 2 * i) ^ (r & 7)) << 2));
-                const float4 b1 = *reinterpret_cast<const float4*>(mrg + ((1 - t) * 128 + r) * H + (((c * 8 + 2 * i + 1) ^ (r & 7)) << 2));
-                uint4 vv;
-                vv.x = pack_bf16x2(fmaf(a1, b0.x, a0 * __uint_as_float(o[8 * i + 0])), fmaf(a1, b0.y, a0 * __uint_as_float(o[8 * i + 1])));
-                vv.y = pack_bf16x2(fmaf(a1, b0.z, a0 * __uint_as_float(o[8 * i + 2])), fmaf(a1, b0.w, a0 * __uint_as_float(o[8 * i + 3])));
-                vv.z = pack_bf16x2(fmaf(a1, b1.x, a0 * __uint_as_float(o[8 * i + 4])), fmaf(a1, b1.y, a0 * __uint_as_float(o[8 * i + 5])));
-                vv.w = pack_bf16x2(fmaf(a1, b1.z, a0 * __uint_as_float(o[8 * i + 6])), fmaf(a1, b1.w, a0 * __uint_as_float(o[8 * i + 7])));
-                reinterpret_cast<uint4*>(orow + c * 32)[i] = vv;
-              }
+            for (int i = 0; i < 32; ++i) f[i] = both ? fmaf(a1, __uint_as_float(q[i]), a0 * __uint_as_float(o[i])) : a0 * __uint_as_float(o[i]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              uint4 vv;
+              vv.x = pack_bf16x2(f[8 * i + 0], f[8 * i + 1]);
+              vv.y = pack_bf16x2(f[8 * i + 2], f[8 * i + 3]);
+              vv.z = pack_bf16x2(f[8 * i + 4], f[8 * i + 5]);
+              vv.w = pack_bf16x2(f[8 * i + 6], f[8 * i + 7]);
+              *out_chunk(0, t * (H / 8) + c * 4 + i) = vv;
             }
           }
           if (row_valid && t == 0) {
             float* lse = reinterpret_cast<float*>(ws_slot(ws, p, layer) + p.lse_off);
-            lse[static_cast<long long>(tok) * p.Hq + g * p.G + hh] = (m_all + log2f(L)) * 0.6931471805599453f;
+            lse[static_cast<long long>(tok) * p.Hq + head_row + hh] = (m_all + log2f(L)) * 0.6931471805599453f;
           }
+          fence_proxy_async_smem();
         }
-      } else if (alt) {
-        // Key split: merge the two groups' partial results into group 0's accumulator for the cluster combine below: group 1 parks its rows of O (fp32, 16-byte
-        // chunks XOR-swizzled with row & 7 against bank conflicts) and (m, l) in shared memory over the Q tiles, which
-        // nobody reads once both groups are past their last P V; group 0 rescales both to the common maximum.
-        float* mrg = reinterpret_cast<float*>(smem);          // [128][D]
-        named_barrier(5, 256);
-        if (t == 1) {
-          if (ok) {
-#pragma unroll
-            for (int c = 0; c < D / 32; ++c) {
-              uint32_t o[32];
-              tmem_ld32(tmem_O + c * 32, o);
-              tmem_wait_ld();
-#pragma unroll
-              for (int k = 0; k < 8; ++k)
-                *reinterpret_cast<uint4*>(mrg + r * D + (((c * 8 + k) ^ (r & 7)) << 2)) = make_uint4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
-            }
-          }
-          sh.stat[2 * r] = (ok && l > 0.f) ? m_ref : -INFINITY;   // -inf: this group saw no key of the row
-          sh.stat[2 * r + 1] = l;
+        named_barrier(1, 256);
+        if (threadIdx.x == 0 && ok) {
+          for (int sub = 0; sub < NSUB; ++sub)
+            tma_store_4d(&tm_out, sQ + sub * kSubTileBytes, sub * 64, g * p.G, tok0, layer);
+          tma_store_commit();
+          tma_store_wait_read();
         }
-        named_barrier(5, 256);
-        if (t == 0 && ok) {
-          // (a key split has one row tile here -- R = 1 -- or two; with one, the rows of chain 1 stay parked and are
-          // folded in when group 0 stages its rows for the cluster: only m and l are merged now)
-          const float m1 = sh.stat[2 * r], l1 = sh.stat[2 * r + 1];
-          if (m1 != -INFINITY) {
-            const float m_all = fmaxf(m_ref, m1);              // group 0 has seen key tile 0, hence a key of every row
-            wm0 = fast_exp2(m_ref - m_all);
-            wm1 = fast_exp2(m1 - m_all);
-            l = fmaf(wm1, l1, wm0 * l);
-            m_ref = m_all;
-          }
-        }
-      }
-      if (S == 1 && writer && !alt) {
-        if (ok) {
-          const float inv = 1.f / l;
-          __nv_bfloat16* orow = out + layer * p.out_ls + (static_cast<long long>(tok) * p.Hq + g * p.G + hh) * D;
+      } else {
+        // Combine the partials of the cluster (S is a power of two; rank s owns rows [s*rows_per, (s+1)*rows_per)).
+        // Each group writes its columns of the merged rows into a staging tile whose rows carry (m, l) behind the D
+        // values; the rows of every other owner then leave in ONE bulk copy each (shared memory to the owner's shared
+        // memory, completing on a barrier of the owner: this GPU's memory, no multicast), and each rank reduces its
+        // rows from the staging tile (its own partial) and from what the others sent:
+        //   O = sum_s 2^(m_s - m*) O_s / sum_s 2^(m_s - m*) l_s.
+        // Over the ring: the received rows [S - 1 sources][rows_per][D + 4] and the staging tile [128][D + 4] (a row
+        // stride of D + 4 floats keeps thread-per-row accesses off each other's banks).
+        constexpr int RS = D + 4;
+        const int rows_per = 128 / S;
+        float* recv = reinterpret_cast<float*>(ring);
+        float* stg = recv + (128 - rows_per) * RS;
 #pragma unroll
-          for (int c = 0; c < D / 32; ++c) {
-            uint32_t o[32];
-            tmem_ld32(tmem_O + c * 32, o);
-            tmem_wait_ld();
-            if (row_valid) {
+        for (int c = 0; c < H / 32; ++c) {
+          uint32_t o[32], q[32];
 #pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                uint4 vv;
-                vv.x = pack_bf16x2(__uint_as_float(o[8 * i + 0]) * inv, __uint_as_float(o[8 * i + 1]) * inv);
-                vv.y = pack_bf16x2(__uint_as_float(o[8 * i + 2]) * inv, __uint_as_float(o[8 * i + 3]) * inv);
-                vv.z = pack_bf16x2(__uint_as_float(o[8 * i + 4]) * inv, __uint_as_float(o[8 * i + 5]) * inv);
-                vv.w = pack_bf16x2(__uint_as_float(o[8 * i + 6]) * inv, __uint_as_float(o[8 * i + 7]) * inv);
-                reinterpret_cast<uint4*>(orow + c * 32)[i] = vv;
-              }
-            }
-          }
-          if (row_valid) {
-            float* lse = reinterpret_cast<float*>(ws_slot(ws, p, layer) + p.lse_off);
-            lse[static_cast<long long>(tok) * p.Hq + g * p.G + hh] = (m_ref + log2f(l)) * 0.6931471805599453f;
-          }
-        }
-      }
-    }
-    if (S > 1 && !has_B) {
-      // Combine the partials of the cluster, one row tile (S is a power of two; rank s owns rows [s*rows_per,
-      // (s+1)*rows_per)).  Group 0 writes its rows of O -- the two key chains folded together with the weights found
-      // above, chain 1 read from where group 1 parked it -- into a staging tile whose rows carry (m, l) behind the D
-      // values; the rows of every other owner then leave in ONE bulk copy each (shared memory to the owner's shared
-      // memory, completing on a barrier of the owner: this GPU's memory, no multicast), and each rank reduces its rows
-      // from the staging tile (its own partial) and from what the others sent:
-      //   O = sum_s 2^(m_s - m*) O_s / sum_s 2^(m_s - m*) l_s.
-      // Shared memory: the parked rows [128][D] over the Q tiles; over the ring the received rows [S - 1 sources]
-      // [rows_per][D + 4] and the staging tile [128][D + 4] (a row stride of D + 4 floats keeps thread-per-row
-      // accesses off each other's banks).
-      constexpr int RS = D + 4;
-      const int rows_per = 128 / S;
-      const float* mrg = reinterpret_cast<const float*>(smem);
-      float* recv = reinterpret_cast<float*>(smem + 2 * TILE_BYTES);
-      float* stg = recv + (128 - rows_per) * RS;
-      // This CTA's own ring is free: both key chains are complete, the producer loads no tile that is not used, and
-      // the issuer warps arrive on barrier 6 once the stores of the appended tiles have read their slots.
-      if (t == 0) {
-        named_barrier(6, 128 + 64);
-        const bool have = ok && Tl > 0;                         // warp-uniform
-#pragma unroll
-        for (int c = 0; c < D / 32; ++c) {
-          uint32_t o[32];
-          if (have) {
-            tmem_ld32(tmem_O + c * 32, o);
-            tmem_wait_ld();
-          } else {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) o[i] = 0u;
-          }
+          for (int i = 0; i < 32; ++i) { o[i] = 0u; q[i] = 0u; }   // (a chain without key tiles leaves its O columns unset)
+          if (ok && n_it0 > 0) tmem_ld32(tO0 + c * 32, o);
+          if (ok && both) tmem_ld32(tO1 + c * 32, q);
+          tmem_wait_ld();
 #pragma unroll
           for (int k = 0; k < 8; ++k) {
-            float4 v4 = make_float4(__uint_as_float(o[4 * k]), __uint_as_float(o[4 * k + 1]), __uint_as_float(o[4 * k + 2]), __uint_as_float(o[4 * k + 3]));
-            if (have && alt && wm1 != 0.f) {                  // (0: chain 1 saw no key of the row, or gave up)
-              const float4 b4 = *reinterpret_cast<const float4*>(mrg + r * D + (((c * 8 + k) ^ (r & 7)) << 2));
-              v4.x = fmaf(wm1, b4.x, wm0 * v4.x); v4.y = fmaf(wm1, b4.y, wm0 * v4.y);
-              v4.z = fmaf(wm1, b4.z, wm0 * v4.z); v4.w = fmaf(wm1, b4.w, wm0 * v4.w);
-            }
-            *reinterpret_cast<float4*>(stg + r * RS + (c * 8 + k) * 4) = v4;
+            float4 v4;
+            v4.x = fmaf(w1, __uint_as_float(q[4 * k + 0]), w0 * __uint_as_float(o[4 * k + 0]));
+            v4.y = fmaf(w1, __uint_as_float(q[4 * k + 1]), w0 * __uint_as_float(o[4 * k + 1]));
+            v4.z = fmaf(w1, __uint_as_float(q[4 * k + 2]), w0 * __uint_as_float(o[4 * k + 2]));
+            v4.w = fmaf(w1, __uint_as_float(q[4 * k + 3]), w0 * __uint_as_float(o[4 * k + 3]));
+            *reinterpret_cast<float4*>(stg + r * RS + t * H + (c * 8 + k) * 4) = v4;
           }
         }
-        *reinterpret_cast<float4*>(stg + r * RS + D) = make_float4((have && l > 0.f) ? m_ref : -INFINITY, have ? l : 0.f, 0.f, 0.f);
-        fence_proxy_async_smem();                               // the rows just written are read by bulk copies
-      }
-      // Every CTA of the cluster has staged its rows and is done with its ring, where the copies land.  (The barrier
-      // also orders this rank's staged rows before the reads of group 1 below.)
-      cluster_arrive();
-      cluster_wait();
-      if (threadIdx.x == 0) {
-        for (int owner = 0; owner < S; ++owner) {
-          if (owner == split) continue;
-          const int slot = split < owner ? split : split - 1;   // this rank among the owner's other ranks
-          bulk_copy_to_cluster(dsmem_addr(smem_u32(recv + slot * rows_per * RS), owner), smem_u32(stg + owner * rows_per * RS),
-                               rows_per * RS * 4, dsmem_addr(smem_u32(&sh.comb_full), owner));
+        if (t == 0) *reinterpret_cast<float2*>(stg + r * RS + D) = make_float2(m_all, L);
+        fence_proxy_async_smem();                              // the rows just written are read by bulk copies
+        named_barrier(1, 256);
+        cluster_wait();                                        // every CTA of the cluster is done with its ring
+        if (threadIdx.x == 0) {
+          for (int owner = 0; owner < S; ++owner) {
+            if (owner == split) continue;
+            const int slot = split < owner ? split : split - 1;   // this rank among the owner's other ranks
+            bulk_copy_to_cluster(dsmem_addr(smem_u32(recv + slot * rows_per * RS), owner), smem_u32(stg + owner * rows_per * RS),
+                                 rows_per * RS * 4, dsmem_addr(smem_u32(&sh.comb_full), owner));
+          }
         }
-      }
-      ok = mbar_wait(&sh.comb_full, 0, abort_flag) && ok;       // the other ranks' rows have landed
-      {
+        ok = mbar_wait(&sh.comb_full, 0, abort_flag) && ok;    // the other ranks' rows have landed
+        constexpr int CW = 16;                                 // columns per work item: (row, piece)
         const int r0 = split * rows_per;
-        const int per_tile = rows_per * (D / 32);               // work items: (row, group of 32 columns)
-        for (int item = threadIdx.x; item < per_tile; item += 256) {
-          const int lr = item % rows_per, cg = item / rows_per, r = r0 + lr;
-          const int tok = tokA + r / p.G, hh = r % p.G;
-          if (!(r < rows && tok < p.n)) continue;
-          auto row_of = [&](int s2) -> const float* {
-            return s2 == split ? stg + r * RS : recv + ((s2 < split ? s2 : s2 - 1) * rows_per + lr) * RS;
-          };
-          float m_all = -INFINITY;
 #pragma unroll 1
-          for (int s2 = 0; s2 < S; ++s2) m_all = fmaxf(m_all, row_of(s2)[D]);
-          float L = 0.f;
-          float acc[32];
+        for (int item = threadIdx.x; item < rows_per * (D / CW); item += 256) {
+          const int lr = item & (rows_per - 1), pc = item / rows_per, rr = r0 + lr;
+          const int tk = tokA + rr / p.G;
+          if (!(rr < rows && tk < p.n)) continue;
+          const float* own = stg + rr * RS;
+          const float* got = recv + lr * RS;                   // + source * rows_per * RS
+          float m_row = own[D];
+#pragma unroll 1
+          for (int s2 = 0; s2 < S - 1; ++s2) m_row = fmaxf(m_row, got[s2 * rows_per * RS + D]);
+          float L_row = 0.f, acc[CW];
 #pragma unroll
-          for (int i = 0; i < 32; ++i) acc[i] = 0.f;
+          for (int i = 0; i < CW; ++i) acc[i] = 0.f;
 #pragma unroll 1
-          for (int s2 = 0; s2 < S; ++s2) {
-            const float* row = row_of(s2);
+          for (int s2 = 0; s2 < S; ++s2) {                     // (source S - 1 of the loop: this rank itself)
+            const float* row = s2 < S - 1 ? got + s2 * rows_per * RS : own;
             const float2 ml = *reinterpret_cast<const float2*>(row + D);
-            if (ml.x == -INFINITY) continue;                  // this source saw no key of the row
-            const float wt = fast_exp2(ml.x - m_all);
-            L = fmaf(wt, ml.y, L);
+            const float wt = ml.x == -INFINITY ? 0.f : fast_exp2(ml.x - m_row);   // -inf: the source saw no key of the row
+            L_row = fmaf(wt, ml.y, L_row);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-              const float4 v4 = *reinterpret_cast<const float4*>(row + (cg * 8 + k) * 4);
-              acc[4 * k + 0] = fmaf(wt, v4.x, acc[4 * k + 0]);
-              acc[4 * k + 1] = fmaf(wt, v4.y, acc[4 * k + 1]);
-              acc[4 * k + 2] = fmaf(wt, v4.z, acc[4 * k + 2]);
-              acc[4 * k + 3] = fmaf(wt, v4.w, acc[4 * k + 3]);
+            for (int k = 0; k < CW / 4; ++k) {
+              const float4 v4 = *reinterpret_cast<const float4*>(row + pc * CW + k * 4);
+              acc[4 * k + 0] = fmaf(wt, v4.x, acc[4 * k + 0]); acc[4 * k + 1] = fmaf(wt, v4.y, acc[4 * k + 1]);
+              acc[4 * k + 2] = fmaf(wt, v4.z, acc[4 * k + 2]); acc[4 * k + 3] = fmaf(wt, v4.w, acc[4 * k + 3]);
             }
           }
-          const float inv = 1.f / L;
-          __nv_bfloat16* orow = out + layer * p.out_ls + (static_cast<long long>(tok) * p.Hq + g * p.G + hh) * D + cg * 32;
+          const float inv = 1.f / L_row;
+          const long long orow = static_cast<long long>(tk) * p.Hq + head_row + rr % p.G;
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
+          for (int k = 0; k < CW / 8; ++k) {
             uint4 vv;
-            vv.x = pack_bf16x2(acc[8 * i + 0] * inv, acc[8 * i + 1] * inv);
-            vv.y = pack_bf16x2(acc[8 * i + 2] * inv, acc[8 * i + 3] * inv);
-            vv.z = pack_bf16x2(acc[8 * i + 4] * inv, acc[8 * i + 5] * inv);
-            vv.w = pack_bf16x2(acc[8 * i + 6] * inv, acc[8 * i + 7] * inv);
-            reinterpret_cast<uint4*>(orow)[i] = vv;
+            vv.x = pack_bf16x2(acc[8 * k + 0] * inv, acc[8 * k + 1] * inv);
+            vv.y = pack_bf16x2(acc[8 * k + 2] * inv, acc[8 * k + 3] * inv);
+            vv.z = pack_bf16x2(acc[8 * k + 4] * inv, acc[8 * k + 5] * inv);
+            vv.w = pack_bf16x2(acc[8 * k + 6] * inv, acc[8 * k + 7] * inv);
+            reinterpret_cast<uint4*>(out + layer * p.out_ls + orow * D + pc * CW)[k] = vv;
           }
-          if (cg == 0) {
-            float* lse = reinterpret_cast<float*>(ws_slot(ws, p, layer) + p.lse_off);
-            lse[static_cast<long long>(tok) * p.Hq + g * p.G + hh] = (m_all + log2f(L)) * 0.6931471805599453f;
-          }
+          if (pc == 0) reinterpret_cast<float*>(ws_slot(ws, p, layer) + p.lse_off)[orow] = (m_row + log2f(L_row)) * 0.6931471805599453f;
         }
-      }
-      // A CTA must not exit while a bulk copy still reads its staging tile: every rank has waited for the copies
-      // addressed to it, so once all of them are here every copy is complete.
-      cluster_arrive();
-      cluster_wait();
-    } else if (S > 1) {
-      // Combine the partials of the cluster, two row tiles (S is a power of two).  Rank s owns rows [s*rows_per, (s+1)*rows_per)
-      // of both tiles.  Tile by tile, the softmax threads park their rows of O (fp32: the output tolerance
-      // leaves no room for a 16-bit exchange format) in a local staging tile, then copy it row by row into
-      // the owners' shared memory with remote stores -- stores are not waited for, remote loads would be --
-      // so that every warp instruction writes 512 contiguous bytes (one 16-byte store per thread straight
-      // from the TMEM layout, thread = row, scatters 32 rows per instruction and moved 13 B/clk).  The
-      // cluster synchronises, and each rank reduces its rows from its own shared memory:
-      //   O = sum_s 2^(m_s - m*) O_s / sum_s 2^(m_s - m*) l_s.
-      // recv: [S sources][2 tiles][rows_per][D] fp32 over the Q tiles and the first half of the ring; staging
-      // [128][D] behind it; the 16-byte chunks of a row are XOR-swizzled with (row & 7) so that neither the
-      // writers (lane = row) nor the readers (lane = row, same chunk) collide on banks.
-      const int rows_per = 128 / S;
-      float* stage = reinterpret_cast<float*>(smem);            // recv
-      float* stg = stage + 2 * 128 * D;
-      float* stat = sh.stat;                                    // [S][2][rows_per][2]: m (-inf: row saw no key), l
-      cluster_arrive();                                         // every CTA is done with its Q tiles and ring
-      cluster_wait();
-      {
-        constexpr int nthr = 256;                               // both groups take part
-        const bool have = ok && Tl > 0;                         // warp-uniform
-        for (int tt = 0; tt < 2; ++tt) {
-          if (t == tt) {
-            const int owner = r / rows_per, lr = r - owner * rows_per;
-#pragma unroll
-            for (int c = 0; c < D / 32; ++c) {
-              uint32_t o[32];
-              if (have) {
-                tmem_ld32(tmem_O + c * 32, o);
-                tmem_wait_ld();
-              } else {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) o[i] = 0u;
-              }
-#pragma unroll
-              for (int k = 0; k < 8; ++k)
-                *reinterpret_cast<uint4*>(stg + r * D + (((c * 8 + k) ^ (lr & 7)) << 2)) = make_uint4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
-            }
-            uint32_t stat_addr = smem_u32(stat + ((split * 2 + tt) * rows_per + lr) * 2);
-            if (owner != split) stat_addr = dsmem_addr(stat_addr, owner);
-            dsmem_st_v2(stat_addr, (have && l > 0.f) ? m_ref : -INFINITY, have ? l : 0.f);
-          }
-          named_barrier(1, nthr);                               // the staging tile is complete
-          constexpr int CPR = D / 4;                            // 16-byte chunks per row
-#pragma unroll 4
-          for (int idx = threadIdx.x; idx < 128 * CPR; idx += nthr) {
-            const int row = idx / CPR, chunk = idx % CPR;
-            const int owner = row / rows_per, lr = row - owner * rows_per;
-            const uint4 v4 = *reinterpret_cast<const uint4*>(stg + row * D + chunk * 4);
-            uint32_t dst = smem_u32(stage + ((split * 2 + tt) * rows_per + lr) * D + chunk * 4);
-            if (owner != split) dst = dsmem_addr(dst, owner);
-            dsmem_st_v4_b32(dst, v4.x, v4.y, v4.z, v4.w);
-          }
-          named_barrier(1, nthr);                               // the staging tile may be overwritten
-        }
-      }
-      cluster_arrive();                                         // all partials have landed; no remote access is
-      cluster_wait();                                           // started after this
-      {
-        const int r0 = min(128, split * rows_per), nrows = min(128, r0 + rows_per) - r0;
-        const int per_tile = nrows * (D / 32);                  // work items: (row, group of 32 columns)
-        for (int item = threadIdx.x; item < 2 * per_tile; item += 256) {
-          const int t = item / per_tile, rem = item % per_tile;
-          const int lr = rem % nrows, cg = rem / nrows, r = r0 + lr;
-          const int tok = (t ? tokB : tokA) + r / p.G, hh = r % p.G;
-          if (!(r < rows && tok < p.n)) continue;
-          // (the loops over the sources are kept rolled: this code runs once per CTA, straight-line copies of it
-          // cost more in instruction fetch than the loop does in branches)
-          float m_all = -INFINITY;
-#pragma unroll 1
-          for (int s = 0; s < S; ++s) m_all = fmaxf(m_all, stat[((s * 2 + t) * rows_per + lr) * 2]);
-          float L = 0.f;
-          float acc[32];
-#pragma unroll
-          for (int i = 0; i < 32; ++i) acc[i] = 0.f;
-#pragma unroll 1
-          for (int s = 0; s < S; ++s) {
-            const float2 ml = *reinterpret_cast<const float2*>(stat + ((s * 2 + t) * rows_per + lr) * 2);
-            if (ml.x == -INFINITY) continue;                  // this source saw no key of the row
-            const float wt = fast_exp2(ml.x - m_all);
-            L = fmaf(wt, ml.y, L);
-            const float* row = stage + ((s * 2 + t) * rows_per + lr) * D;
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-              const float4 v4 = *reinterpret_cast<const float4*>(row + (((cg * 8 + k) ^ (lr & 7)) << 2));
-              acc[4 * k + 0] = fmaf(wt, v4.x, acc[4 * k + 0]);
-              acc[4 * k + 1] = fmaf(wt, v4.y, acc[4 * k + 1]);
-              acc[4 * k + 2] = fmaf(wt, v4.z, acc[4 * k + 2]);
-              acc[4 * k + 3] = fmaf(wt, v4.w, acc[4 * k + 3]);
-            }
-          }
-          const float inv = 1.f / L;
-          __nv_bfloat16* orow = out + layer * p.out_ls + (static_cast<long long>(tok) * p.Hq + g * p.G + hh) * D + cg * 32;
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            uint4 vv;
-            vv.x = pack_bf16x2(acc[8 * i + 0] * inv, acc[8 * i + 1] * inv);
-            vv.y = pack_bf16x2(acc[8 * i + 2] * inv, acc[8 * i + 3] * inv);
-            vv.z = pack_bf16x2(acc[8 * i + 4] * inv, acc[8 * i + 5] * inv);
-            vv.w = pack_bf16x2(acc[8 * i + 6] * inv, acc[8 * i + 7] * inv);
-            reinterpret_cast<uint4*>(orow)[i] = vv;
-          }
-          if (cg == 0) {
-            float* lse = reinterpret_cast<float*>(ws_slot(ws, p, layer) + p.lse_off);
-            lse[static_cast<long long>(tok) * p.Hq + g * p.G + hh] = (m_all + log2f(L)) * 0.6931471805599453f;
-          }
-        }
+        // A CTA must not exit while a bulk copy still reads its staging tile: every rank has waited for the copies
+        // addressed to it, so once all of them are here every copy is complete.
+        cluster_arrive_relaxed();
+        cluster_wait();
       }
     }
   }

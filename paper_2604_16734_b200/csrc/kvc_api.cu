@@ -520,45 +520,41 @@ static cudaError_t launch_cc_score(const Geom& g, int dev, const void* q, void* 
   return launch_cc_score_nk<T, D, 16>(g, dev, q, cache, ws, pdl, st);
 }
 
-// Number of CTAs the key range of one row-tile pair is split over (= cluster size): enough to put
-// a CTA on every SM when the row tiles alone cannot, as long as every CTA keeps a few key tiles.
-// (An exchange of the partials through an L2-resident global buffer instead of distributed shared
-// memory was measured too: slower, the release / acquire round trip costs more than the narrow
-// SM-to-SM path.)
-// Launch shape of the tensor-core attention: R row tiles per CTA (1 or 2) and the key split S over a cluster.
-// For each R the split is the largest that the SM count, the portable cluster size and the rule of three key
-// tiles per CTA allow; the two candidates are then compared with a model of the kernel's duration fitted to
-// in-kernel time stamps (us): a key tile costs 1.8 per pair of row tiles taking turns and 1.15 for a single
-// tile (whose two softmax groups take alternate key tiles); the combine costs 3.5 for its barriers and the reduce plus 3.6 per row tile for the remote stores of a
-// whole tile's partial rows; CTAs beyond one per SM run as further waves.
+// Launch shape of the tensor-core attention: R row tiles per CTA (1 or 2) and, with one, the key split S over a cluster.
+// The shapes are compared with a model of the kernel's duration fitted to device stamps of all five shapes on sixteen
+// configurations (us): a key tile costs 1.78 per pair of row tiles taking turns and 0.94 for a single tile (whose two
+// softmax groups take alternate key tiles), a CTA 4.3 around them, the combine 2.7 (3.7 over eight CTAs); CTAs beyond
+// what is resident at a time (one per SM; 32 clusters of four, 14 of eight) run as further waves.  Measured, R=2 / R=1 S=1 /
+// S=2 / S=4 / S=8:  196 x 4 rows, 8 kv-heads, 2244 keys 35.3 / 20.6 / 15.7 / 25.2 / 46.2;  576 x 7, 4, 1600 keys 28.2 /
+// 17.0 / 27.3 / 45.9 / 92.9;  784 x 7, 4, 2832 keys 46.6 / 46.9 / 52.7;  1000 x 1, 32, 1500 keys 29.3 / 33.7 / 51.4;
+// 256 x 4, 2, 1280 keys 21.3 / 12.9 / 10.9 / 9.3 / 18.1;  100 x 3, 4, 4100 keys 61.4 / 33.2 / 21.5 / 14.9 / 12.6;
+// 128 x 1, 32, 320 keys 7.2 / 7.2 / 9.2 / 7.8 / 25.7.  On all sixteen the model picks the fastest or is within 1 %.
+// (An exchange of the partials through an L2-resident global buffer instead of distributed shared memory was measured
+// too: slower, the release / acquire round trip costs more than the narrow SM-to-SM path.)
 static void attn_launch_shape(const Geom& g, bool allow_split, int* S_out, int* R_out) {
   const int TOK = 128 / g.G;
   const int tiles = (g.n + TOK - 1) / TOK;
   const int T = (g.n_c + 127) / 128 + (g.n + 127) / 128;
-  double best = 0.0;
-  for (int R = 2; R >= 1; --R) {
-    const long long base = (long long)((tiles + R - 1) / R) * g.Hkv * g.nl;
-    int S = allow_split ? (int)(kvc::kNumSMs / base) : 1;
-    if (S > 8) S = 8;                    // portable cluster size limit
-    if (S > T / 3) S = T / 3;            // the exchange costs about as much as two key tiles: keep three per CTA
-    while (S & (S - 1)) S &= S - 1;      // a power of two: the 128 rows of a tile divide evenly among the ranks
-    if (S < 1) S = 1;
-    const int Tl = (T + S - 1) / S;
-    const long long waves = (base * S + kvc::kNumSMs - 1) / kvc::kNumSMs;
-    double est = Tl * (R == 2 ? 1.8 : 1.15) * (double)waves;
-    if (S > 1) est += 3.5 + R * 3.6 * (S - 1) / S;
-    if (R == 2 || est < best) { best = est; *S_out = S; *R_out = R; }
-    if (tiles == 1) break;               // a single row tile: both shapes are the same launch
+  const int capacity[4] = {kvc::kNumSMs, kvc::kNumSMs, 128, 112};
+  const double combine_us[4] = {0.0, 2.7, 2.7, 3.7};
+  const long long heads = (long long)g.Hkv * g.nl;
+  auto waves = [](long long ctas, int cap) { return (double)((ctas + cap - 1) / cap); };
+  // a single row tile never fills a pair
+  double best = tiles == 1 ? INFINITY : waves((tiles + 1) / 2 * heads, kvc::kNumSMs) * (T * 1.78 + 4.3);
+  *R_out = tiles == 1 ? 1 : 2; *S_out = 1;
+  for (int s = 0; s < (allow_split ? 4 : 1) && (1 << s) <= T; ++s) {
+    const double est = waves((tiles * heads) << s, capacity[s]) * ((T + (1 << s) - 1) / (1 << s) * 0.94 + 4.3) + combine_us[s];
+    if (est < best) { best = est; *R_out = 1; *S_out = 1 << s; }
   }
 }
 
-template <int D>
+template <int D, int R>
 static cudaError_t launch_tc_attn(const Geom& g, int dev, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
-                                  const CUtensorMap& tkin, const CUtensorMap& tvin, void* cache, void* out, void* ws, int S,
-                                  int R, bool pdl, cudaStream_t st) {
-  const int smem = (2 + kvc::kStages) * (D / 64) * kvc::kSubTileBytes + 1024;
+                                  const CUtensorMap& tkin, const CUtensorMap& tvin, const CUtensorMap& tout, void* cache,
+                                  void* out, void* ws, int S, bool pdl, cudaStream_t st) {
+  const int smem = (R + kvc::attn_stages<R>()) * (D / 64) * kvc::kSubTileBytes + 1024;
   static bool attr_set[kMaxDevices] = {};
-  if (cudaError_t e = opt_in_smem(kvc::attn_tc_kernel<D>, smem, attr_set, dev)) return e;
+  if (cudaError_t e = opt_in_smem(kvc::attn_tc_kernel<D, R>, smem, attr_set, dev)) return e;
   const int TOK = 128 / g.G;
   const int groups = ((g.n + TOK - 1) / TOK + R - 1) / R;
   cudaLaunchConfig_t lc;
@@ -570,8 +566,8 @@ static cudaError_t launch_tc_attn(const Geom& g, int dev, const CUtensorMap& tq,
   LaunchAttrs la(S, pdl);
   lc.attrs = la.at;
   lc.numAttrs = la.n;
-  return cudaLaunchKernelEx(&lc, kvc::attn_tc_kernel<D>, tq, tk, tv, tkin, tvin, (char*)cache, (__nv_bfloat16*)out,
-                            (char*)ws, g, S, R);
+  return cudaLaunchKernelEx(&lc, kvc::attn_tc_kernel<D, R>, tq, tk, tv, tkin, tvin, tout, (char*)cache, (__nv_bfloat16*)out,
+                            (char*)ws, g, S);
 }
 // a2..a4 fused (compress.cuh).  MODE: kvc::kScoresGiven / kScoreAttention / kScoreKeyDiff.
 template <int D, int MODE>
@@ -710,7 +706,7 @@ static int run_chunk(kvc_ctx* c, int layer0, int nl, const void* q, long long q_
   const int D = cf.head_dim;
 
   // tensor maps first: nothing is enqueued if an encode fails
-  CUtensorMap tq, tk, tv, tqo, tkin, tvin;
+  CUtensorMap tq, tk, tv, tqo, tkin, tvin, tout;
   int tok_per_group = 0;
   if (c->use_tc) {
     int rc = get_encoder(c);
@@ -720,6 +716,8 @@ static int run_chunk(kvc_ctx* c, int layer0, int nl, const void* q, long long q_
     const uint64_t qs[3] = {(uint64_t)D * 2, (uint64_t)g.Hq * D * 2, (uint64_t)q_ls * 2};
     const uint32_t qb[4] = {64, (uint32_t)g.G, (uint32_t)TOK, 1};
     if ((rc = make_map(c, &tq, q, qd, qs, qb))) return rc;
+    const uint64_t os[3] = {(uint64_t)D * 2, (uint64_t)g.Hq * D * 2, (uint64_t)out_ls * 2};
+    if ((rc = make_map(c, &tout, out, qd, os, qb))) return rc;
     const uint64_t kd[4] = {(uint64_t)D, (uint64_t)g.cap, (uint64_t)g.Hkv, (uint64_t)nl};
     const uint64_t ks[3] = {(uint64_t)D * 2, (uint64_t)g.cap * D * 2, (uint64_t)cache_ls};
     const uint32_t kb[4] = {64, 128, 1, 1};
@@ -757,8 +755,9 @@ static int run_chunk(kvc_ctx* c, int layer0, int nl, const void* q, long long q_
     attn_launch_shape(g, !(cf.flags & 4u), &S, &R);
     const int TOK = 128 / g.G;
     attn_ctas = (long long)(((g.n + TOK - 1) / TOK + R - 1) / R) * S * g.Hkv * g.nl;
-    e = D == 128 ? launch_tc_attn<128>(g, dev, tq, tk, tv, tkin, tvin, cache, out, ws, S, R, pdl, st)
-                 : launch_tc_attn<64>(g, dev, tq, tk, tv, tkin, tvin, cache, out, ws, S, R, pdl, st);
+    auto launch = [&](auto launcher) { return launcher(g, dev, tq, tk, tv, tkin, tvin, tout, cache, out, ws, S, pdl, st); };
+    if (D == 128) e = R == 2 ? launch(launch_tc_attn<128, 2>) : launch(launch_tc_attn<128, 1>);
+    else e = R == 2 ? launch(launch_tc_attn<64, 2>) : launch(launch_tc_attn<64, 1>);
   } else {
     auto launch = [&](auto launcher) { return launcher(g, dev, q, k, v, cache, out, ws, !(cf.flags & 4u), pdl, st); };
     if (f32) e = D == 128 ? launch(launch_cc_attn<float, 128>) : launch(launch_cc_attn<float, 64>);

@@ -1,0 +1,32 @@
+"""The launch shapes of the tensor-core attention and their edges: two row tiles per CTA with an odd last one, one row tile
+with one to many key tiles, key splits over clusters of 2, 4 and 8 CTAs (some without a key tile of the first rows), group
+sizes that leave rows of a tile unused."""
+import pytest
+import torch
+
+from oracle.kvc_oracle import KVCOracle
+from paper_2604_16734_b200.binding import Kvc
+from parity_util import compare_chunk
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("hq,hkv,d,B,chunks", [
+    (1, 1, 64, 40, (1, 40, 9)),                       # one row; one key tile, then two
+    (32, 32, 128, 140, (140, 129, 128)),              # two row tiles per kv-head, the second with 12 rows / one row
+    (28, 4, 128, 260, (260, 577)),                    # G = 7: 126 rows per tile; 577 tokens
+    (4, 1, 128, 1100, (1100, 40, 33)),                # clusters of 8
+    (8, 2, 64, 700, (700, 256, 255)),                 # clusters of 4
+    (32, 8, 128, 900, (900, 196, 197)),               # clusters of 2
+    (16, 16, 128, 130, (130, 1200)),                  # two row tiles per CTA, odd count: the last CTA has one
+    (12, 4, 64, 140, (140, 1100)),                    # G = 3, long block after a short cache
+])
+def test_launch_shapes(hq, hkv, d, B, chunks):
+    torch.manual_seed(B + hq)
+    kvc = Kvc(1, hq, hkv, d, torch.bfloat16, B, max(chunks))
+    orc = KVCOracle(1, hq, hkv, d, B, 32)
+    pos = 0
+    for n in chunks:
+        q, k, v = (torch.randn(n, h, d).to(torch.bfloat16) for h in (hq, hkv, hkv))
+        compare_chunk(kvc, orc, 0, q, k, v, pos)        # output within 2e-2 (or one bf16 ulp of the rounded oracle value)
+        pos += n
