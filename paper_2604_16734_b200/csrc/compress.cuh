@@ -34,7 +34,8 @@ static constexpr int kSelBins = 1 << kDigitBits;
 static constexpr int kRankMax = 256;          // keys of the cut-off bin that are ranked directly instead of by further rounds
 static constexpr int kMaxKeysSmem = 6144;     // candidates whose keys fit the shared-memory table (48 KB)
 static constexpr int kMaxMovesSmem = 2048;    // moves whose (src, dst) fit the shared-memory tables (16 KB)
-static constexpr int kMaxObsRowsFused = 128;  // observer rows (w * G) the fused scoring phase takes
+// observer rows (w * G) the fused scoring phase takes: up to 128, or up to 256 with a CTA alone on its SM
+static constexpr int kMaxObsRowsFused = 128, kMaxObsRowsWide = 256;
 static constexpr int kMaxClusterWide = 16;   // largest cluster the host asks for (non-portable size: more than 8 CTAs)
 static constexpr int kScoresGiven = 0, kScoreAttention = 1, kScoreKeyDiff = 2;   // what phase 1 of compress_kernel does
 static constexpr int kSubTileBytesC = 128 * 128;
@@ -60,16 +61,16 @@ struct CompressSmem {
 };
 
 // grid (Cn, Hkv, nl), cluster (Cn,1,1), block 512.
-// dynamic smem: the larger of the scoring buffers (two K tiles + up to 128 observer rows) and of the key
+// dynamic smem: the larger of the scoring buffers (two K tiles + OBS observer rows) and of the key
 // and move tables with the two histograms (80 KB), + 1 KB.
-template <int D, int MODE>
+template <int D, int MODE, int OBS>
 __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __grid_constant__ CUtensorMap tm_k,
                                                                        const __grid_constant__ CUtensorMap tm_qobs,
                                                                        char* __restrict__ cache, char* __restrict__ ws,
                                                                        Geom p, int Cn, int elem_bytes) {
   constexpr int NSUB = D / 64;
   constexpr int K_TILE_BYTES = NSUB * kSubTileBytesC;
-  constexpr int kQSubBytes = kMaxObsRowsFused * 128;   // up to 128 observer rows x 128 B
+  constexpr int kQSubBytes = OBS * 128;                // OBS observer rows x 128 B
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ CompressSmem sh;
@@ -94,7 +95,7 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
     uint8_t* sQ = smem + 2 * K_TILE_BYTES;           // observer rows
     const int n_tiles = (p.n_cand + 127) / 128;
     const int my_tiles = rank < n_tiles ? (n_tiles - rank + Cn - 1) / Cn : 0;
-    const int cols = p.w * p.G;                      // observer columns (<= 128: one MMA, two accumulators of 128 columns)
+    const int cols = p.w * p.G;                      // observer columns (<= OBS: one MMA, two accumulators of OBS columns)
     const int n_mma = (cols + 15) & ~15;
     if (tid == 0) {
       mbar_init(&sh.q_full, 1);
@@ -105,7 +106,7 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
     for (int i = tid; i < NSUB * kQSubBytes / 16; i += kCompressThreads) reinterpret_cast<uint4*>(sQ)[i] = make_uint4(0, 0, 0, 0);
     fence_proxy_async_smem();
     if (warp == 8) {
-      tmem_alloc(&sh.tmem_base, 256);
+      tmem_alloc(&sh.tmem_base, 2 * OBS);
       tmem_relinquish();
     }
     tc_fence_before_sync();
@@ -141,7 +142,7 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
           tc_fence_after_sync();
 #pragma unroll
           for (int kk = 0; kk < D / 16; ++kk)
-            mma_ss_lh(tmem + b * 128, k_lo0 + ((b * K_TILE_BYTES + (kk / 4) * kSubTileBytesC + (kk % 4) * 32) >> 4), hi,
+            mma_ss_lh(tmem + b * OBS, k_lo0 + ((b * K_TILE_BYTES + (kk / 4) * kSubTileBytesC + (kk % 4) * 32) >> 4), hi,
                       q_lo + (((kk / 4) * kQSubBytes + (kk % 4) * 32) >> 4), hi, idesc, kk > 0);
           mma_commit(&sh.s_full[b]);
           if (i + 2 < my_tiles) {                    // refill K buffer b once the MMAs that read it are done
@@ -178,8 +179,8 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
         for (int c0 = 0; c0 < n_mma; c0 += 32) {       // n_mma is a multiple of 16: the second half may be absent
           uint32_t sr[32];
           const bool two = c0 + 16 < n_mma;
-          tmem_ld16(tmem + b * 128 + lane_addr + c0, sr);
-          if (two) tmem_ld16(tmem + b * 128 + lane_addr + c0 + 16, sr + 16);
+          tmem_ld16(tmem + b * OBS + lane_addr + c0, sr);
+          if (two) tmem_ld16(tmem + b * OBS + lane_addr + c0 + 16, sr + 16);
           tmem_wait_ld();
 #pragma unroll
           for (int k = 0; k < 16; ++k) acc += fast_exp2(fmaf(__uint_as_float(sr[k]), p.scale_log2, -sh.lse2[c0 + k]));
@@ -200,7 +201,7 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
     __syncthreads();
     if (warp == 8) {
       tc_fence_after_sync();
-      tmem_dealloc(tmem, 256);
+      tmem_dealloc(tmem, 2 * OBS);
     }
   } else if constexpr (MODE == kScoreKeyDiff) {
     // Query-agnostic score (Sec. 3.2): anchor mu = mean of the tot keys the cache holds after the append,
@@ -507,7 +508,7 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
   const int total_holes = sh.s_remaining;
   if (rank == 0 && tid == 0) mcount[g] = total_holes;
   if (Cn > 1) {                                                  // the moves overwrite positions (and rows) that the
-    cluster_arrive();                                            // other CTAs of the cluster read while selecting
+    cluster_arrive_relaxed();                                    // other CTAs of the cluster read while selecting
     cluster_wait();
   }
 

@@ -10,6 +10,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 #include <vector>
 
@@ -570,15 +571,18 @@ static cudaError_t launch_tc_attn(const Geom& g, int dev, const CUtensorMap& tq,
                             (char*)ws, g, S);
 }
 // a2..a4 fused (compress.cuh).  MODE: kvc::kScoresGiven / kScoreAttention / kScoreKeyDiff.
-template <int D, int MODE>
+template <int D, int MODE, int OBS = kvc::kMaxObsRowsFused>
 static cudaError_t launch_compress(const Geom& g, int dev, const CUtensorMap& tk, const CUtensorMap& tqo, void* cache, void* ws,
                                    int elem_bytes, bool pdl, bool wide_ok, int cn_cap, cudaStream_t st) {
-  const int score_bytes = MODE == kvc::kScoreAttention ? 2 * (D / 64) * kvc::kSubTileBytesC + (D / 64) * kvc::kMaxObsRowsFused * 128 : 0;
+  const int score_bytes = MODE == kvc::kScoreAttention ? 2 * (D / 64) * kvc::kSubTileBytesC + (D / 64) * OBS * 128 : 0;
   const int table_bytes = kvc::kMaxKeysSmem * 8 + 2 * kvc::kMaxMovesSmem * 4 + 2 * kvc::kSelBins * 4;   // keys, move tables, histograms
   const int smem_min = (score_bytes > table_bytes ? score_bytes : table_bytes) + 1024;
-  const int smem_solo = 120 * 1024;                      // more than half an SM: one CTA per SM
+  // More than half an SM: one CTA per SM.  With more than 128 observer rows that is a must: the CTA takes all of the SM's
+  // TMEM, and CTAs of two clusters sharing SMs could each hold what the other's peer waits for.
+  const int smem_solo = smem_min > 120 * 1024 ? smem_min : 120 * 1024;
+  constexpr bool kAlone = OBS > kvc::kMaxObsRowsFused;
   static bool attr_set[kMaxDevices] = {};
-  if (cudaError_t e = opt_in_smem(kvc::compress_kernel<D, MODE>, smem_solo, attr_set, dev)) return e;
+  if (cudaError_t e = opt_in_smem(kvc::compress_kernel<D, MODE, OBS>, smem_solo, attr_set, dev)) return e;
   // Clusters of more than 8 CTAs are not portable: the kernel must allow them, and the device says how many clusters
   // of a size (one CTA per SM) it can hold at a time -- asked once per device and size; 0 where it refuses.
   static int wide_clusters[kMaxDevices][kvc::kMaxClusterWide + 1] = {};   // 0: not asked yet, -1: none, else clusters in flight
@@ -586,7 +590,7 @@ static cudaError_t launch_compress(const Geom& g, int dev, const CUtensorMap& tk
     int& slot = wide_clusters[dev][size];
     if (slot == 0) {
       int n_wide = 0;
-      if (cudaFuncSetAttribute(kvc::compress_kernel<D, MODE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+      if (cudaFuncSetAttribute(kvc::compress_kernel<D, MODE, OBS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
         cudaLaunchConfig_t q;
         memset(&q, 0, sizeof(q));
         q.gridDim = dim3(size, 1, 1);
@@ -595,7 +599,7 @@ static cudaError_t launch_compress(const Geom& g, int dev, const CUtensorMap& tk
         LaunchAttrs qa(size, false);
         q.attrs = qa.at;
         q.numAttrs = qa.n;
-        if (cudaOccupancyMaxActiveClusters(&n_wide, kvc::compress_kernel<D, MODE>, &q) != cudaSuccess) n_wide = 0;
+        if (cudaOccupancyMaxActiveClusters(&n_wide, kvc::compress_kernel<D, MODE, OBS>, &q) != cudaSuccess) n_wide = 0;
       }
       (void)cudaGetLastError();                           // a refusal is an answer, not an error of this call
       slot = n_wide > 0 ? n_wide : -1;
@@ -618,7 +622,7 @@ static cudaError_t launch_compress(const Geom& g, int dev, const CUtensorMap& tk
   // Two CTAs share an SM only when there are more CTAs than SMs (then one scores while the other selects);
   // a launch that fits the GPU asks for more than half an SM's shared memory so that every CTA gets an SM
   // of its own instead of being packed in pairs.
-  const int smem = (long long)Cn * g.Hkv * g.nl > kvc::kNumSMs ? smem_min : smem_solo;
+  const int smem = !kAlone && (long long)Cn * g.Hkv * g.nl > kvc::kNumSMs ? smem_min : smem_solo;
   cudaLaunchConfig_t lc;
   memset(&lc, 0, sizeof(lc));
   lc.gridDim = dim3(Cn, g.Hkv, g.nl);
@@ -628,7 +632,7 @@ static cudaError_t launch_compress(const Geom& g, int dev, const CUtensorMap& tk
   LaunchAttrs la(Cn, pdl);
   lc.attrs = la.at;
   lc.numAttrs = la.n;
-  return cudaLaunchKernelEx(&lc, kvc::compress_kernel<D, MODE>, tk, tqo, (char*)cache, (char*)ws, g, Cn, elem_bytes);
+  return cudaLaunchKernelEx(&lc, kvc::compress_kernel<D, MODE, OBS>, tk, tqo, (char*)cache, (char*)ws, g, Cn, elem_bytes);
 }
 
 template <int D>
@@ -789,10 +793,17 @@ static int run_chunk(kvc_ctx* c, int layer0, int nl, const void* q, long long q_
       if (cn_cap > per_gpc) cn_cap = per_gpc > 0 ? per_gpc : 1;
     }
     const bool keydiff = cf.policy == KVC_SCORE_KEYDIFF;      // query-agnostic: always scored inside the fused kernel
-    const bool fused_score = !keydiff && c->use_tc && g.w * g.G <= kvc::kMaxObsRowsFused;   // few observer rows: likewise
+    // Up to 128 observer rows are scored inside the fused kernel too, up to 256 with the CTA alone on its SM: that saves
+    // the score kernel's launch and start-up (4 kv-heads x 2300 keys x 224 rows, in stream order: 12.3 us against 5.0 + 8.0
+    // and 1.5 between them; 16 x 1250 x 256: 12.9 against 6.7 + 7.9).  Exception: two such launches in flight on the side
+    // streams that would not both fit the SMs the attention leaves idle (8 kv-heads, 20 idle SMs: 4 % of a step slower).
+    const bool wide_obs = g.w * g.G > kvc::kMaxObsRowsFused;
+    const long long side_ctas = 2ll * g.Hkv * g.nl * std::min(cn_cap, (int)((g.n_cand + 255) / 256));
+    const bool crowded = cn_cap > 0 && side_ctas > kvc::kNumSMs - attn_ctas;
+    const bool fused_score = !keydiff && c->use_tc && g.w * g.G <= (crowded ? kvc::kMaxObsRowsFused : kvc::kMaxObsRowsWide);
     if (!fused_score && !keydiff) {
-      // a2 score as a kernel of its own (fp32 on CUDA cores; bf16 with more than 128 observer rows per kv-head:
-      // fusing up to 256 rows was measured and is slower, the stand-alone kernel spreads the key tiles wider)
+      // a2 score as a kernel of its own (fp32 on CUDA cores; bf16 with more observer rows per kv-head than the fused
+      // kernel takes)
       ProfScope ps(c, 2, st);
       g.stamps = next_stamp(c, 2);
       if (c->use_tc) {
@@ -810,6 +821,9 @@ static int run_chunk(kvc_ctx* c, int layer0, int nl, const void* q, long long q_
       ProfScope ps(c, 3, st);
       g.stamps = next_stamp(c, 3);
       if (keydiff) e = launch_compress<64, kvc::kScoreKeyDiff>(g, dev, tk, tk, cache, ws, (int)c->elem, pdl, !async_compress, cn_cap, st);
+      else if (fused_score && wide_obs)
+        e = D == 128 ? launch_compress<128, kvc::kScoreAttention, kvc::kMaxObsRowsWide>(g, dev, tk, tqo, cache, ws, (int)c->elem, pdl, !async_compress, cn_cap, st)
+                     : launch_compress<64, kvc::kScoreAttention, kvc::kMaxObsRowsWide>(g, dev, tk, tqo, cache, ws, (int)c->elem, pdl, !async_compress, cn_cap, st);
       else if (fused_score) e = D == 128 ? launch_compress<128, kvc::kScoreAttention>(g, dev, tk, tqo, cache, ws, (int)c->elem, pdl, !async_compress, cn_cap, st)
                                          : launch_compress<64, kvc::kScoreAttention>(g, dev, tk, tqo, cache, ws, (int)c->elem, pdl, !async_compress, cn_cap, st);
       else e = launch_compress<64, kvc::kScoresGiven>(g, dev, tk, tk, cache, ws, (int)c->elem, pdl, !async_compress, cn_cap, st);

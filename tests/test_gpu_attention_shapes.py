@@ -5,7 +5,7 @@ import pytest
 import torch
 
 from oracle.kvc_oracle import KVCOracle
-from paper_2604_16734_b200.binding import Kvc
+from paper_2604_16734_b200.binding import KVC_FLAG_ASYNC_COMPRESS, Kvc
 from parity_util import compare_chunk
 
 pytestmark = pytest.mark.gpu
@@ -29,4 +29,22 @@ def test_launch_shapes(hq, hkv, d, B, chunks):
     for n in chunks:
         q, k, v = (torch.randn(n, h, d).to(torch.bfloat16) for h in (hq, hkv, hkv))
         compare_chunk(kvc, orc, 0, q, k, v, pos)        # output within 2e-2 (or one bf16 ulp of the rounded oracle value)
+        pos += n
+
+
+@pytest.mark.parametrize("hq,hkv,d,B,chunks,window,flags", [
+    (28, 4, 128, 300, (300, 130, 129), 32, 0),        # 224 observer rows, two to four key tiles
+    (32, 8, 64, 200, (200, 90, 33), 64, 0),           # 256 observer rows, the most that are scored in the fused kernel
+    (20, 4, 64, 260, (260, 60, 27), 26, 0),           # 130 observer rows, the fewest that take the wide form
+    (66, 2, 64, 200, (200, 64, 31), 8, 0),            # 264: a score kernel of its own
+    (64, 8, 128, 300, (300, 64, 64), 32, KVC_FLAG_ASYNC_COMPRESS),   # side stream without room for two launches
+])
+def test_observer_rows(hq, hkv, d, B, chunks, window, flags):
+    torch.manual_seed(B + hq)
+    kvc = Kvc(1, hq, hkv, d, torch.bfloat16, B, max(chunks), window, flags=flags)
+    orc = KVCOracle(1, hq, hkv, d, B, window)
+    pos = 0
+    for n in chunks:
+        q, k, v = (torch.randn(n, h, d).to(torch.bfloat16) for h in (hq, hkv, hkv))
+        compare_chunk(kvc, orc, 0, q, k, v, pos)
         pos += n
