@@ -118,6 +118,17 @@ __device__ __forceinline__ void tma_prefetch_l2_4d(const void* tmap, int c0, int
                : "memory");
 }
 
+// Untiled bulk load: contiguous bytes (both addresses and the size multiples of 16) into this CTA's shared memory.
+__device__ __forceinline__ void bulk_load(void* smem_dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(smem_u32(smem_dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ uint32_t dynamic_smem_bytes() {
+  uint32_t n;
+  asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(n));
+  return n;
+}
+
 // TMA store of one box from shared memory (bulk async-group completion).  Coordinates past the tensor's extent
 // are clipped.  The innermost coordinate must be a multiple of 16 bytes, the others are free.
 __device__ __forceinline__ void tma_store_4d(const void* tmap, const void* smem_src, int c0, int c1, int c2, int c3) {
