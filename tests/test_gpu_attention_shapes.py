@@ -48,3 +48,18 @@ def test_observer_rows(hq, hkv, d, B, chunks, window, flags):
         q, k, v = (torch.randn(n, h, d).to(torch.bfloat16) for h in (hq, hkv, hkv))
         compare_chunk(kvc, orc, 0, q, k, v, pos)
         pos += n
+
+
+def test_output_at_sixteen_byte_alignment():
+    # `out` needs 16-byte alignment only: at 16 modulo 32 the one-row-tile launch stores in smaller pieces, same values
+    n, hq, hkv, d = 70, 8, 2, 128
+    torch.manual_seed(1)
+    q, k, v = (torch.randn(n, h, d, device="cuda", dtype=torch.bfloat16) for h in (hq, hkv, hkv))
+    a, b = Kvc(1, hq, hkv, d, torch.bfloat16, 100, n), Kvc(1, hq, hkv, d, torch.bfloat16, 100, n)
+    whole = torch.zeros(n * hq * d + 24, device="cuda", dtype=torch.bfloat16)
+    shifted = whole[8:8 + n * hq * d].view(n, hq, d)
+    assert shifted.data_ptr() % 32 == 16
+    ref = a.prefill_chunk(0, q, k, v, 0)
+    b.prefill_chunk(0, q, k, v, 0, shifted)
+    assert a.status() == 0 and b.status() == 0
+    assert torch.equal(ref, shifted) and not whole[:8].any() and not whole[8 + n * hq * d:].any()
