@@ -60,7 +60,7 @@ template <int R> __host__ __device__ constexpr int attn_stages() { return R == 1
 // shared memory, the merge from TMEM, the six-slot ring and cluster barriers that order no memory: tiled image (13 key
 // tiles, 128 CTAs) 16.4 -> 14.5, video (18 key tiles split over two, 112 CTAs) 17.5 -> 15.3; two row tiles (long video)
 // 73.3 -> 73.1.
-// grid (ceil(ceil(n/TOK)/R) * S, Hkv, nl), cluster (S,1,1), block 384,
+// grid (R == 1 ? tiles * S : tiles - n_pairs, Hkv, nl) with tiles = ceil(n/TOK), cluster (S,1,1), block 384,
 // dynamic smem (R + attn_stages<R>()) * (D/64) * 16 KB + 1 KB.
 static constexpr int kAttnThreads = 384;
 
@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
                                                                    const __grid_constant__ CUtensorMap tm_out,
                                                                    char* __restrict__ cache,
                                                                    __nv_bfloat16* __restrict__ out,
-                                                                   char* __restrict__ ws, Geom p, int S) {
+                                                                   char* __restrict__ ws, Geom p, int S, int n_pairs) {
   constexpr int kStages = attn_stages<R>();
   constexpr int NSUB = D / 64;
   constexpr int TILE_BYTES = NSUB * kSubTileBytes;
@@ -94,12 +94,14 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
 
   const int layer = blockIdx.z, g = blockIdx.y;
   const int split = S > 1 ? static_cast<int>(cluster_ctarank()) : 0;
-  const int pair = blockIdx.x / S;               // index of this CTA's group of R row tiles (R = 1 or 2)
+  // R = 1: a row tile per CTA (or per cluster).  R = 2: the first n_pairs CTAs of a kv-head take two row tiles each, the
+  // others one of the rest.
   const int TOK = 128 / p.G, rows = TOK * p.G;
-  const int tokA = pair * R * TOK, tokB = tokA + TOK;
-  const bool has_B = R == 2 && tokB < p.n;
+  const bool has_B = R == 2 && static_cast<int>(blockIdx.x) < n_pairs;
+  const int tile0 = R == 1 ? blockIdx.x / S : has_B ? 2 * blockIdx.x : n_pairs + blockIdx.x;
+  const int tokA = tile0 * TOK, tokB = tokA + TOK, tok_end = has_B ? tokB + TOK : tokB;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int last_tok = min(tokA + R * TOK, p.n) - 1;
+  const int last_tok = min(tok_end, p.n) - 1;
   // Key tiles this pair of row tiles can see: Tc tiles of the cache (rows [0, n_c), the last one possibly
   // partial), then the block's own keys in tiles of 128 tokens, read straight from the k/v inputs.
   const int Tc = (p.n_c + 127) / 128;
@@ -146,7 +148,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
   volatile int* abort_flag = sh.wait_ctl;
 
   if (warp >= 8) {
-    reg_dec<72>();
+    reg_dec<56>();                               // (with 64 or 72 the compiler spills in the softmax groups of some forms: 2 - 8 % slower)
     if (warp == 8) {
       // ---------------------------------------------------------------- TMA producer
       if (lane == 0) {
@@ -175,11 +177,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
         mbar_expect_tx(&sh.q_full[0], NSUB * rows * 128);
         for (int sub = 0; sub < NSUB; ++sub)
           tma_load_4d(sQ + sub * kSubTileBytes, &tm_q, &sh.q_full[0], sub * 64, g * p.G, tokA, layer);
-        if (has_B) {
-          mbar_expect_tx(&sh.q_full[1], NSUB * rows * 128);
-          for (int sub = 0; sub < NSUB; ++sub)
-            tma_load_4d(sQ + TILE_BYTES + sub * kSubTileBytes, &tm_q, &sh.q_full[1], sub * 64, g * p.G, tokB, layer);
-        }
         for (int i = 0; i < 2 * Tl; ++i) {         // item 2j = K of tile t_begin + j, item 2j+1 = V of it
           const int slot = i % kStages, round = i / kStages;
           if (round > 0 && !mbar_wait(&sh.kv_empty[slot], (round - 1) & 1, abort_flag)) break;
@@ -194,6 +191,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
             for (int sub = 0; sub < NSUB; ++sub)
               tma_load_4d(ring + slot * TILE_BYTES + sub * kSubTileBytes, tm, &sh.kv_full[slot], sub * 64, g, (kt - Tc) * 128, layer);
           }
+          if (i == 0 && has_B) {                   // (row tile A can start on Q_A and the first K tile)
+            mbar_expect_tx(&sh.q_full[1], NSUB * rows * 128);
+            for (int sub = 0; sub < NSUB; ++sub)
+              tma_load_4d(sQ + TILE_BYTES + sub * kSubTileBytes, &tm_q, &sh.q_full[1], sub * 64, g * p.G, tokB, layer);
+          }
         }
       }
     } else if (warp == 9 || warp == 10) {
@@ -204,7 +206,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
       // clipped at cap).  Among the CTAs that load block tile u, the one whose rows contain token 128u owns it.
       // Nobody in this kernel reads the appended rows.  The lanes of the warp write the positions.
       const int u_lo = max(t_begin, Tc) - Tc, u_hi = t_end - Tc;            // block tiles of this CTA: [u_lo, u_hi)
-      auto owns = [&](int u) { return (u * 128) / (R * TOK) == pair; };
+      auto owns = [&](int u) { return u * 128 >= tokA && u * 128 < tok_end; };
       if (warp == 9 && u_hi > u_lo) {
         bool waited = false;
         for (int u = u_lo; u < u_hi; ++u) {

@@ -533,35 +533,48 @@ static cudaError_t launch_cc_score(const Geom& g, int dev, const void* q, void* 
 // 128 x 1, 32, 320 keys 7.2 / 7.2 / 9.2 / 7.8 / 25.7.  On all sixteen the model picks the fastest or is within 1 %.
 // (An exchange of the partials through an L2-resident global buffer instead of distributed shared memory was measured
 // too: slower, the release / acquire round trip costs more than the narrow SM-to-SM path.)
-static void attn_launch_shape(const Geom& g, bool allow_split, int* S_out, int* R_out) {
+struct AttnShape { int R, S, n_pairs; long long ctas; };
+static AttnShape attn_launch_shape(const Geom& g, bool allow_split, int reserve) {
   const int TOK = 128 / g.G;
   const int tiles = (g.n + TOK - 1) / TOK;
-  const int T = (g.n_c + 127) / 128 + (g.n + 127) / 128;
+  const int Tc = (g.n_c + 127) / 128, T = Tc + (g.n + 127) / 128;
   const int capacity[4] = {kvc::kNumSMs, kvc::kNumSMs, 128, 112};
   const double combine_us[4] = {0.0, 2.7, 2.7, 3.7};
   const long long heads = (long long)g.Hkv * g.nl;
   auto waves = [](long long ctas, int cap) { return (double)((ctas + cap - 1) / cap); };
-  // a single row tile never fills a pair
-  double best = tiles == 1 ? INFINITY : waves((tiles + 1) / 2 * heads, kvc::kNumSMs) * (T * 1.78 + 4.3);
-  *R_out = tiles == 1 ? 1 : 2; *S_out = 1;
-  for (int s = 0; s < (allow_split ? 4 : 1) && (1 << s) <= T; ++s) {
-    const double est = waves((tiles * heads) << s, capacity[s]) * ((T + (1 << s) - 1) / (1 << s) * 0.94 + 4.3) + combine_us[s];
-    if (est < best) { best = est; *R_out = 1; *S_out = 1 << s; }
+  AttnShape best = {2, 1, tiles / 2, (tiles - tiles / 2) * heads};
+  double best_us = tiles == 1 ? INFINITY : waves(best.ctas, kvc::kNumSMs) * (T * 1.78 + 4.3);   // a single row tile never fills a pair
+  // Pairs that would leave SMs idle: the row tiles with the most keys, the last ones, get a CTA each instead (1.2 us per
+  // key tile there: their ring has four slots).  784 x 7 rows, 4 kv-heads, 2832 keys: 46.5 -> 38.2 us; 640 x 4, 8, d = 64
+  // 31.5 -> 25.7; 1024 x 4, 8, 5120 keys 78.4 -> 76.6.  With compress on a side stream four SMs per kv-head stay free for
+  // it (`reserve`): per step 1190 -> 1054, 311 -> 275 and 1120 -> 1108 us; two or none are slower on most shapes.
+  const long long per_head = (kvc::kNumSMs - reserve) / heads;
+  if (per_head > tiles - tiles / 2 && per_head < tiles) {
+    const int n_pairs = (int)(tiles - per_head);
+    const int T_pair = Tc + (std::min(g.n, 2 * n_pairs * TOK) + 127) / 128;
+    const double est = std::max(T_pair * 1.78, T * 1.2) + 4.3;
+    if (est < best_us) { best_us = est; best = {2, 1, n_pairs, (tiles - n_pairs) * heads}; }
   }
+  for (int s = 0; s < (allow_split ? 4 : 1) && (1 << s) <= T; ++s) {
+    const long long ctas = (tiles * heads) << s;
+    const double est = waves(ctas, capacity[s]) * ((T + (1 << s) - 1) / (1 << s) * 0.94 + 4.3) + combine_us[s];
+    if (est < best_us) { best_us = est; best = {1, 1 << s, 0, ctas}; }
+  }
+  return best;
 }
 
 template <int D, int R>
 static cudaError_t launch_tc_attn(const Geom& g, int dev, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                                   const CUtensorMap& tkin, const CUtensorMap& tvin, const CUtensorMap& tout, void* cache,
-                                  void* out, void* ws, int S, bool pdl, cudaStream_t st) {
+                                  void* out, void* ws, int S, int n_pairs, bool pdl, cudaStream_t st) {
   const int smem = (R + kvc::attn_stages<R>()) * (D / 64) * kvc::kSubTileBytes + 1024;
   static bool attr_set[kMaxDevices] = {};
   if (cudaError_t e = opt_in_smem(kvc::attn_tc_kernel<D, R>, smem, attr_set, dev)) return e;
   const int TOK = 128 / g.G;
-  const int groups = ((g.n + TOK - 1) / TOK + R - 1) / R;
+  const int tiles = (g.n + TOK - 1) / TOK;
   cudaLaunchConfig_t lc;
   memset(&lc, 0, sizeof(lc));
-  lc.gridDim = dim3(groups * S, g.Hkv, g.nl);
+  lc.gridDim = dim3(R == 1 ? tiles * S : tiles - n_pairs, g.Hkv, g.nl);
   lc.blockDim = dim3(kvc::kAttnThreads, 1, 1);
   lc.dynamicSmemBytes = smem;
   lc.stream = st;
@@ -569,7 +582,7 @@ static cudaError_t launch_tc_attn(const Geom& g, int dev, const CUtensorMap& tq,
   lc.attrs = la.at;
   lc.numAttrs = la.n;
   return cudaLaunchKernelEx(&lc, kvc::attn_tc_kernel<D, R>, tq, tk, tv, tkin, tvin, tout, (char*)cache, (__nv_bfloat16*)out,
-                            (char*)ws, g, S);
+                            (char*)ws, g, S, n_pairs);
 }
 // a2..a4 fused (compress.cuh).  MODE: kvc::kScoresGiven / kScoreAttention / kScoreKeyDiff.
 template <int D, int MODE, int OBS = kvc::kMaxObsRowsFused>
@@ -756,13 +769,12 @@ static int run_chunk(kvc_ctx* c, int layer0, int nl, const void* q, long long q_
   ProfScope ps(c, 1, st);
   g.stamps = next_stamp(c, 1);
   if (c->use_tc) {
-    int S = 1, R = 2;
-    attn_launch_shape(g, !(cf.flags & 4u), &S, &R);
-    const int TOK = 128 / g.G;
-    attn_ctas = (long long)(((g.n + TOK - 1) / TOK + R - 1) / R) * S * g.Hkv * g.nl;
-    auto launch = [&](auto launcher) { return launcher(g, dev, tq, tk, tv, tkin, tvin, tout, cache, out, ws, S, pdl, st); };
-    if (D == 128) e = R == 2 ? launch(launch_tc_attn<128, 2>) : launch(launch_tc_attn<128, 1>);
-    else e = R == 2 ? launch(launch_tc_attn<64, 2>) : launch(launch_tc_attn<64, 1>);
+    // (a layer whose compress kernel runs beside the next attention wants SMs left for it)
+    const AttnShape sh = attn_launch_shape(g, !(cf.flags & 4u), async_compress && evict ? std::min(4 * g.Hkv * g.nl, kvc::kNumSMs) : 0);
+    attn_ctas = sh.ctas;
+    auto launch = [&](auto launcher) { return launcher(g, dev, tq, tk, tv, tkin, tvin, tout, cache, out, ws, sh.S, sh.n_pairs, pdl, st); };
+    if (D == 128) e = sh.R == 2 ? launch(launch_tc_attn<128, 2>) : launch(launch_tc_attn<128, 1>);
+    else e = sh.R == 2 ? launch(launch_tc_attn<64, 2>) : launch(launch_tc_attn<64, 1>);
   } else {
     auto launch = [&](auto launcher) { return launcher(g, dev, q, k, v, cache, out, ws, !(cf.flags & 4u), pdl, st); };
     if (f32) e = D == 128 ? launch(launch_cc_attn<float, 128>) : launch(launch_cc_attn<float, 64>);

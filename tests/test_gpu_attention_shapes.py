@@ -20,6 +20,8 @@ pytestmark = pytest.mark.gpu
     (32, 8, 128, 900, (900, 196, 197)),               # clusters of 2
     (16, 16, 128, 130, (130, 1200)),                  # two row tiles per CTA, odd count: the last CTA has one
     (12, 4, 64, 140, (140, 1100)),                    # G = 3, long block after a short cache
+    (28, 4, 128, 150, (150, 784, 703)),               # pairs first, then single row tiles (the last one ragged)
+    (32, 8, 64, 300, (300, 600, 641)),                # the same with d = 64; more single tiles than pairs
 ])
 def test_launch_shapes(hq, hkv, d, B, chunks):
     torch.manual_seed(B + hq)
@@ -38,6 +40,7 @@ def test_launch_shapes(hq, hkv, d, B, chunks):
     (20, 4, 64, 260, (260, 60, 27), 26, 0),           # 130 observer rows, the fewest that take the wide form
     (66, 2, 64, 200, (200, 64, 31), 8, 0),            # 264: a score kernel of its own
     (64, 8, 128, 300, (300, 64, 64), 32, KVC_FLAG_ASYNC_COMPRESS),   # side stream without room for two launches
+    (28, 4, 64, 150, (150, 784, 784), 32, KVC_FLAG_ASYNC_COMPRESS),  # pairs and single row tiles, SMs left for compress
 ])
 def test_observer_rows(hq, hkv, d, B, chunks, window, flags):
     torch.manual_seed(B + hq)
