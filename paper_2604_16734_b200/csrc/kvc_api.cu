@@ -933,10 +933,15 @@ extern "C" int kvc_prefill_chunk_host(kvc_ctx* c, int layer, const void* q_host,
   // caller's stream then waits for the outbound copy of the PREVIOUS call (the other half: its `out` area is the
   // next block's), which has had this call's kernels to finish.
   const int half = (int)(c->host_calls++ & 1u);
+  // The areas of a half start where those of the largest block do, whatever n is: the inbound copies of a call may run
+  // while `out` of the call two before it, in the same half, is still on its way out.
+  const size_t rows = c->cfg.max_chunk > c->cfg.budget ? c->cfg.max_chunk : c->cfg.budget;
+  const size_t q_area = align_up(rows * c->cfg.n_q_heads * c->cfg.head_dim * c->elem, 256);
+  const size_t k_area = align_up(rows * c->cfg.n_kv_heads * c->cfg.head_dim * c->elem, 256);
   char* dq = (char*)staging + half * (total / 2);
-  char* dk = dq + align_up(qb, 256);
-  char* dv = dk + align_up(kb, 256);
-  char* dout = dv + align_up(kb, 256);
+  char* dk = dq + q_area;
+  char* dv = dk + k_area;
+  char* dout = dv + k_area;
   if ((rc = check_cuda(c, cudaStreamWaitEvent(c->copy_in, c->ev_free[half], 0), "cudaStreamWaitEvent"))) return rc;
   if ((rc = check_cuda(c, cudaMemcpyAsync(dq, q_host, qb, cudaMemcpyHostToDevice, c->copy_in), "H2D q"))) return rc;
   if ((rc = check_cuda(c, cudaMemcpyAsync(dk, k_host, kb, cudaMemcpyHostToDevice, c->copy_in), "H2D k"))) return rc;

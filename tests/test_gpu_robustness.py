@@ -193,3 +193,32 @@ def test_device_time_stamps_count_every_launch(dtype):
     b.prefill_chunk(0, q, k, v, p)
     torch.cuda.synchronize()
     assert b.status() == 0
+
+
+# ------------------------------------------------------------------------------------------------
+# host buffers: blocks of different sizes back to back
+
+def test_host_blocks_of_different_sizes_do_not_overwrite_each_other():
+    # a small block's result must not share staging memory with the inputs of the larger block two calls later: its copy
+    # to the host may still be on its way when those arrive
+    hq, hkv, d, layers, blocks = 12, 4, 128, 6, (300, 4, 300, 30, 300)
+    torch.manual_seed(3)
+    a, b = (Kvc(layers, hq, hkv, d, torch.bfloat16, 64, max(blocks)) for _ in range(2))
+    calls, pos = [], 0
+    for n in blocks:
+        for layer in range(layers):
+            calls.append((layer, pos, [torch.randn(n, h, d).to(torch.bfloat16).pin_memory() for h in (hq, hkv, hkv)]))
+        pos += n
+    want = [a.prefill_chunk(layer, *(t.cuda() for t in qkv), p) for layer, p, qkv in calls]
+    outs = [torch.empty_like(qkv[0]).pin_memory() for _, _, qkv in calls]
+    for _ in range(20):
+        for o in outs:
+            o.zero_()
+        b.reset()
+        for (layer, p, qkv), o in zip(calls, outs):
+            b.prefill_chunk_host(layer, *qkv, p, o)
+        b.host_flush()
+        torch.cuda.synchronize()
+        assert b.status() == 0
+        for (layer, p, _), o, w in zip(calls, outs, want):
+            assert torch.equal(o, w.cpu()), f"layer {layer}, position {p}"
