@@ -210,18 +210,16 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
   } else if constexpr (MODE == kScoreKeyDiff) {
     // Query-agnostic score (Sec. 3.2): anchor mu = mean of the tot keys the cache holds after the append,
     // score_j = max(0, 1 - cos(k_j, mu)) for the candidates (>= 0, so its bit pattern orders like an integer; a
-    // zero key or anchor has cosine 0).  A CTA takes a contiguous share of the rows, a row is read by lpr lanes of 16
-    // bytes; the CTAs of the cluster add their partial sums through distributed shared memory, and every CTA scores its
-    // own rows (second read of K: L2).
+    // zero key or anchor has cosine 0).  A row is read by lpr lanes of 16 bytes; the CTAs of the cluster take the 128-row
+    // tiles round-robin, add their partial sums through distributed shared memory, and every CTA scores its own tiles
+    // (second read of K: L2).  The order of every sum is fixed by the cluster size alone.
     // Bound: latency and instruction fetch.  4 kv-heads x 1833 keys, d = 64: the kernel 13.6 -> 9.8 us (8 x 5120, d = 128
-    // 23.9 -> 19.2) with contiguous shares (every lane's loads in flight at once), the remote sums fetched together
+    // 23.9 -> 19.2) with loads in flight across tiles, the remote sums fetched together
     // (one at a time each costs a round trip), no array in local memory, one lane per row finishing its score, and the
     // shorter selection.  (Fetching the share into shared memory with bulk copies, or keeping it in registers: no faster.)
     float* s_part = reinterpret_cast<float*>(smem);                 // [16 warps][d] partial sums
     float* s_sum = s_part + (kCompressThreads / 32) * 128;         // [d] this CTA's sum (read by the cluster)
     float* s_mu = s_sum + 128;                                      // [d] the anchor
-    const int share = (p.tot + Cn - 1) / Cn;                        // rows per CTA
-    const int r_lo = min(rank * share, p.tot), r_hi = min(r_lo + share, p.tot);
     pdl_wait();
     if (tid == 0) stamp_begin(p);
     const int d = p.d, epl = 16 / elem_bytes;                       // elements per 16-byte piece: 8 (bf16) or 4 (fp32)
@@ -246,16 +244,20 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
     for (int e = 0; e < 8; ++e) acc[e] = 0.f;
     constexpr int kRowsInFlight = 4;                               // independent loads per lane
     const int rstep = (kCompressThreads / 32) * rpw;               // rows the CTA covers per step
-    const int first = r_lo + warp * rpw + sub;
+    const int tiles_all = (p.tot + 127) / 128, my_tiles = rank < tiles_all ? (tiles_all - rank + Cn - 1) / Cn : 0;
+    const int log_steps = __ffs(128 / rstep) - 1, n_steps = my_tiles << log_steps;   // steps per tile: 2, 4 or 8
+    auto row_of = [&](int i) { return (rank + (i >> log_steps) * Cn) * 128 + warp * rpw + sub + (i & ((1 << log_steps) - 1)) * rstep; };
     uint4 raw[kRowsInFlight];
-    auto load = [&](int row) {
+    auto load = [&](int i0) {
 #pragma unroll
-      for (int u = 0; u < kRowsInFlight; ++u)
-        raw[u] = row + u * rstep < r_hi ? fetch(row + u * rstep) : make_uint4(0u, 0u, 0u, 0u);
+      for (int u = 0; u < kRowsInFlight; ++u) {
+        const int row = row_of(i0 + u);
+        raw[u] = i0 + u < n_steps && row < p.tot ? fetch(row) : make_uint4(0u, 0u, 0u, 0u);
+      }
     };
 #pragma unroll 1
-    for (int row = first; row - sub < r_hi; row += rstep * kRowsInFlight) {
-      load(row);
+    for (int i0 = 0; i0 < n_steps; i0 += kRowsInFlight) {
+      load(i0);
 #pragma unroll
       for (int u = 0; u < kRowsInFlight; ++u) {
         float f[8];
@@ -297,12 +299,14 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
     __syncthreads();
     float mu[8], mu_norm = 0.f;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) { mu[e] = e < epl ? s_mu[piece * epl + e] : 0.f; mu_norm = fmaf(mu[e], mu[e], mu_norm); }
-    for (int o = 1; o < lpr; o <<= 1) mu_norm += __shfl_xor_sync(0xffffffffu, mu_norm, o);
+    for (int e = 0; e < 8; ++e) mu[e] = e < epl ? s_mu[piece * epl + e] : 0.f;
+    for (int i = lane; i < d; i += 32) mu_norm += s_mu[i] * s_mu[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mu_norm += __shfl_xor_sync(0xffffffffu, mu_norm, o);
     mu_norm = sqrtf(mu_norm);
 #pragma unroll 1
-    for (int row = first; row - sub < r_hi; row += rstep * kRowsInFlight) {   // (row - sub: the same in the whole warp)
-      load(row);
+    for (int i0 = 0; i0 < n_steps; i0 += kRowsInFlight) {
+      load(i0);
       float dot[kRowsInFlight], nrm[kRowsInFlight];
 #pragma unroll
       for (int u = 0; u < kRowsInFlight; ++u) {
@@ -324,11 +328,11 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
 #pragma unroll
       for (int u = 1; u < kRowsInFlight; ++u)
         if (piece == u) { dt = dot[u]; nm = nrm[u]; }
-      const int r = row + piece * rstep;
+      const int r = row_of(i0 + piece);
       // fp32 rounding can put the cosine of a key (nearly) parallel to the anchor a little above 1: clamp, so
       // that the score stays >= 0 and select_key's ordering by bit pattern holds
       const float den = sqrtf(nm) * mu_norm;
-      if (piece < kRowsInFlight && r < min(r_hi, p.n_cand)) score[r] = den > 0.f ? fmaxf(0.f, 1.f - dt / den) : 1.f;
+      if (piece < kRowsInFlight && i0 + piece < n_steps && r < p.n_cand) score[r] = den > 0.f ? fmaxf(0.f, 1.f - dt / den) : 1.f;
     }
     __syncthreads();
   } else {
