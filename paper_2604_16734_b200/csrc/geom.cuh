@@ -15,6 +15,8 @@ struct Geom {
   int G, Hq, Hkv, d, cap, nl, max_chunk;
   int n_cand;     // tot - w : entries that compete for the budget
   int n_keep;     // B - w   : how many of them survive
+  int n_sc;       // keys of rows [0, n_sc) are scored from the cache, those of later rows from the k input
+  int early;      // the attention kernel lets its dependent start at once instead of at the end of its key loop
   float scale_log2;           // softmax scale times log2(e): probabilities are 2^(s*scale_log2 - lse2)
   long long pos0;             // absolute position of the block's first token
   long long q_ls, kv_ls, out_ls;   // layer strides of q/out and k/v inputs, in elements

@@ -86,8 +86,9 @@ __global__ void __launch_bounds__(kCcThreads, 1) attn_cc_kernel(const T* __restr
   const T* qb = q + layer * p.q_ls + static_cast<long long>(g) * p.G * D;
   auto row_off = [&](int r) { return (static_cast<long long>(r / p.G) * p.Hq + r % p.G) * D; };   // row r of q / out
 
-  pdl_launch_dependents();
   pdl_wait();                                               // the previous block's compaction is done with the cache
+  // (after the wait: the score kernel reads the inputs and the old cache rows before its own)
+  pdl_launch_dependents();
   if (threadIdx.x == 0) stamp_begin(p);
 
   const int kv_end = p.n_c + (min(row0 + BM, rows) - 1) / p.G + 1;     // keys the last row of this CTA sees
@@ -306,13 +307,15 @@ __global__ void __launch_bounds__(kCcThreads, 1) attn_cc_kernel(const T* __restr
 // a2 score on CUDA cores (Eq. 4): score_j = sum over the w observer rows and the G heads of the
 // group of 2^(s_ij*scale_log2 - lse2_i).  A CTA owns NK candidate keys; its eight warps take 16 observer rows each,
 // 128 at a time, and their sums are added in a fixed order at the end.  Bound: loading the observer rows, then the
-// FMA pipe (2 kv-heads x 1056 keys x 128 rows, d = 128: 7.9 us; one key per 16 threads took 65 us).
+// FMA pipe (2 kv-heads x 1056 keys x 128 rows, d = 128: 7.9 us; one key per 16 threads took 65 us), of which all but the
+// exponentials overlaps the attention's end (1 x 160 keys, d = 64: 3.2 -> 1.1 us behind the dependency wait).
 // grid (ceil(n_cand/NK), Hkv, nl), block 256, dynamic smem score_cc_bytes.
 static constexpr int kScoreCcRows = 128;
 template <int D, int NK> constexpr int score_cc_bytes() { return ((NK + kScoreCcRows) * (D + 4) + kScoreCcRows + kCcWarps * NK) * 4; }
 
 template <typename T, int D, int NK>
-__global__ void __launch_bounds__(kCcThreads) score_cc_kernel(const T* __restrict__ q, const char* __restrict__ cache,
+__global__ void __launch_bounds__(kCcThreads) score_cc_kernel(const T* __restrict__ q, const T* __restrict__ k,
+                                                              const char* __restrict__ cache,
                                                               char* __restrict__ ws, Geom p) {
   constexpr int KS = D + 4, RT = 4, JT = NK / 8;
   constexpr int EPC = 16 / (int)sizeof(T), CPR = D / EPC;
@@ -330,12 +333,15 @@ __global__ void __launch_bounds__(kCcThreads) score_cc_kernel(const T* __restric
   const float* lse = reinterpret_cast<const float*>(slot + p.lse_off);
   float* score = reinterpret_cast<float*>(slot + p.score_off) + static_cast<long long>(g) * p.cap;
 
+  // Keys, observer rows and the first group's products come before the dependency wait: the inputs and the cache rows
+  // below n_c are complete (the attention kernel allows this launch after its own wait), the block's keys are read from
+  // the input.  Only the exponentials need what the attention kernel leaves.
   pdl_launch_dependents();
-  pdl_wait();
-  if (threadIdx.x == 0) stamp_begin(p);
+  const long long in_stride = static_cast<long long>(p.Hkv) * D;
+  const T* Kn = k + layer * p.kv_ls + static_cast<long long>(g) * D;
   for (int i = threadIdx.x; i < NK * CPR; i += kCcThreads) {
-    const int r = i / CPR, c = i % CPR * EPC;
-    stage16<T>(sK + r * KS + c, Kc + static_cast<long long>(min(key0 + r, p.n_cand - 1)) * D + c);
+    const int r = i / CPR, c = i % CPR * EPC, key = min(key0 + r, p.n_cand - 1);
+    stage16<T>(sK + r * KS + c, (key < p.n_sc ? Kc + static_cast<long long>(key) * D : Kn + (key - p.n_sc) * in_stride) + c);
   }
   const int rows = p.w * p.G;
   float acc[JT];
@@ -349,13 +355,12 @@ __global__ void __launch_bounds__(kCcThreads) score_cc_kernel(const T* __restric
       const int r = i / CPR, c = i % CPR * EPC;
       stage16<T>(sQ + r * KS + c, qb + token_head(r0 + r) * D + c);
     }
-    if (threadIdx.x < cnt) sL[threadIdx.x] = lse[token_head(r0 + threadIdx.x)] * 1.4426950408889634f;
     cp_async_commit();
     cp_async_wait<0>();
     __syncthreads();
     const int w0 = warp * 16;                  // this warp's rows of the group (rows past the last: a copy of it, not summed)
+    uint64_t s2[RT][JT];
     if (w0 < cnt) {
-      uint64_t s2[RT][JT];
       const float* qr[RT];
 #pragma unroll
       for (int i = 0; i < RT; ++i) {
@@ -375,6 +380,14 @@ __global__ void __launch_bounds__(kCcThreads) score_cc_kernel(const T* __restric
           for (int j = 0; j < JT; ++j) { s2[i][j] = fma_f32x2(a.x, b[j].x, s2[i][j]); s2[i][j] = fma_f32x2(a.y, b[j].y, s2[i][j]); }
         }
       }
+    }
+    if (r0 == 0) {
+      pdl_wait();
+      if (threadIdx.x == 0) stamp_begin(p);
+    }
+    if (threadIdx.x < cnt) sL[threadIdx.x] = lse[token_head(r0 + threadIdx.x)] * 1.4426950408889634f;
+    __syncthreads();
+    if (w0 < cnt) {
 #pragma unroll
       for (int i = 0; i < RT; ++i) {
         const int r = w0 + rg + 4 * i;

@@ -170,7 +170,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
       }
       __syncwarp();
       if (lane == 0) {
-        pdl_wait();                                // the block's keys were appended by the previous kernel
+        pdl_wait();                                // the previous block's compaction is done with the cache
+        if (p.early) pdl_launch_dependents();
         stamp_begin(p);
       }
       if (lane == 0 && Tl > 0) {

@@ -499,7 +499,7 @@ static cudaError_t launch_cc_attn(const Geom& g, int dev, const void* q, const v
   return launch_cc_attn_bm<T, D, 8>(g, dev, q, k, v, cache, out, ws, S, pdl, st);
 }
 template <typename T, int D, int NK>
-static cudaError_t launch_cc_score_nk(const Geom& g, int dev, const void* q, void* cache, void* ws, bool pdl, cudaStream_t st) {
+static cudaError_t launch_cc_score_nk(const Geom& g, int dev, const void* q, const void* k, void* cache, void* ws, bool pdl, cudaStream_t st) {
   constexpr int smem = kvc::score_cc_bytes<D, NK>();
   static bool attr_set[kMaxDevices] = {};
   if (cudaError_t e = opt_in_smem(kvc::score_cc_kernel<T, D, NK>, smem, attr_set, dev)) return e;
@@ -512,14 +512,14 @@ static cudaError_t launch_cc_score_nk(const Geom& g, int dev, const void* q, voi
   LaunchAttrs la(0, pdl);
   lc.attrs = la.at;
   lc.numAttrs = la.n;
-  return cudaLaunchKernelEx(&lc, kvc::score_cc_kernel<T, D, NK>, (const T*)q, (const char*)cache, (char*)ws, g);
+  return cudaLaunchKernelEx(&lc, kvc::score_cc_kernel<T, D, NK>, (const T*)q, (const T*)k, (const char*)cache, (char*)ws, g);
 }
 template <typename T, int D>
-static cudaError_t launch_cc_score(const Geom& g, int dev, const void* q, void* cache, void* ws, bool pdl, cudaStream_t st) {
+static cudaError_t launch_cc_score(const Geom& g, int dev, const void* q, const void* k, void* cache, void* ws, bool pdl, cudaStream_t st) {
   // 32 keys per CTA read the observer rows half as often (8 kv-heads x 608 keys, d = 64: 6.5 us against 7.5); 16 spread
   // a launch that does not fill the GPU over twice the SMs (2 x 1056 keys, d = 128: 7.9 us against 11.1)
-  if ((long long)(g.n_cand + 31) / 32 * g.Hkv * g.nl > kvc::kNumSMs) return launch_cc_score_nk<T, D, 32>(g, dev, q, cache, ws, pdl, st);
-  return launch_cc_score_nk<T, D, 16>(g, dev, q, cache, ws, pdl, st);
+  if ((long long)(g.n_cand + 31) / 32 * g.Hkv * g.nl > kvc::kNumSMs) return launch_cc_score_nk<T, D, 32>(g, dev, q, k, cache, ws, pdl, st);
+  return launch_cc_score_nk<T, D, 16>(g, dev, q, k, cache, ws, pdl, st);
 }
 
 // Launch shape of the tensor-core attention: R row tiles per CTA (1 or 2) and, with one, the key split S over a cluster.
@@ -586,8 +586,8 @@ static cudaError_t launch_tc_attn(const Geom& g, int dev, const CUtensorMap& tq,
 }
 // a2..a4 fused (compress.cuh).  MODE: kvc::kScoresGiven / kScoreAttention / kScoreKeyDiff.
 template <int D, int MODE, int OBS = kvc::kMaxObsRowsFused>
-static cudaError_t launch_compress(const Geom& g, int dev, const CUtensorMap& tk, const CUtensorMap& tqo, void* cache, void* ws,
-                                   int elem_bytes, bool pdl, bool wide_ok, int cn_cap, cudaStream_t st) {
+static cudaError_t launch_compress(const Geom& g, int dev, const CUtensorMap& tk, const CUtensorMap& tqo, const CUtensorMap& tkin,
+                                   const void* k, void* cache, void* ws, int elem_bytes, bool pdl, bool wide_ok, int cn_cap, cudaStream_t st) {
   const int score_bytes = MODE == kvc::kScoreAttention ? 2 * (D / 64) * kvc::kSubTileBytesC + (D / 64) * OBS * 128 : 0;
   const int table_bytes = kvc::kMaxKeysSmem * 8 + 2 * kvc::kMaxMovesSmem * 4 + 2 * kvc::kSelBins * 4;   // keys, move tables, histograms
   const int smem_min = (score_bytes > table_bytes ? score_bytes : table_bytes) + 1024;
@@ -621,7 +621,7 @@ static cudaError_t launch_compress(const Geom& g, int dev, const CUtensorMap& tk
     return slot;
   };
   // cluster size: spread one kv-head over several SMs when the heads alone cannot fill the GPU
-  const int n_tiles = (g.n_cand + 127) / 128;
+  const int n_tiles = MODE == kvc::kScoreAttention ? (g.n_sc + 127) / 128 + (g.n_cand - g.n_sc + 127) / 128 : (g.n_cand + 127) / 128;
   int Cn = (int)(kvc::kNumSMs / ((long long)g.Hkv * g.nl));
   if (Cn > kvc::kMaxClusterWide) Cn = kvc::kMaxClusterWide;
   // More than the portable 8 CTAs only while every cluster of the launch can be resident at once, and only in stream
@@ -646,7 +646,7 @@ static cudaError_t launch_compress(const Geom& g, int dev, const CUtensorMap& tk
   LaunchAttrs la(Cn, pdl);
   lc.attrs = la.at;
   lc.numAttrs = la.n;
-  return cudaLaunchKernelEx(&lc, kvc::compress_kernel<D, MODE, OBS>, tk, tqo, (char*)cache, (char*)ws, g, Cn, elem_bytes);
+  return cudaLaunchKernelEx(&lc, kvc::compress_kernel<D, MODE, OBS>, tk, tqo, tkin, (const char*)k, (char*)cache, (char*)ws, g, Cn, elem_bytes);
 }
 
 template <int D>
@@ -716,6 +716,10 @@ static int run_chunk(kvc_ctx* c, int layer0, int nl, const void* q, long long q_
   // cache); the layer then works in its own workspace slot, and the next call that touches the layer waits
   const bool async_compress = (cf.flags & 16u) && nl == 1 && allow_async && c->use_tc;
   g.slot0 = async_compress ? layer0 : 0;
+  // In stream order the score phase reads the block's keys from the input and so can start before the attention has
+  // ended; on a side stream the caller may reuse k by then.
+  g.n_sc = async_compress ? g.tot : g.n_c;
+  if (g.n_sc > g.n_cand && cf.policy != KVC_SCORE_KEYDIFF) g.n_sc = g.n_cand;
   g.lse_off = c->lse_off; g.score_off = c->score_off; g.msrc_off = c->msrc_off; g.mdst_off = c->mdst_off;
   g.mcount_off = c->mcount_off;
   g.wait_limit_k = c->wait_limit_k;
@@ -772,6 +776,12 @@ static int run_chunk(kvc_ctx* c, int layer0, int nl, const void* q, long long q_
     // (a layer whose compress kernel runs beside the next attention wants SMs left for it)
     const AttnShape sh = attn_launch_shape(g, !(cf.flags & 4u), async_compress && evict ? std::min(4 * g.Hkv * g.nl, kvc::kNumSMs) : 0);
     attn_ctas = sh.ctas;
+    // The query-agnostic score needs nothing of the attention: its kernel starts at once if it fits beside it (4 kv-heads,
+    // 88 + 32 CTAs: 1519 us per request against 1594; 112 + 72 CTAs: 2909 against 2888).  The query-aware one has only
+    // loads and products to do early, for which the end of the key loop is soon enough.
+    const long long heads = (long long)g.Hkv * g.nl;
+    const long long cluster = std::min<long long>({kvc::kMaxClusterWide, kvc::kNumSMs / heads, (g.n_cand + 255) / 256});
+    g.early = evict && !async_compress && cf.policy == KVC_SCORE_KEYDIFF && cluster > 0 && attn_ctas + heads * cluster <= kvc::kNumSMs;
     auto launch = [&](auto launcher) { return launcher(g, dev, tq, tk, tv, tkin, tvin, tout, cache, out, ws, sh.S, sh.n_pairs, pdl, st); };
     if (D == 128) e = sh.R == 2 ? launch(launch_tc_attn<128, 2>) : launch(launch_tc_attn<128, 1>);
     else e = sh.R == 2 ? launch(launch_tc_attn<64, 2>) : launch(launch_tc_attn<64, 1>);
@@ -822,9 +832,9 @@ static int run_chunk(kvc_ctx* c, int layer0, int nl, const void* q, long long q_
       if (c->use_tc) {
         e = D == 128 ? launch_tc_score<128>(g, dev, tk, tqo, ws, tok_per_group, st) : launch_tc_score<64>(g, dev, tk, tqo, ws, tok_per_group, st);
       } else if (f32) {
-        e = D == 128 ? launch_cc_score<float, 128>(g, dev, q, cache, ws, pdl, st) : launch_cc_score<float, 64>(g, dev, q, cache, ws, pdl, st);
+        e = D == 128 ? launch_cc_score<float, 128>(g, dev, q, k, cache, ws, pdl, st) : launch_cc_score<float, 64>(g, dev, q, k, cache, ws, pdl, st);
       } else {
-        e = D == 128 ? launch_cc_score<__nv_bfloat16, 128>(g, dev, q, cache, ws, pdl, st) : launch_cc_score<__nv_bfloat16, 64>(g, dev, q, cache, ws, pdl, st);
+        e = D == 128 ? launch_cc_score<__nv_bfloat16, 128>(g, dev, q, k, cache, ws, pdl, st) : launch_cc_score<__nv_bfloat16, 64>(g, dev, q, k, cache, ws, pdl, st);
       }
       if (e != cudaSuccess) return check_cuda(c, e, "score launch");
       c->launches++;
@@ -833,13 +843,13 @@ static int run_chunk(kvc_ctx* c, int layer0, int nl, const void* q, long long q_
     {
       ProfScope ps(c, 3, st);
       g.stamps = next_stamp(c, 3);
-      if (keydiff) e = launch_compress<64, kvc::kScoreKeyDiff>(g, dev, tk, tk, cache, ws, (int)c->elem, pdl, !async_compress, cn_cap, st);
+      if (keydiff) e = launch_compress<64, kvc::kScoreKeyDiff>(g, dev, tk, tk, tkin, k, cache, ws, (int)c->elem, pdl, !async_compress, cn_cap, st);
       else if (fused_score && wide_obs)
-        e = D == 128 ? launch_compress<128, kvc::kScoreAttention, kvc::kMaxObsRowsWide>(g, dev, tk, tqo, cache, ws, (int)c->elem, pdl, !async_compress, cn_cap, st)
-                     : launch_compress<64, kvc::kScoreAttention, kvc::kMaxObsRowsWide>(g, dev, tk, tqo, cache, ws, (int)c->elem, pdl, !async_compress, cn_cap, st);
-      else if (fused_score) e = D == 128 ? launch_compress<128, kvc::kScoreAttention>(g, dev, tk, tqo, cache, ws, (int)c->elem, pdl, !async_compress, cn_cap, st)
-                                         : launch_compress<64, kvc::kScoreAttention>(g, dev, tk, tqo, cache, ws, (int)c->elem, pdl, !async_compress, cn_cap, st);
-      else e = launch_compress<64, kvc::kScoresGiven>(g, dev, tk, tk, cache, ws, (int)c->elem, pdl, !async_compress, cn_cap, st);
+        e = D == 128 ? launch_compress<128, kvc::kScoreAttention, kvc::kMaxObsRowsWide>(g, dev, tk, tqo, tkin, k, cache, ws, (int)c->elem, pdl, !async_compress, cn_cap, st)
+                     : launch_compress<64, kvc::kScoreAttention, kvc::kMaxObsRowsWide>(g, dev, tk, tqo, tkin, k, cache, ws, (int)c->elem, pdl, !async_compress, cn_cap, st);
+      else if (fused_score) e = D == 128 ? launch_compress<128, kvc::kScoreAttention>(g, dev, tk, tqo, tkin, k, cache, ws, (int)c->elem, pdl, !async_compress, cn_cap, st)
+                                         : launch_compress<64, kvc::kScoreAttention>(g, dev, tk, tqo, tkin, k, cache, ws, (int)c->elem, pdl, !async_compress, cn_cap, st);
+      else e = launch_compress<64, kvc::kScoresGiven>(g, dev, tk, tk, tkin, k, cache, ws, (int)c->elem, pdl, !async_compress, cn_cap, st);
     }
     if (e != cudaSuccess) return check_cuda(c, e, "compress launch");
     c->launches++;

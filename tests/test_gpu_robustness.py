@@ -222,3 +222,39 @@ def test_host_blocks_of_different_sizes_do_not_overwrite_each_other():
         assert b.status() == 0
         for (layer, p, _), o, w in zip(calls, outs, want):
             assert torch.equal(o, w.cpu()), f"layer {layer}, position {p}"
+
+
+# ------------------------------------------------------------------------------------------------
+# inputs reused in stream order right behind a call
+
+@pytest.mark.parametrize("dtype,policy,flags", [(torch.bfloat16, 0, 0), (torch.bfloat16, 0, 16), (torch.bfloat16, 1, 0),
+                                                 (torch.bfloat16, 1, 16), (torch.float32, 0, 0), (torch.float32, 1, 0)])
+def test_inputs_may_be_reused_behind_a_call(dtype, policy, flags):
+    # k and v (and q, unless compress runs on a side stream) may be overwritten by the stream's next work although the
+    # scoring reads q and k: results equal those of calls whose inputs stay
+    hq, hkv, d, n, B, layers = 8, 4, 128, 200, 300, 2
+    torch.manual_seed(5)
+    data = [[torch.randn(n, h, d, device="cuda").to(dtype) for h in (hq, hkv, hkv)] for _ in range(5 * layers)]
+    res = []
+    for reuse in (False, True):
+        kvc = Kvc(layers, hq, hkv, d, dtype, B, n, policy=policy, flags=flags)
+        buf = [[torch.empty_like(t) for t in data[0]] for _ in range(layers)]
+        outs = []
+        for i, qkv in enumerate(data):
+            layer = i % layers
+            ins = buf[layer] if reuse else [t.clone() for t in qkv]
+            if reuse:
+                for b, t in zip(ins, qkv):
+                    b.copy_(t)
+            out = kvc.prefill_chunk(layer, *ins, (i // layers) * n)
+            if reuse:
+                for t in (ins[1:] if flags & 16 else ins):
+                    t.fill_(7.0)
+                if flags & 16:
+                    kvc.join()                  # q is overwritten by the next use of the buffer
+            outs.append(out)
+        kvc.join()
+        assert kvc.status() == 0
+        res.append((outs, [kvc.cache_view(l)[2][:, :B].clone() for l in range(layers)]))
+    assert all(torch.equal(a, b) for a, b in zip(res[0][0], res[1][0]))
+    assert all(torch.equal(a, b) for a, b in zip(res[0][1], res[1][1]))
