@@ -566,10 +566,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
         }
       } else {
         // Combine the partials of the cluster (S is a power of two; rank s owns rows [s*rows_per, (s+1)*rows_per)).
-        // Each group writes its columns of the merged rows into a staging tile whose rows carry (m, l) behind the D
-        // values; the rows of every other owner then leave in ONE bulk copy each (shared memory to the owner's shared
-        // memory, completing on a barrier of the owner: this GPU's memory, no multicast), and each rank reduces its
-        // rows from the staging tile (its own partial) and from what the others sent:
+        // A thread has its row's merged columns in registers.  The owner's threads keep them (up to S = 4; clusters of two
+        // 15.6 -> 15.0 us, 16.6 -> 15.9; with eight 12.5 -> 13.0, hence not there); the others write theirs into
+        // a staging tile whose rows carry (m, l) behind the D values, the rows of every other owner leave in ONE bulk copy
+        // each (shared memory to the owner's shared memory, completing on a barrier of the owner: this GPU's memory, no
+        // multicast), and the owner's threads fold in what arrived and write:
         //   O = sum_s 2^(m_s - m*) O_s / sum_s 2^(m_s - m*) l_s.
         // Over the ring: the received rows [S - 1 sources][rows_per][D + 4] and the staging tile [128][D + 4] (a row
         // stride of D + 4 floats keeps thread-per-row accesses off each other's banks).
@@ -577,6 +578,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
         const int rows_per = 128 / S;
         float* recv = reinterpret_cast<float*>(ring);
         float* stg = recv + (128 - rows_per) * RS;
+        const bool own = S < 8 && r / rows_per == split;
+        float f[H];
 #pragma unroll
         for (int c = 0; c < H / 32; ++c) {
           uint32_t o[32], q[32];
@@ -586,16 +589,14 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
           if (ok && both) tmem_ld32(tO1 + c * 32, q);
           tmem_wait_ld();
 #pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            float4 v4;
-            v4.x = fmaf(w1, __uint_as_float(q[4 * k + 0]), w0 * __uint_as_float(o[4 * k + 0]));
-            v4.y = fmaf(w1, __uint_as_float(q[4 * k + 1]), w0 * __uint_as_float(o[4 * k + 1]));
-            v4.z = fmaf(w1, __uint_as_float(q[4 * k + 2]), w0 * __uint_as_float(o[4 * k + 2]));
-            v4.w = fmaf(w1, __uint_as_float(q[4 * k + 3]), w0 * __uint_as_float(o[4 * k + 3]));
-            *reinterpret_cast<float4*>(stg + r * RS + t * H + (c * 8 + k) * 4) = v4;
-          }
+          for (int i = 0; i < 32; ++i) f[c * 32 + i] = fmaf(w1, __uint_as_float(q[i]), w0 * __uint_as_float(o[i]));
         }
-        if (t == 0) *reinterpret_cast<float2*>(stg + r * RS + D) = make_float2(m_all, L);
+        if (!own) {
+#pragma unroll
+          for (int k = 0; k < H / 4; ++k)
+            *reinterpret_cast<float4*>(stg + r * RS + t * H + k * 4) = make_float4(f[4 * k], f[4 * k + 1], f[4 * k + 2], f[4 * k + 3]);
+          if (t == 0) *reinterpret_cast<float2*>(stg + r * RS + D) = make_float2(m_all, L);
+        }
         fence_proxy_async_smem();                              // the rows just written are read by bulk copies
         named_barrier(1, 256);
         cluster_wait();                                        // every CTA of the cluster is done with its ring
@@ -608,46 +609,87 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
           }
         }
         ok = mbar_wait(&sh.comb_full, 0, abort_flag) && ok;    // the other ranks' rows have landed
-        constexpr int CW = 16;                                 // columns per work item: (row, piece)
-        const int r0 = split * rows_per;
+        if (S == 8) {
+          // (16 rows per owner: two warps with a row per thread would be alone; every thread takes a piece of a row)
+          constexpr int CW = 16;                                 // columns per work item: (row, piece)
+          const int r0 = split * rows_per;
 #pragma unroll 1
-        for (int item = threadIdx.x; item < rows_per * (D / CW); item += 256) {
-          const int lr = item & (rows_per - 1), pc = item / rows_per, rr = r0 + lr;
-          const int tk = tokA + rr / p.G;
-          if (!(rr < rows && tk < p.n)) continue;
-          const float* own = stg + rr * RS;
-          const float* got = recv + lr * RS;                   // + source * rows_per * RS
-          float m_row = own[D];
+          for (int item = threadIdx.x; item < rows_per * (D / CW); item += 256) {
+            const int lr = item & (rows_per - 1), pc = item / rows_per, rr = r0 + lr;
+            const int tk = tokA + rr / p.G;
+            if (!(rr < rows && tk < p.n)) continue;
+            const float* own = stg + rr * RS;
+            const float* got = recv + lr * RS;                   // + source * rows_per * RS
+            float m_row = own[D];
+#pragma unroll 1
+            for (int s2 = 0; s2 < S - 1; ++s2) m_row = fmaxf(m_row, got[s2 * rows_per * RS + D]);
+            float L_row = 0.f, acc[CW];
+#pragma unroll
+            for (int i = 0; i < CW; ++i) acc[i] = 0.f;
+#pragma unroll 1
+            for (int s2 = 0; s2 < S; ++s2) {                     // (source S - 1 of the loop: this rank itself)
+              const float* row = s2 < S - 1 ? got + s2 * rows_per * RS : own;
+              const float2 ml = *reinterpret_cast<const float2*>(row + D);
+              const float wt = ml.x == -INFINITY ? 0.f : fast_exp2(ml.x - m_row);   // -inf: the source saw no key of the row
+              L_row = fmaf(wt, ml.y, L_row);
+#pragma unroll
+              for (int k = 0; k < CW / 4; ++k) {
+                const float4 v4 = *reinterpret_cast<const float4*>(row + pc * CW + k * 4);
+                acc[4 * k + 0] = fmaf(wt, v4.x, acc[4 * k + 0]); acc[4 * k + 1] = fmaf(wt, v4.y, acc[4 * k + 1]);
+                acc[4 * k + 2] = fmaf(wt, v4.z, acc[4 * k + 2]); acc[4 * k + 3] = fmaf(wt, v4.w, acc[4 * k + 3]);
+              }
+            }
+            const float inv = 1.f / L_row;
+            const long long orow = static_cast<long long>(tk) * p.Hq + head_row + rr % p.G;
+#pragma unroll
+            for (int k = 0; k < CW / 8; ++k) {
+              uint4 vv;
+              vv.x = pack_bf16x2(acc[8 * k + 0] * inv, acc[8 * k + 1] * inv);
+              vv.y = pack_bf16x2(acc[8 * k + 2] * inv, acc[8 * k + 3] * inv);
+              vv.z = pack_bf16x2(acc[8 * k + 4] * inv, acc[8 * k + 5] * inv);
+              vv.w = pack_bf16x2(acc[8 * k + 6] * inv, acc[8 * k + 7] * inv);
+              reinterpret_cast<uint4*>(out + layer * p.out_ls + orow * D + pc * CW)[k] = vv;
+            }
+            if (pc == 0) reinterpret_cast<float*>(ws_slot(ws, p, layer) + p.lse_off)[orow] = (m_row + log2f(L_row)) * 0.6931471805599453f;
+          }
+        } else if (own && row_valid) {
+          const float* got = recv + (r - split * rows_per) * RS;   // + source * rows_per * RS
+          float m_row = m_all;
 #pragma unroll 1
           for (int s2 = 0; s2 < S - 1; ++s2) m_row = fmaxf(m_row, got[s2 * rows_per * RS + D]);
-          float L_row = 0.f, acc[CW];
+          const float wt0 = m_all == -INFINITY ? 0.f : fast_exp2(m_all - m_row);   // -inf: this rank saw no key of the row
+          float L_row = wt0 * L;
 #pragma unroll
-          for (int i = 0; i < CW; ++i) acc[i] = 0.f;
+          for (int i = 0; i < H; ++i) f[i] *= wt0;
 #pragma unroll 1
-          for (int s2 = 0; s2 < S; ++s2) {                     // (source S - 1 of the loop: this rank itself)
-            const float* row = s2 < S - 1 ? got + s2 * rows_per * RS : own;
+          for (int s2 = 0; s2 < S - 1; ++s2) {
+            const float* row = got + s2 * rows_per * RS;
             const float2 ml = *reinterpret_cast<const float2*>(row + D);
-            const float wt = ml.x == -INFINITY ? 0.f : fast_exp2(ml.x - m_row);   // -inf: the source saw no key of the row
+            const float wt = ml.x == -INFINITY ? 0.f : fast_exp2(ml.x - m_row);
             L_row = fmaf(wt, ml.y, L_row);
 #pragma unroll
-            for (int k = 0; k < CW / 4; ++k) {
-              const float4 v4 = *reinterpret_cast<const float4*>(row + pc * CW + k * 4);
-              acc[4 * k + 0] = fmaf(wt, v4.x, acc[4 * k + 0]); acc[4 * k + 1] = fmaf(wt, v4.y, acc[4 * k + 1]);
-              acc[4 * k + 2] = fmaf(wt, v4.z, acc[4 * k + 2]); acc[4 * k + 3] = fmaf(wt, v4.w, acc[4 * k + 3]);
+            for (int k = 0; k < H / 4; ++k) {
+              const float4 v4 = *reinterpret_cast<const float4*>(row + t * H + k * 4);
+              f[4 * k + 0] = fmaf(wt, v4.x, f[4 * k + 0]); f[4 * k + 1] = fmaf(wt, v4.y, f[4 * k + 1]);
+              f[4 * k + 2] = fmaf(wt, v4.z, f[4 * k + 2]); f[4 * k + 3] = fmaf(wt, v4.w, f[4 * k + 3]);
             }
           }
           const float inv = 1.f / L_row;
-          const long long orow = static_cast<long long>(tk) * p.Hq + head_row + rr % p.G;
+          const long long orow = static_cast<long long>(tok) * p.Hq + head_row + hh;
+          __nv_bfloat16* dst = out + layer * p.out_ls + orow * D + t * H;
 #pragma unroll
-          for (int k = 0; k < CW / 8; ++k) {
-            uint4 vv;
-            vv.x = pack_bf16x2(acc[8 * k + 0] * inv, acc[8 * k + 1] * inv);
-            vv.y = pack_bf16x2(acc[8 * k + 2] * inv, acc[8 * k + 3] * inv);
-            vv.z = pack_bf16x2(acc[8 * k + 4] * inv, acc[8 * k + 5] * inv);
-            vv.w = pack_bf16x2(acc[8 * k + 6] * inv, acc[8 * k + 7] * inv);
-            reinterpret_cast<uint4*>(out + layer * p.out_ls + orow * D + pc * CW)[k] = vv;
+          for (int k = 0; k < H / 16; ++k) {
+            uint32_t pk[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) pk[i] = pack_bf16x2(f[16 * k + 2 * i] * inv, f[16 * k + 2 * i + 1] * inv);
+            if ((reinterpret_cast<uintptr_t>(dst) & 31) == 0) {
+              st_global_v8(dst + 16 * k, pk);
+            } else {
+              reinterpret_cast<uint4*>(dst)[2 * k] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+              reinterpret_cast<uint4*>(dst)[2 * k + 1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+            }
           }
-          if (pc == 0) reinterpret_cast<float*>(ws_slot(ws, p, layer) + p.lse_off)[orow] = (m_row + log2f(L_row)) * 0.6931471805599453f;
+          if (t == 0) reinterpret_cast<float*>(ws_slot(ws, p, layer) + p.lse_off)[orow] = (m_row + log2f(L_row)) * 0.6931471805599453f;
         }
         // A CTA must not exit while a bulk copy still reads its staging tile: every rank has waited for the copies
         // addressed to it, so once all of them are here every copy is complete.
