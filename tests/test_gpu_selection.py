@@ -1,0 +1,50 @@
+"""The selection where its form changes: few candidates (all ranked directly), one more, and cut-offs decided by age."""
+import pytest
+import torch
+
+from oracle.kvc_oracle import KVCOracle
+from paper_2604_16734_b200.binding import Kvc
+from parity_util import compare_chunk
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype,B,chunks", [
+    (torch.float32, 96, (96, 32, 64, 65, 1)),           # 96, 128 (ranked directly), 129 and 96 candidates
+    (torch.bfloat16, 40, (40, 33, 1, 2)),               # windows of one and two rows
+])
+def test_candidate_counts(dtype, B, chunks):
+    torch.manual_seed(B)
+    d, hq, hkv = 64, 2, 2
+    kvc = Kvc(1, hq, hkv, d, dtype, B, max(chunks))
+    orc = KVCOracle(1, hq, hkv, d, B, 32)
+    pos = 0
+    for n in chunks:
+        q, k, v = (torch.randn(n, h, d).to(dtype) for h in (hq, hkv, hkv))
+        compare_chunk(kvc, orc, 0, q, k, v, pos)        # retained sets bit-exact above a gap of 1e-3
+        pos += n
+
+
+@pytest.mark.parametrize("groups", [1, 3])
+@pytest.mark.parametrize("B,n", [(64, 64), (600, 400)])
+def test_equal_scores_keep_the_oldest(groups, B, n):
+    # keys of a group are identical, so their scores are equal: whole groups stay by score, the cut-off group by age
+    d, w, N = 64, 32, 4 * n - 7
+    gen = torch.Generator().manual_seed(groups)
+    u = torch.nn.functional.normalize(torch.randn(d, generator=gen), dim=0)
+    rank = torch.arange(N) % groups                                   # group 0 scores highest
+    k = ((3.0 * (1.0 - rank.float() / groups))[:, None] * u)[:, None, :].contiguous()
+    v = torch.randn(N, 1, d, generator=gen)
+    q = (u * 8.0).expand(N, 1, d).contiguous()
+    kvc = Kvc(1, 1, 1, d, torch.float32, B, n)
+    held = []
+    for p in range(0, N, n):
+        m = min(n, N - p)
+        kvc.prefill_chunk(0, q[p:p + m].cuda(), k[p:p + m].cuda(), v[p:p + m].cuda(), p)
+        cand, new = held + list(range(p, p + m - w)), list(range(p + m - w, p + m))
+        if len(cand) + w > B:
+            cand = sorted(cand, key=lambda t: (int(rank[t]), t))[:B - w]
+        held = sorted(cand + new)
+    assert kvc.status() == 0
+    _, _, pos, length = kvc.cache_view(0)
+    assert length == B and pos[0, :B].sort().values.cpu().tolist() == held
