@@ -92,13 +92,20 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
   uint8_t* ring = smem + R * TILE_BYTES;         // kStages tiles; after the key loop: the partials of a key split
   __shared__ TcSmemAttn sh;
 
-  const int layer = blockIdx.z, g = blockIdx.y;
+  // Without a key split the row tiles that see the most keys, the last ones, start first, and the kv-heads take turns: in
+  // a launch of several waves the short CTAs then fill the end (2048 tokens in one pass, 28 / 4 heads, 4 layers with five
+  // short blocks behind it: 316 -> 241 us), and in one wave the longest CTAs are not the last to get an SM (long video
+  // with compress on a side stream: 1121 -> 1060 us per request).
+  const int lin = blockIdx.y * gridDim.x + blockIdx.x;
+  const bool ordered = S == 1;
+  const int layer = blockIdx.z, g = ordered ? lin % gridDim.y : blockIdx.y;
+  const int bx = ordered ? gridDim.x - 1 - lin / gridDim.y : blockIdx.x;
   const int split = S > 1 ? static_cast<int>(cluster_ctarank()) : 0;
   // R = 1: a row tile per CTA (or per cluster).  R = 2: the first n_pairs CTAs of a kv-head take two row tiles each, the
   // others one of the rest.
   const int TOK = 128 / p.G, rows = TOK * p.G;
-  const bool has_B = R == 2 && static_cast<int>(blockIdx.x) < n_pairs;
-  const int tile0 = R == 1 ? blockIdx.x / S : has_B ? 2 * blockIdx.x : n_pairs + blockIdx.x;
+  const bool has_B = R == 2 && bx < n_pairs;
+  const int tile0 = R == 1 ? bx / S : has_B ? 2 * bx : n_pairs + bx;
   const int tokA = tile0 * TOK, tokB = tokA + TOK, tok_end = has_B ? tokB + TOK : tokB;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int last_tok = min(tok_end, p.n) - 1;
