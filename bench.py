@@ -473,7 +473,7 @@ def profile_pass(r: Runner, steps: int, batched: bool = False, events: bool = Fa
                                                     o, kv._stream()))
             moves = kv.move_counts(0).tolist() if n_c + n - t > cfg.budget else None
             w_call = t if t else min(cfg.obs_window, n)
-            fused = r.policy == 1 or (cfg.dtype == "bf16" and not (r.flags & 1) and w_call * cfg.group <= 128)
+            fused = r.policy == 1 or (cfg.dtype == "bf16" and not (r.flags & 1) and w_call * cfg.group <= 256)
             for s, wv in work_of_call(cfg, n, n_c, moves, fused, t).items():
                 work[s]["bytes"] += wv["bytes"]; work[s]["flops"] += wv["flops"]
         n_c = min(n_c + n - t, cfg.budget)

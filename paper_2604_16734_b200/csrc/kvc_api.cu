@@ -630,7 +630,12 @@ static cudaError_t launch_compress(const Geom& g, int dev, const CUtensorMap& tk
   if (!wide_ok && Cn > 8) Cn = 8;
   if (cn_cap > 0 && Cn > cn_cap) Cn = cn_cap;             // (side stream: stay within the SMs the attention leaves idle)
   while (Cn > 8 && clusters_in_flight(Cn) < (long long)g.Hkv * g.nl) --Cn;
-  const int tiles_per_cta = 2;                            // fewer, and the cluster barriers cost more than the tiles
+  // One key tile per CTA in stream order while the launch stays small, else two: 2 kv-heads x 10 tiles 8.1 -> 7.6 us, 8 x 5 7.7 -> 7.3,
+  // 8 x 18 9.7 -> 9.4; but 32 x 5 7.5 -> 7.7, 16 clusters of nine CTAs do not find their SMs at once (12.9 -> 24),
+  // beside another attention (side stream) 32 x 3 1509 -> 1541 per request, and with 224 observer rows 1682 -> 1692.
+  // (The query-agnostic score keeps two: the order of its sums depends on the cluster size.)
+  const bool small = MODE == kvc::kScoreAttention && !kAlone && wide_ok && (long long)std::min(Cn, n_tiles) * g.Hkv * g.nl <= 100;
+  const int tiles_per_cta = small ? 1 : 2;                // fewer, and the cluster barriers cost more than the tiles
   if (Cn > (n_tiles + tiles_per_cta - 1) / tiles_per_cta) Cn = (n_tiles + tiles_per_cta - 1) / tiles_per_cta;
   if (Cn < 1) Cn = 1;
   // Two CTAs share an SM only when there are more CTAs than SMs (then one scores while the other selects);
