@@ -534,7 +534,12 @@ static cudaError_t launch_cc_score(const Geom& g, int dev, const void* q, const 
 // (An exchange of the partials through an L2-resident global buffer instead of distributed shared memory was measured
 // too: slower, the release / acquire round trip costs more than the narrow SM-to-SM path.)
 struct AttnShape { int R, S, n_pairs; long long ctas; };
-static AttnShape attn_launch_shape(const Geom& g, bool allow_split, int reserve) {
+static AttnShape attn_launch_shape(const Geom& g, bool allow_split, bool evict) {
+  // SMs that mixed launches leave to a compress kernel on a side stream.  In stream order nobody needs them, but the
+  // launch shape decides how a row's keys are grouped and thereby the last bits of the output: results must not depend on
+  // KVC_FLAG_ASYNC_COMPRESS.  (In stream order this costs 4 - 6 % of a request whose launches are mixed, e.g. 784 x 7 rows
+  // 1073 -> 1119 us; no reserve in either mode would cost 2 - 14 % on the side streams.)
+  const int reserve = evict && g.nl == 1 ? std::min(4 * g.Hkv, kvc::kNumSMs) : 0;
   const int TOK = 128 / g.G;
   const int tiles = (g.n + TOK - 1) / TOK;
   const int Tc = (g.n_c + 127) / 128, T = Tc + (g.n + 127) / 128;
@@ -546,8 +551,9 @@ static AttnShape attn_launch_shape(const Geom& g, bool allow_split, int reserve)
   double best_us = tiles == 1 ? INFINITY : waves(best.ctas, kvc::kNumSMs) * (T * 1.78 + 4.3);   // a single row tile never fills a pair
   // Pairs that would leave SMs idle: the row tiles with the most keys, the last ones, get a CTA each instead (1.2 us per
   // key tile there: their ring has four slots).  784 x 7 rows, 4 kv-heads, 2832 keys: 46.5 -> 38.2 us; 640 x 4, 8, d = 64
-  // 31.5 -> 25.7; 1024 x 4, 8, 5120 keys 78.4 -> 76.6.  With compress on a side stream four SMs per kv-head stay free for
-  // it (`reserve`): per step 1190 -> 1054, 311 -> 275 and 1120 -> 1108 us; two or none are slower on most shapes.
+  // 31.5 -> 25.7; 1024 x 4, 8, 5120 keys 78.4 -> 76.6, all without the reserve.  With it, requests with compress on a side
+  // stream take, against none: 700 x 1 rows, 32 kv-heads 469 -> 411 us, 640 x 4, 8, d = 64 620 -> 604, 1024 x 4,
+  // 8 2654 -> 2589, 784 x 7, 4 891 -> 898.
   const long long per_head = (kvc::kNumSMs - reserve) / heads;
   if (per_head > tiles - tiles / 2 && per_head < tiles) {
     const int n_pairs = (int)(tiles - per_head);
@@ -778,8 +784,7 @@ static int run_chunk(kvc_ctx* c, int layer0, int nl, const void* q, long long q_
   ProfScope ps(c, 1, st);
   g.stamps = next_stamp(c, 1);
   if (c->use_tc) {
-    // (a layer whose compress kernel runs beside the next attention wants SMs left for it)
-    const AttnShape sh = attn_launch_shape(g, !(cf.flags & 4u), async_compress && evict ? std::min(4 * g.Hkv * g.nl, kvc::kNumSMs) : 0);
+    const AttnShape sh = attn_launch_shape(g, !(cf.flags & 4u), evict);
     attn_ctas = sh.ctas;
     // The query-agnostic score needs nothing of the attention: its kernel starts at once if it fits beside it (4 kv-heads,
     // 88 + 32 CTAs: 1519 us per request against 1594; 112 + 72 CTAs: 2909 against 2888).  The query-aware one has only

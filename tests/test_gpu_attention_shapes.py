@@ -66,3 +66,27 @@ def test_output_at_sixteen_byte_alignment():
     b.prefill_chunk(0, q, k, v, 0, shifted)
     assert a.status() == 0 and b.status() == 0
     assert torch.equal(ref, shifted) and not whole[:8].any() and not whole[8 + n * hq * d:].any()
+
+
+@pytest.mark.parametrize("hq,hkv,d,n,B,window", [
+    (28, 4, 128, 784, 2048, 32),                      # pairs and single row tiles
+    (32, 8, 64, 640, 1000, 32),
+    (32, 32, 128, 700, 500, 8),                       # the first block already evicts
+])
+def test_compress_on_a_side_stream_gives_the_same_bits(hq, hkv, d, n, B, window):
+    layers, N = 2, B + 4 * n - 5
+    torch.manual_seed(n)
+    qkv = [[torch.randn(N, h, d, device="cuda", dtype=torch.bfloat16) for h in (hq, hkv, hkv)] for _ in range(layers)]
+    res = []
+    for flags in (0, KVC_FLAG_ASYNC_COMPRESS):
+        kvc = Kvc(layers, hq, hkv, d, torch.bfloat16, B, n, window, flags=flags)
+        outs = [kvc.prefill_chunk(l, *(x[p:p + n] for x in qkv[l]), p) for p in range(0, N, n) for l in range(layers)]
+        kvc.join()
+        assert kvc.status() == 0
+        last = B + len(range(N)[(N - 1) // n * n:]) - window
+        res.append((outs, [t for l in range(layers) for t in kvc.cache_view(l)[:3]],
+                    kvc.workspace_view(kvc.slot_of(layers - 1))[1][:, :last].clone()))
+    (outs_a, cache_a, score_a), (outs_b, cache_b, score_b) = res
+    assert all(torch.equal(a, b) for a, b in zip(outs_a, outs_b))
+    assert all(torch.equal(a[:, :B], b[:, :B]) for a, b in zip(cache_a, cache_b))
+    assert torch.equal(score_a, score_b)
