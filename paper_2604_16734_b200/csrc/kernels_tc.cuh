@@ -774,7 +774,9 @@ __global__ void __launch_bounds__(128) score_tc_kernel(const __grid_constant__ C
     for (int sub = 0; sub < NSUB; ++sub)
       tma_load_4d(sK + sub * kSubTileBytes, &tm_k, &sh.bar_k, sub * 64, key0, g, layer);
   }
-  float acc = 0.f;
+  // two sums, over the even and the odd 16-column pieces, as in the fused kernel: a launch of up to 256 observer rows may
+  // take either form, and its scores must not depend on which
+  float acc[2] = {0.f, 0.f};
   bool ok = true;
   const int n_groups = (p.w + tok_per_group - 1) / tok_per_group;
   for (int grp = 0; grp < n_groups && ok; ++grp) {
@@ -813,16 +815,22 @@ __global__ void __launch_bounds__(128) score_tc_kernel(const __grid_constant__ C
     ok = mbar_wait(&sh.bar_s, grp & 1, abort_flag);
     if (!ok) break;
     tc_fence_after_sync();
-    for (int c0 = 0; c0 < n_mma; c0 += 16) {
-      uint32_t sr[16];
+    for (int c0 = 0; c0 < n_mma; c0 += 32) {                           // the second half may be absent
+      uint32_t sr[32];
+      const bool two = c0 + 16 < n_mma;
       tmem_ld16(tmem + lane_addr + c0, sr);
+      if (two) tmem_ld16(tmem + lane_addr + c0 + 16, sr + 16);
       tmem_wait_ld();
 #pragma unroll
-      for (int i = 0; i < 16; ++i) acc += fast_exp2(__uint_as_float(sr[i]) * p.scale_log2 - sh.lse2[c0 + i]);
+      for (int i = 0; i < 16; ++i) acc[0] += fast_exp2(fmaf(__uint_as_float(sr[i]), p.scale_log2, -sh.lse2[c0 + i]));
+      if (two) {
+#pragma unroll
+        for (int i = 16; i < 32; ++i) acc[1] += fast_exp2(fmaf(__uint_as_float(sr[i]), p.scale_log2, -sh.lse2[c0 + i]));
+      }
     }
   }
   const int key = key0 + threadIdx.x;
-  if (ok && key < p.n_cand) score[key] = acc;
+  if (ok && key < p.n_cand) score[key] = acc[0] + acc[1];
   tc_fence_before_sync();
   __syncthreads();
   if (warp == 0) {
