@@ -58,7 +58,7 @@ struct CompressSmem {
   alignas(16) float lse2[256];
   unsigned long long list[2 * (kTeam / 32) + 2];
   int scan_scratch[kTeam / 32 + 1];
-  unsigned long long s_prefix;
+  unsigned long long s_prefix, lowest_kept;
   int s_remaining, s_bin_count, s_count;
 };
 
@@ -399,6 +399,7 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
     if (lane == 0) { sh.list[warp] = (static_cast<unsigned long long>(a_hi) << 32) | a_lo; sh.list[kTeam / 32 + warp] = (static_cast<unsigned long long>(o_hi) << 32) | o_lo; }
   }
   for (int i = tid; i < kSelBins; i += kTeam) hists[0][i] = 0;
+  if (tid == 0) sh.s_prefix = sh.lowest_kept = ~0ull;
   __syncthreads();
   // Selection and listing exist twice, for keys in shared memory and for keys re-read from the workspace: with the
   // choice made per access the compiler issues the global loads of the second form in both cases.
@@ -416,9 +417,11 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
   unsigned long long thr = ~0ull;                                // n_keep == 0: nothing among the candidates survives
   if (kInSmem && p.n_keep > 0 && p.n_cand <= kDirectMax) {
     // few candidates: rank all of them (the bits they share, a histogram round and the list would cost more)
+    unsigned long long my = 0ull;
+    int larger = p.n_keep;
     if (tid < p.n_cand) {
-      const unsigned long long my = keys[tid];
-      int larger = 0;
+      my = keys[tid];
+      larger = 0;
       int i = 0;
 #pragma unroll 4
       for (; i + 1 < p.n_cand; i += 2) {
@@ -430,6 +433,11 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
     }
     __syncthreads();
     thr = sh.s_prefix;
+    if (thr == ~0ull) {                                          // nobody has that rank: equal keys at the cut-off (a caller
+      if (larger < p.n_keep) atomicMin(&sh.lowest_kept, my);     // that repeats positions); the smallest key that survives
+      __syncthreads();
+      thr = sh.lowest_kept;
+    }
   } else if (p.n_keep > 0) {
     {                                                            // (every thread: the same values)
       static_assert(kTeam == 512, "sixteen ANDs and sixteen ORs, one per lane");

@@ -48,3 +48,24 @@ def test_equal_scores_keep_the_oldest(groups, B, n):
     assert kvc.status() == 0
     _, _, pos, length = kvc.cache_view(0)
     assert length == B and pos[0, :B].sort().values.cpu().tolist() == held
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_equal_keys_at_the_cutoff(dtype):
+    # a caller that gives two blocks the same positions: entries with equal score and position, two of them at ranks 15 and
+    # 16 of the 16 that stay
+    d, w, B, n = 64, 4, 20, 16
+    torch.manual_seed(2)
+    k = torch.randn(1, 1, d, device="cuda").expand(n, 1, d).to(dtype).contiguous()
+    q = torch.randn(1, 1, d, device="cuda").expand(n, 1, d).to(dtype).contiguous()
+    kvc = Kvc(1, 1, 1, d, dtype, B, n, w)
+    vs = [torch.randn(n, 1, d, device="cuda").to(dtype) for _ in range(2)]
+    for v in vs:
+        kvc.prefill_chunk(0, q, k, v, 0)
+    assert kvc.status() == 0
+    _, V, pos, length = kvc.cache_view(0)
+    held = pos[0, :B].cpu().tolist()
+    assert length == B and sorted(held) == sorted(2 * list(range(8)) + [12, 13, 14, 15])
+    rows = {tuple(x[0].tolist()) for v in vs for x in v.cpu()}
+    assert all(tuple(x) in rows for x in V[0, :B].cpu().tolist())
+    assert len({tuple(x) for x in V[0, :B].cpu().tolist()}) == B
