@@ -94,7 +94,19 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
   int* mcount = reinterpret_cast<int*>(slot + p.mcount_off);
   volatile int* abort_flag = sh.wait_ctl;
   if (tid == 0) { sh.wait_ctl[0] = 0; sh.wait_ctl[1] = p.wait_limit_k; }
-  pdl_launch_dependents();                        // the next kernel of the stream may set itself up meanwhile
+  // The next kernel of the stream may set itself up meanwhile -- once this one has its tensor memory: a dependent that
+  // allocates some in front of its own dependency wait could otherwise take what this CTA still needs, and both would wait.
+  // (Allocating first, in this warp alone, keeps the trigger early: image request 2736 -> 2755 us, behind the block's first
+  // barrier 2759.)
+  if constexpr (MODE == kScoreAttention) {
+    if (warp == 8) {
+      tmem_alloc(&sh.tmem_base, 2 * OBS);
+      tmem_relinquish();
+      pdl_launch_dependents();
+    }
+  } else {
+    pdl_launch_dependents();
+  }
   // Before the dependency wait this kernel may read what was complete before the attention kernel of the same call began
   // its work: the call's inputs and the cache rows below n_c = n_sc (on a
   // side stream, where the caller may reuse k by now, n_sc covers all rows and there is nothing to wait for).  The attention kernel allows this launch only after its own
@@ -121,10 +133,6 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
     // observer rows beyond the real ones are padding: keep them finite
     for (int i = tid; i < NSUB * kQSubBytes / 16; i += kCompressThreads) reinterpret_cast<uint4*>(sQ)[i] = make_uint4(0, 0, 0, 0);
     fence_proxy_async_smem();
-    if (warp == 8) {
-      tmem_alloc(&sh.tmem_base, 2 * OBS);
-      tmem_relinquish();
-    }
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();

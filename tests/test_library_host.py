@@ -95,3 +95,17 @@ def test_binding_refuses_to_run_without_a_gpu():
         pytest.skip("GPU present")
     with pytest.raises(RuntimeError):
         binding.Kvc(1, 4, 1, 64, torch.float32, 128, 64)
+
+
+def test_kernels_hold_their_tensor_memory_before_a_dependent_may_start():
+    # by reading: running into it would take a dependent that holds tensor memory and waits, with no limit on either wait
+    csrc = os.path.join(ROOT, "paper_2604_16734_b200", "csrc")
+    seen = 0
+    for name in os.listdir(csrc):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, name)).read())
+        for body in text.split("__global__")[1:]:
+            body = body[:body.find("\n}\n")]
+            if "tmem_alloc(" in body and "pdl_launch_dependents()" in body:
+                seen += 1
+                assert body.index("tmem_alloc(") < body.index("pdl_launch_dependents()"), name
+    assert seen == 2
