@@ -108,9 +108,10 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
     pdl_launch_dependents();
   }
   // Before the dependency wait this kernel may read what was complete before the attention kernel of the same call began
-  // its work: the call's inputs and the cache rows below n_c = n_sc (on a
-  // side stream, where the caller may reuse k by now, n_sc covers all rows and there is nothing to wait for).  The attention kernel allows this launch only after its own
-  // wait, so everything that precedes it in the stream has finished and is visible.  (Loads, products and, for the
+  // its work: the call's inputs and the cache rows below n_c = n_sc (on a side stream, where the caller may reuse k by now,
+  // n_sc covers all rows and there is nothing to wait for).  The attention kernel allows this launch only after its own
+  // wait, so everything that precedes it in the stream has finished and is in L2; these reads go there (TMA, ld.global.cg)
+  // and never through L1, which is only known to be current behind this kernel's own wait.  (Loads, products and, for the
   // query-agnostic score, the whole phase then overlap the attention's end: 32 kv-heads x 288 candidates 7.0 -> 6.4 us
   // behind the wait, 4 x 2300 x 224 observer rows 11.6 -> 10.6, 4 x 1833 query-agnostic 10.3 -> 5.8.)
 
@@ -247,8 +248,8 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
     const long long row_bytes = static_cast<long long>(d) * elem_bytes;
     const char* Kg = blob + static_cast<long long>(g) * p.cap * row_bytes + piece * 16;
     const char* Kn = kin + (layer * p.kv_ls + static_cast<long long>(g) * d) * elem_bytes + piece * 16;
-    auto fetch = [&](int row) {                                     // (the block's rows from the input, as above)
-      return *reinterpret_cast<const uint4*>(row < p.n_sc ? Kg + row * row_bytes : Kn + (row - p.n_sc) * p.Hkv * row_bytes);
+    auto fetch = [&](int row) {                                     // (the block's rows from the input, as above; through L2)
+      return __ldcg(reinterpret_cast<const uint4*>(row < p.n_sc ? Kg + row * row_bytes : Kn + (row - p.n_sc) * p.Hkv * row_bytes));
     };
     auto widen = [&](const uint4 raw, float* f) {
       if (elem_bytes == 2) {

@@ -15,12 +15,13 @@ static constexpr int kCcThreads = 256, kCcWarps = 8;
 __device__ __forceinline__ ulonglong2 lds_f32x4(const float* s) { return *reinterpret_cast<const ulonglong2*>(s); }
 
 // Eight or four consecutive elements to shared memory as fp32: fp32 asynchronously (cp.async), bf16 through registers.
+// Both read through L2 only: the score kernel stages inputs in front of its dependency wait, where L1 may be stale.
 template <typename T>
 __device__ __forceinline__ void stage16(float* dst, const T* src) {
   if constexpr (sizeof(T) == 4) {
     cp_async16(dst, src);
   } else {
-    const uint4 raw = *reinterpret_cast<const uint4*>(src);
+    const uint4 raw = __ldcg(reinterpret_cast<const uint4*>(src));
     reinterpret_cast<float4*>(dst)[0] = make_float4(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u),
                                                     __uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u));
     reinterpret_cast<float4*>(dst)[1] = make_float4(__uint_as_float(raw.z << 16), __uint_as_float(raw.z & 0xffff0000u),

@@ -97,6 +97,15 @@ def test_binding_refuses_to_run_without_a_gpu():
         binding.Kvc(1, 4, 1, 64, torch.float32, 128, 64)
 
 
+def test_loads_in_front_of_the_dependency_wait_bypass_l1():
+    # by reading: whether a stale L1 line would ever be met cannot be provoked.  TMA and cp.async.cg read L2 by nature.
+    csrc = os.path.join(ROOT, "paper_2604_16734_b200", "csrc")
+    fetch = re.search(r"auto fetch = .*?;\n    };", open(os.path.join(csrc, "compress.cuh")).read(), re.S).group()
+    stage = re.search(r"void stage16\(.*?\n}", open(os.path.join(csrc, "kernels_cc.cuh")).read(), re.S).group()
+    for body in (fetch, stage):
+        assert "__ldcg(reinterpret_cast<const uint4*>" in body and "*reinterpret_cast<const uint4*>" not in body
+
+
 def test_kernels_hold_their_tensor_memory_before_a_dependent_may_start():
     # by reading: running into it would take a dependent that holds tensor memory and waits, with no limit on either wait
     csrc = os.path.join(ROOT, "paper_2604_16734_b200", "csrc")
