@@ -952,7 +952,7 @@ extern "C" int kvc_prefill_chunk_host(kvc_ctx* c, int layer, const void* q_host,
   // call i+1, the kernels of call i+1 (other half) and the outbound copy of call i all run at the same time.  The
   // caller's stream then waits for the outbound copy of the PREVIOUS call (the other half: its `out` area is the
   // next block's), which has had this call's kernels to finish.
-  const int half = (int)(c->host_calls++ & 1u);
+  const int half = (int)(c->host_calls & 1u);
   // The areas of a half start where those of the largest block do, whatever n is: the inbound copies of a call may run
   // while `out` of the call two before it, in the same half, is still on its way out.
   const size_t rows = c->cfg.max_chunk > c->cfg.budget ? c->cfg.max_chunk : c->cfg.budget;
@@ -970,6 +970,7 @@ extern "C" int kvc_prefill_chunk_host(kvc_ctx* c, int layer, const void* q_host,
   if ((rc = check_cuda(c, cudaStreamWaitEvent(st, c->ev_in[half], 0), "cudaStreamWaitEvent"))) return rc;
   rc = run_chunk(c, layer, 1, dq, 0, dk, dv, 0, n, pos0, cache, 0, workspace, dout, 0, st, 0, false);   // staging is reused: no side stream
   if (rc) return rc;
+  c->host_calls++;                                           // (a rejected call leaves its half to the next one)
   if ((rc = check_cuda(c, cudaEventRecord(c->ev_free[half], st), "cudaEventRecord"))) return rc;
   if ((rc = check_cuda(c, cudaStreamWaitEvent(c->copy_out, c->ev_free[half], 0), "cudaStreamWaitEvent"))) return rc;
   if ((rc = check_cuda(c, cudaMemcpyAsync(out_host, dout, qb, cudaMemcpyDeviceToHost, c->copy_out), "D2H out"))) return rc;

@@ -224,6 +224,26 @@ def test_host_blocks_of_different_sizes_do_not_overwrite_each_other():
             assert torch.equal(o, w.cpu()), f"layer {layer}, position {p}"
 
 
+def test_a_rejected_host_call_does_not_expose_the_result_of_the_call_before_it():
+    # the call after a rejected one must not put its result where that of the last accepted call may still be on its way to
+    # the host: both results lie in the staging buffer afterwards
+    hq, hkv, d, n = 8, 2, 64, 40
+    torch.manual_seed(4)
+    a, b = (Kvc(1, hq, hkv, d, torch.bfloat16, 64, n) for _ in range(2))
+    blocks = [[torch.randn(n, h, d).to(torch.bfloat16).pin_memory() for h in (hq, hkv, hkv)] for _ in range(2)]
+    want = [a.prefill_chunk(0, *(t.cuda() for t in qkv), i * n).cpu() for i, qkv in enumerate(blocks)]
+    outs = [torch.empty_like(qkv[0]).pin_memory() for qkv in blocks]
+    b.prefill_chunk_host(0, *blocks[0], 0, outs[0])
+    with pytest.raises(binding.KvcError):
+        b.prefill_chunk_host(0, *blocks[1], -1, outs[1])
+    b.prefill_chunk_host(0, *blocks[1], n, outs[1])
+    b.host_flush()
+    torch.cuda.synchronize()
+    assert b.status() == 0 and all(torch.equal(o, w) for o, w in zip(outs, want))
+    staged = b.staging.cpu().numpy().tobytes()
+    assert all(w.view(torch.uint8).numpy().tobytes() in staged for w in want)
+
+
 # ------------------------------------------------------------------------------------------------
 # inputs reused in stream order right behind a call
 
