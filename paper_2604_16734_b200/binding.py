@@ -160,7 +160,7 @@ class Kvc:
         cache = self.cache
         if layer >= cache.shape[0]:           # (a negative layer is refused by the library)
             raise IndexError(f"layer {layer} outside [0, {cache.shape[0]})")
-        return cache.data_ptr() + layer * cache.stride(0)
+        return cache.data_ptr() + layer * cache.stride(0) * cache.element_size()
 
     def _check(self, rc: int):
         if rc != KVC_OK:

@@ -89,6 +89,17 @@ def test_fp32_config_and_error_text():
     assert lib.kvc_destroy(h) == KVC_OK
 
 
+def test_blob_address_of_any_cache_tensor():
+    # a caller's own cache tensor may be of any type and row stride
+    import torch
+    kvc = binding.Kvc.__new__(binding.Kvc)
+    for cache in (torch.empty(3, 64, dtype=torch.uint8), torch.empty(3, 32, dtype=torch.bfloat16), torch.empty(3, 96, dtype=torch.int32)[:, :16]):
+        kvc.cache = cache
+        assert [kvc._blob(i) for i in range(3)] == [cache[i].data_ptr() for i in range(3)]
+        with pytest.raises(IndexError):
+            kvc._blob(3)
+
+
 def test_binding_refuses_to_run_without_a_gpu():
     import torch
     if torch.cuda.is_available():
