@@ -225,6 +225,11 @@ int kvc_workspace_view(const kvc_ctx* ctx, void* workspace, int slot, float** ls
  * entries the most recent eviction moved per kv-head during compaction. */
 int kvc_move_counts(const kvc_ctx* ctx, void* workspace, int slot, int** counts);
 
+/* The launch shape of the tensor-core attention for a call of n tokens into caches of n_c entries (n_layers: 1 unless
+ * kvc_prefill_chunk_layers): row tiles per CTA (1 or 2), the CTAs a row tile's keys are split over, and how many CTAs per
+ * kv-head take two row tiles.  Host only; KVC_EINVAL for configurations that run on the CUDA cores. */
+int kvc_attention_shape(const kvc_ctx* ctx, int n, int n_c, int n_layers, int* row_tiles, int* key_split, int* pairs);
+
 /* Orders `stream` after every compress kernel that KVC_FLAG_ASYNC_COMPRESS left on the context's own stream
  * (no host wait; a no-op when nothing is pending).  After it, work enqueued on `stream` sees the compacted
  * caches, and a stream capture that the calls were part of may end. */

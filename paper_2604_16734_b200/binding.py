@@ -24,7 +24,7 @@ EXPORTS = [
     "kvc_create", "kvc_destroy", "kvc_cache_nbytes", "kvc_workspace_init", "kvc_reset",
     "kvc_prefill_chunk", "kvc_prefill_chunk_layers", "kvc_staging_nbytes", "kvc_prefill_chunk_host", "kvc_host_flush",
     "kvc_prefill_chunk_static", "kvc_status_static", "kvc_prefill_chunk_proxy",
-    "kvc_join", "kvc_cache_view", "kvc_workspace_view", "kvc_move_counts", "kvc_status", "kvc_kv_bytes", "kvc_profile_enable",
+    "kvc_join", "kvc_cache_view", "kvc_attention_shape", "kvc_workspace_view", "kvc_move_counts", "kvc_status", "kvc_kv_bytes", "kvc_profile_enable",
     "kvc_profile_read", "kvc_launch_count", "kvc_last_error", "kvc_set_wait_limit", "kvc_selftest_wait_timeout",
     "kvc_profile_device", "kvc_profile_device_read",
 ]
@@ -69,6 +69,7 @@ def load_library() -> ctypes.CDLL:
     lib.kvc_cache_view.argtypes = [vp, i, vp, ctypes.POINTER(KvcView)]
     lib.kvc_workspace_view.argtypes = [vp, vp, i, ctypes.POINTER(vp), ctypes.POINTER(vp)]
     lib.kvc_move_counts.argtypes = [vp, vp, i, ctypes.POINTER(vp)]
+    lib.kvc_attention_shape.argtypes = [vp, i, i, i] + [ctypes.POINTER(i)] * 3
     lib.kvc_status.argtypes = [vp, vp, vp]
     lib.kvc_join.argtypes = [vp, vp]
     lib.kvc_set_wait_limit.argtypes = [vp, ll]

@@ -563,10 +563,25 @@ static AttnShape attn_launch_shape(const Geom& g, bool allow_split, bool evict) 
   }
   for (int s = 0; s < (allow_split ? 4 : 1) && (1 << s) <= T; ++s) {
     const long long ctas = (tiles * heads) << s;
-    const double est = waves(ctas, capacity[s]) * ((T + (1 << s) - 1) / (1 << s) * 0.94 + 4.3) + combine_us[s];
+    double est = waves(ctas, capacity[s]) * ((T + (1 << s) - 1) / (1 << s) * 0.94 + 4.3) + combine_us[s];
+    // A split that takes the last SMs a compress kernel on a side stream could run on must be worth that (whole calls, 32
+    // kv-heads: 4 key tiles 13.2 us with S = 4 against 8.9 with S = 1; 11: 20.7 against 14.5 with S = 2; but 37 in stream order,
+    // where the shape has to be the same, 37.4 against 43.9 with S = 2).
+    if (s > 0 && evict && g.nl == 1 && ctas + heads > kvc::kNumSMs) est += 3.0;
     if (est < best_us) { best_us = est; best = {1, 1 << s, 0, ctas}; }
   }
   return best;
+}
+
+extern "C" int kvc_attention_shape(const kvc_ctx* c, int n, int n_c, int n_layers, int* row_tiles, int* key_split, int* pairs) {
+  if (!live(c)) return KVC_ESTATE;
+  if (!c->use_tc || n < 1 || n_c < 0 || n_layers < 1 || n_layers > c->cfg.n_layers || !row_tiles || !key_split || !pairs) return KVC_EINVAL;
+  Geom g;
+  memset(&g, 0, sizeof(g));
+  g.n = n; g.n_c = n_c; g.G = c->G; g.Hkv = c->cfg.n_kv_heads; g.nl = n_layers;
+  const AttnShape s = attn_launch_shape(g, !(c->cfg.flags & KVC_FLAG_NO_KEY_SPLIT), (long long)n_c + n > c->cfg.budget);
+  *row_tiles = s.R; *key_split = s.S; *pairs = s.n_pairs;
+  return KVC_OK;
 }
 
 template <int D, int R>

@@ -81,6 +81,24 @@ def test_sizes_follow_the_memory_formula():
     assert lib.kvc_destroy(h) == KVC_OK
 
 
+def attention_shape(h, n, n_c, layers=1):
+    x = [ctypes.c_int() for _ in range(3)]
+    assert binding.lib().kvc_attention_shape(h, n, n_c, layers, *(ctypes.byref(v) for v in x)) == KVC_OK
+    return tuple(v.value for v in x)
+
+
+def test_a_short_key_range_is_not_split_at_the_price_of_the_compress_kernel():
+    # 32 kv-heads of one row tile each: split over four, the attention leaves the compress kernel beside it no SM per kv-head,
+    # which pays for long key ranges only; with fewer kv-heads there is room
+    for hkv, G, n, n_c, split in ((32, 1, 11, 270, 1), (32, 1, 4, 1639, 2), (32, 2, 4, 409, 1), (32, 1, 11, 4500, 4), (16, 1, 100, 1200, 4)):
+        rc, h = _create(n_q_heads=hkv * G, n_kv_heads=hkv, budget=n_c, max_chunk=128)
+        assert rc == KVC_OK and attention_shape(h, n, n_c) == (1, split, 0), (hkv, n, n_c)
+        assert binding.lib().kvc_destroy(h) == KVC_OK
+    rc, h = _create(dtype=KVC_F32)
+    assert binding.lib().kvc_attention_shape(h, 8, 8, 1, *[ctypes.byref(ctypes.c_int()) for _ in range(3)]) == KVC_EINVAL
+    assert binding.lib().kvc_destroy(h) == KVC_OK
+
+
 def test_fp32_config_and_error_text():
     lib = binding.lib()
     rc, h = _create(dtype=KVC_F32, head_dim=64, n_q_heads=4, n_kv_heads=1, budget=128, max_chunk=64)
