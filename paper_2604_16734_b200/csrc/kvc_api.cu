@@ -658,6 +658,10 @@ static cudaError_t launch_compress(const Geom& g, int dev, const CUtensorMap& tk
   const bool small = MODE == kvc::kScoreAttention && !kAlone && wide_ok && (long long)std::min(Cn, n_tiles) * g.Hkv * g.nl <= 100;
   const int tiles_per_cta = small ? 1 : 2;                // fewer, and the cluster barriers cost more than the tiles
   if (Cn > (n_tiles + tiles_per_cta - 1) / tiles_per_cta) Cn = (n_tiles + tiles_per_cta - 1) / tiles_per_cta;
+  // Clusters that the GPU cannot hold at once (one CTA per SM: 15 of seven to nine, 22 of six, 33 of four) run in two waves:
+  // 16 kv-heads x 12 key tiles 30.1 -> 24.2 us per call with clusters of six for seven, 24 x 32 46.3 -> 34.1 with five for six.
+  if (MODE != kvc::kScoreKeyDiff)
+    while (Cn > 1 && (long long)Cn * g.Hkv * g.nl <= kvc::kNumSMs && clusters_in_flight(Cn) < (long long)g.Hkv * g.nl) --Cn;
   if (Cn < 1) Cn = 1;
   // Two CTAs share an SM only when there are more CTAs than SMs (then one scores while the other selects);
   // a launch that fits the GPU asks for more than half an SM's shared memory so that every CTA gets an SM

@@ -22,6 +22,8 @@ pytestmark = pytest.mark.gpu
     (12, 4, 64, 140, (140, 1100)),                    # G = 3, long block after a short cache
     (28, 4, 128, 150, (150, 784, 703)),               # pairs first, then single row tiles (the last one ragged)
     (32, 8, 64, 300, (300, 600, 641)),                # the same with d = 64; more single tiles than pairs
+    (16, 16, 64, 1400, (1400, 154, 33)),              # compress clusters of six, where seven would not all fit the GPU
+    (24, 24, 64, 1300, (1300, 60)),                   # five for six
 ])
 def test_launch_shapes(hq, hkv, d, B, chunks):
     torch.manual_seed(B + hq)
