@@ -141,6 +141,7 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
     if (warp == 8) {
       if (lane == 0) {
         tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_qobs); tma_prefetch_desc(&tm_kin);
+        if (p.stamp_early) stamp_begin(p);
         bool ok = true;
         auto load_tile = [&](int i) {                  // tile i of this CTA into K buffer i & 1
           const int b = i & 1, kt = rank + i * Cn;
@@ -242,6 +243,7 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
     float* s_part = reinterpret_cast<float*>(smem);                 // [16 warps][d] partial sums
     float* s_sum = s_part + (kCompressThreads / 32) * 128;         // [d] this CTA's sum (read by the cluster)
     float* s_mu = s_sum + 128;                                      // [d] the anchor
+    if (tid == 0 && p.stamp_early) stamp_begin(p);
     const int d = p.d, epl = 16 / elem_bytes;                       // elements per 16-byte piece: 8 (bf16) or 4 (fp32)
     const int lpr = d / epl, rpw = 32 / lpr;                        // lanes per row, rows per warp and step
     const int sub = lane / lpr, piece = lane % lpr;

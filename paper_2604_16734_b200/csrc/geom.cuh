@@ -29,6 +29,7 @@ struct Geom {
   // measurement runs only (else null): this launch's pair of time stamps, {earliest begin of work, latest end} over
   // its CTAs, in nanoseconds of the global timer
   unsigned long long* stamps;
+  int stamp_early;                 // launched in plain stream order: the begin of the work in front of the dependency wait counts
 };
 
 static constexpr int kNumSMs = 148;          // B200

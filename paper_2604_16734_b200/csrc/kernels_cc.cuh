@@ -339,6 +339,7 @@ __global__ void __launch_bounds__(kCcThreads) score_cc_kernel(const T* __restric
   // below n_c are complete (the attention kernel allows this launch after its own wait), the block's keys are read from
   // the input.  Only the exponentials need what the attention kernel leaves.
   pdl_launch_dependents();
+  if (threadIdx.x == 0 && p.stamp_early) stamp_begin(p);
   const long long in_stride = static_cast<long long>(p.Hkv) * D;
   const T* Kn = k + layer * p.kv_ls + static_cast<long long>(g) * D;
   for (int i = threadIdx.x; i < NK * CPR; i += kCcThreads) {

@@ -830,6 +830,7 @@ static int run_chunk(kvc_ctx* c, int layer0, int nl, const void* q, long long q_
       st = c->side[layer0 % kvc_ctx::kSideStreams];                                           // everything below goes to the side stream
     }
     const bool pdl = pdl_main && !async_compress;             // an event, not a kernel, precedes the side stream's launches
+    g.stamp_early = !pdl;
     // On a side stream the kernel runs beside the next layer's attention, a launch of the same shape as this
     // layer's: a cluster per kv-head that fits the SMs that launch leaves idle shares nothing with it, while a wider
     // one takes SMs from attention CTAs, which then start late and lengthen the launch everything else waits for

@@ -195,6 +195,27 @@ def test_device_time_stamps_count_every_launch(dtype):
     assert b.status() == 0
 
 
+@pytest.mark.parametrize("flags", [8, 16])
+def test_device_time_stamps_in_plain_order_cover_the_whole_kernel(flags):
+    # the query-agnostic score reads all keys twice in front of the kernel's dependency wait: inside the record in plain
+    # stream order and on the side stream, outside it where the launch overlaps the attention
+    hq, hkv, d, B, n = 8, 4, 128, 3000, 24
+    torch.manual_seed(1)
+    q, k, v = (torch.randn(B + n, h, d, device="cuda", dtype=torch.bfloat16) for h in (hq, hkv, hkv))
+    us = {}
+    for fl in (0, flags):
+        kvc = Kvc(1, hq, hkv, d, torch.bfloat16, B, n, 32, flags=fl, policy=binding.KVC_SCORE_KEYDIFF)
+        kvc.prefill_chunk(0, q[:B], k[:B], v[:B], 0)
+        kvc.profile_device(16)
+        for i in range(6):
+            kvc.prefill_chunk(0, q[B:], k[B:], v[B:], B + i * n)
+        kvc.join()
+        ms, cnt, _ = kvc.profile_device_read()
+        assert cnt["compress"] == 6 and kvc.status() == 0
+        us[fl] = 1e3 * ms["compress"] / 6
+    assert us[flags] > 1.3 * us[0], us
+
+
 # ------------------------------------------------------------------------------------------------
 # host buffers: blocks of different sizes back to back
 
