@@ -21,7 +21,7 @@ In the direct and graph modes a layer's score / select / compact is enqueued on 
 (KVC_FLAG_ASYNC_COMPRESS) and overlaps the next layer's attention, as it would in a decoder stack, where the
 next layer waits for this layer's output and not for its compacted cache; the step ends after kvc_join, when
 all of it has finished.  --sync-compress keeps everything in stream order.  Per-kernel durations are taken
-in stream order, every kernel alone on the GPU.
+in stream order, every kernel alone on the GPU, without overlap between consecutive launches.
 With N > 1 every rank runs an independent replica of the request on its own GPU: the path has no
 cross-GPU exchange, so there is no collective inside the timed region (weak scaling).
 """
@@ -346,6 +346,10 @@ class Runner:
         self.kvc_in_order = self.kvc if not flags & 16 else Kvc(
             self.L, cfg.n_q_heads, cfg.n_kv_heads, cfg.head_dim, cfg.torch_dtype, cfg.budget, cfg.chunk + proxy,
             cfg.obs_window, device=device_index, flags=flags & ~16, policy=policy)
+        # ... and a third one whose launches do not overlap their predecessors: all of a kernel's work is in its record
+        self.kvc_plain = Kvc(
+            self.L, cfg.n_q_heads, cfg.n_kv_heads, cfg.head_dim, cfg.torch_dtype, cfg.budget, cfg.chunk + proxy,
+            cfg.obs_window, device=device_index, flags=flags & ~16 | 8, policy=policy)
         # raw pointers of every (block, layer) slice, so the per-call host work is one ctypes call
         self.ptrs = {}
         for ci, (o, n, t, p) in enumerate(self.calls):
@@ -431,8 +435,7 @@ def stamps_as_timed(r: Runner):
     """Device time stamps of one step in the configuration the benchmark times (compress kernels on the library's
     side streams when the context has them; calls issued directly, not from the graph): per kernel its launches, mean
     duration, total and share.  On a side stream a compress kernel gets fewer CTAs per kv-head than in stream order
-    and runs longer, beside the next layer's attention -- this is the table the ncu launch list of the same command
-    compares with."""
+    and runs longer, beside the next layer's attention."""
     kv = r.kvc
     r.step_direct()
     torch.cuda.synchronize()
@@ -449,12 +452,29 @@ def stamps_as_timed(r: Runner):
                     share=ms[s] / tot) for s in ms if cnt[s]} | {"span_ms": span_ms}
 
 
+def stamped(r: Runner, kvc, step, steps):
+    """({kernel: milliseconds}, {kernel: launches}) of `steps` steps of a context by device time stamps."""
+    saved = (r.kvc, r.flags)
+    r.kvc, r.flags = kvc, r.flags & ~16
+    before = kvc.launch_count()
+    step()
+    torch.cuda.synchronize()
+    kvc.profile_device((kvc.launch_count() - before) * steps + 16)
+    for _ in range(steps):
+        step()
+    ms, cnt, _ = kvc.profile_device_read()
+    kvc.profile_device(0)
+    r.kvc, r.flags = saved
+    return ms, cnt
+
+
 def profile_pass(r: Runner, steps: int, batched: bool = False, events: bool = False):
     """Per-kernel durations and exact algorithmic work: one call per (block, layer), in stream order, or with
     `batched` one call per block with the layer index in the launch grid.  The durations are device-side time
-    stamps taken inside the kernels (global timer; per launch from the earliest begin of work, past the wait for
-    the preceding kernel, to the latest end over its CTAs): no event pair sits between consecutive launches, so
-    they overlap as they do in the timed step, and the sum of the durations fits inside the step."""
+    stamps taken inside the kernels (global timer; per launch from the earliest begin of work to the latest end over its
+    CTAs), from two contexts: in plain stream order, where a record holds all of a kernel's work (`us_per_launch`, from
+    which the rates follow), and with launches that overlap their predecessors as they do in the timed step, where it
+    holds what a kernel does behind the wait for its predecessor (`us_behind_wait`; their sum fits inside the step)."""
     saved = (r.kvc, r.flags)
     r.kvc, r.flags = r.kvc_in_order, r.flags & ~16
     kv, cfg = r.kvc, r.cfg
@@ -478,15 +498,6 @@ def profile_pass(r: Runner, steps: int, batched: bool = False, events: bool = Fa
                 work[s]["bytes"] += wv["bytes"]; work[s]["flops"] += wv["flops"]
         n_c = min(n_c + n - t, cfg.budget)
     torch.cuda.synchronize()
-    per_step = kv.launch_count()
-    (r.step_batched if batched else r.step_direct)()
-    torch.cuda.synchronize()
-    per_step = kv.launch_count() - per_step
-    kv.profile_device(per_step * steps + 16)
-    for _ in range(steps):
-        (r.step_batched if batched else r.step_direct)()
-    ms, cnt, span_ms = kv.profile_device_read()
-    kv.profile_device(0)
     # the same launches bracketed by CUDA events on the launching stream (a pair per launch: each kernel alone on the
     # GPU, launch latency and the events themselves included)
     ev_ms = ev_cnt = None
@@ -498,11 +509,15 @@ def profile_pass(r: Runner, steps: int, batched: bool = False, events: bool = Fa
         ev_ms, ev_cnt = kv.profile_read()
         kv.profile_enable(False)
     r.kvc, r.flags = saved
+    step = r.step_batched if batched else r.step_direct
+    ms, cnt = stamped(r, r.kvc_plain, step, steps)
+    behind_ms, behind_cnt = stamped(r, r.kvc_in_order, step, steps)
     per = {}
     for s in STEPS:
         if cnt[s]:
             per[s] = dict(ms_total_per_step=ms[s] / steps, launches_per_step=cnt[s] // steps,
-                          us_per_launch=1e3 * ms[s] / cnt[s], bytes_per_step=work[s]["bytes"],
+                          us_per_launch=1e3 * ms[s] / cnt[s], us_behind_wait=1e3 * behind_ms[s] / behind_cnt[s],
+                          ms_behind_wait_per_step=behind_ms[s] / steps, bytes_per_step=work[s]["bytes"],
                           flops_per_step=work[s]["flops"])
             if ev_cnt and ev_cnt[s]:
                 per[s]["us_per_launch_cuda_events"] = 1e3 * ev_ms[s] / ev_cnt[s]
@@ -631,17 +646,18 @@ def measure(cfg, args, L, local_rank, rank, world, dist, barrier, peaks, steps, 
         roof["us_per_launch_device_stamps"] = d["us_per_launch"]
         roof["arithmetic_intensity"] = ai
         roof["timing"] = ("achieved / frac: CUDA events around every launch on the launching stream, kernels in stream order; "
-                          "*_device_stamps: time stamps inside the kernel (global timer, earliest begin of work, past the wait "
-                          "for the preceding kernel, to the latest end over the CTAs of a launch)")
+                          "*_device_stamps: time stamps inside the kernel (global timer, earliest begin of work to the latest "
+                          "end over the CTAs of a launch), launches not overlapping their predecessors")
         # the kernels' durations against the step they have to fit into
-        kernel_ms_sum = sum(x["ms_total_per_step"] for x in per.values())
+        kernel_ms_sum = sum(x["ms_behind_wait_per_step"] for x in per.values())
         out["kernel_ms_sum"] = kernel_ms_sum
         out["overlap"] = dict(
             ms_per_step_in_order=in_order_ms, ms_per_step=ms_per_step,
             hidden_by_side_streams_ms=(in_order_ms - ms_per_step) if in_order_ms is not None else None,
             kernel_ms_sum_over_in_order=kernel_ms_sum / in_order_ms if in_order_ms else None,
-            note="kernel_ms_sum adds the device-stamped durations of all launches of an in-order step; what the in-order "
-                 "step holds beyond it is the time between launches (launch latency, cache resets)")
+            note="kernel_ms_sum adds what the launches of an in-order step do behind the wait for their predecessor, by device "
+                 "stamps; what the step holds beyond it is launch latency, cache resets and work in front of a wait that "
+                 "the predecessor does not cover")
         out["roofline_step"] = step_roofline(cfg, per, L, ms_per_step, peaks)
         if in_order_ms is not None and out["roofline_step"]:
             out["roofline_step"]["frac_in_order"] = out["roofline_step"]["bound_ms"] / in_order_ms
@@ -691,6 +707,7 @@ def measure(cfg, args, L, local_rank, rank, world, dist, barrier, peaks, steps, 
         "compress": "side stream, beside the next layer's attention" if flags & 16 else "in stream order",
         "l2": "inputs exceed L2" if (r.Q.numel() + 2 * r.K.numel()) * cfg.elem_bytes > 126e6 else "inputs fit L2"})
     r.kvc.close()
+    r.kvc_plain.close()
     if r.kvc_in_order is not r.kvc:
         r.kvc_in_order.close()
     del r
