@@ -10,7 +10,8 @@ carries enough work for the roofline targets to be assessed.  At N = 1 the same 
 with fewer steps (--no-extra skips them).
 
 One "step" is one pass of the whole hot path over one synthetic request: every block of the
-workload's prefix through every layer, starting from empty caches.  Prints ONE JSON line.
+workload's prefix through every layer, starting from empty caches.  Prints ONE JSON line, short enough to be kept
+whole where only the end of the output is; --details FILE writes everything that was measured.
 
 Modes (all run the same kernels through the C ABI):
   direct   one kvc_prefill_chunk call per (block, layer), issued from Python each step
@@ -716,6 +717,37 @@ def measure(cfg, args, L, local_rank, rank, world, dist, barrier, peaks, steps, 
 
 
 EXTRA_WORKLOADS = ("C2", "C3", "C4", "T4")
+ROOFLINE_KEYS = ("kernel", "bound", "achieved", "peak", "unit", "frac", "traffic", "peak_source", "frac_device_stamps",
+                 "us_per_launch", "us_per_launch_device_stamps")
+
+
+def short(x):
+    """Numbers of a JSON object to six digits: the line stays below the few thousand characters that are kept of it."""
+    if isinstance(x, dict):
+        return {k: short(v) for k, v in x.items()}
+    if isinstance(x, list):
+        return [short(v) for v in x]
+    return float(f"{x:.6g}") if isinstance(x, float) else x
+
+
+def result_line(args, cfg, world, m, extra):
+    """The JSON line: the metric and what explains it."""
+    line = {"metric": METRIC, "value": m["value"], "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
+            "ms_per_step": m["ms_per_step"], "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
+            "dtype": "bf16" if cfg.dtype == "bf16" else "f32", "data": "synthetic", "config": m["config"],
+            "clocks": m["clocks"], "gpu_launches": m["launches_per_step"] * args.steps,
+            "launches_per_step": m["launches_per_step"], "kv_bytes": m["kv_bytes"]}
+    for k in ("ms_per_step_in_order", "kernel_ms_sum", "e2e", "cpu_baseline", "output_check"):
+        if k in m:
+            line[k] = m[k]
+    if m.get("roofline"):
+        line["roofline"] = {k: v for k, v in m["roofline"].items() if k in ROOFLINE_KEYS}
+    if m.get("roofline_step"):
+        line["roofline_step_frac"] = m["roofline_step"]["frac"]
+    if extra:
+        line["workloads"] = {name: {k: x[k] for k in ("value", "ms_per_step", "ms_per_step_in_order") if k in x}
+                             | {"roofline_step_frac": x["roofline_step"]["frac"]} for name, x in extra.items()}
+    return json.dumps(short(line))
 
 
 def main():
@@ -740,6 +772,7 @@ def main():
     ap.add_argument("--sync-compress", action="store_true",
                     help="keep a layer's score / select / compact in stream order behind its attention instead of "
                          "on the library's side stream (KVC_FLAG_ASYNC_COMPRESS, the default of the graph / direct modes)")
+    ap.add_argument("--details", default="", help="file for everything that was measured (per-kernel tables of every workload)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--no-profile", action="store_true")
@@ -789,22 +822,10 @@ def main():
             extra[name]["unit"] = UNIT
 
     if rank == 0:
-        line = {"metric": METRIC, "value": m["value"], "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
-                "ms_per_step": m["ms_per_step"], "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-                "dtype": "bf16" if cfg.dtype == "bf16" else "f32", "data": "synthetic", "config": m["config"],
-                "clocks": m["clocks"], "gpu_launches": m["launches_per_step"] * args.steps,
-                "launches_per_step": m["launches_per_step"], "kv_bytes": m["kv_bytes"], "kernels": m["kernels"],
-                "kernels_layer_batched": m["kernels_layer_batched"]}
-        if "kernels_as_timed" in m:
-            line["kernels_as_timed"] = m["kernels_as_timed"]
-        for k in ("ms_per_step_in_order", "kernel_ms_sum", "overlap", "roofline_step", "e2e", "cpu_baseline", "output_check"):
-            if k in m:
-                line[k] = m[k]
-        if m.get("roofline"):
-            line["roofline"] = m["roofline"]
-        if extra:
-            line["workloads"] = extra
-        print(json.dumps(line))
+        if args.details:
+            with open(args.details, "w") as f:
+                json.dump(dict(m, workloads=extra), f, indent=1)
+        print(result_line(args, cfg, world, m, extra))
     if dist is not None:
         dist.destroy_process_group()
 

@@ -70,3 +70,25 @@ def test_reference_arm_prints_on_rank_zero_only():
     assert line["impl"] == "reference" and line["n_gpus"] == 2 and line["value"] > 0
     assert line["cpu_baseline"]["kind"] == "oracle" and line["e2e"]["h2d_bytes_per_step"] == 0
     assert line["config"]["workload"] == "C1" and line["unit"] == "tokens/s/layer"
+
+
+def test_the_result_line_is_short_enough_to_be_kept_whole():
+    # with every field at its longest the line stays below the 3000 characters that are kept of the end of an output
+    sys.path.insert(0, ROOT)
+    import argparse
+    import bench
+    f, i = 12345678.901234567, 123456789012
+    args = argparse.Namespace(steps=20, warmup=5, policy="keydiff", hybrid=True, proxy=32, mode="graph")
+    cfg = bench.CONFIGS["C5"]
+    step = dict(value=f, ms_per_step=f, ms_per_step_in_order=f, roofline_step={"frac": f})
+    m = dict(step, launches_per_step=i, kernel_ms_sum=f, output_check=dict(max_abs_err=f, tolerance=f, elements=i, ok=True, sample="x" * 60),
+             clocks=dict(sm_mhz=f, sm_max_mhz=f, reasons=["sw_power_cap"], samples=99, power_w_max=f),
+             config=bench.config_dict(cfg, 32, args, 8, {"compress": "x" * 50, "l2": "inputs exceed L2"}),
+             kv_bytes={k: i for k in ("logical_budget", "physical_allocated", "uncompressed", "blobs_incl_positions")},
+             e2e=dict(value=f, unit=bench.UNIT, h2d_bytes_per_step=i, d2h_bytes_per_step=i, steps=5, ms_per_step=f),
+             cpu_baseline=dict(value=f, unit=bench.UNIT, cores=16, kind="oracle", sample="x" * 70, seconds=f),
+             roofline=dict({k: f for k in bench.ROOFLINE_KEYS}, timing="x" * 300), kernels={"attention": {k: f for k in "abcdefghij"}})
+    line = bench.result_line(args, cfg, 1, m, {name: step for name in bench.EXTRA_WORKLOADS})
+    assert len(line) < 2800 and "\n" not in line
+    got = json.loads(line)
+    assert got["value"] == 12345700.0 and got["gpu_launches"] == 20 * i and got["workloads"]["T4"]["roofline_step_frac"] == 12345700.0
