@@ -1,6 +1,8 @@
 """The launch shapes of the tensor-core attention and their edges: two row tiles per CTA with an odd last one, one row tile
 with one to many key tiles, key splits over clusters of 2, 4 and 8 CTAs (some without a key tile of the first rows), group
 sizes that leave rows of a tile unused."""
+import ctypes
+
 import pytest
 import torch
 
@@ -11,29 +13,40 @@ from parity_util import compare_chunk
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("hq,hkv,d,B,chunks", [
-    (1, 1, 64, 40, (1, 40, 9)),                       # one row; one key tile, then two
-    (32, 32, 128, 140, (140, 129, 128)),              # two row tiles per kv-head, the second with 12 rows / one row
-    (28, 4, 128, 260, (260, 577)),                    # G = 7: 126 rows per tile; 577 tokens
-    (4, 1, 128, 1100, (1100, 40, 33)),                # clusters of 8
-    (8, 2, 64, 700, (700, 256, 255)),                 # clusters of 4
-    (32, 8, 128, 900, (900, 196, 197)),               # clusters of 2
-    (16, 16, 128, 130, (130, 1200)),                  # two row tiles per CTA, odd count: the last CTA has one
-    (12, 4, 64, 140, (140, 1100)),                    # G = 3, long block after a short cache
-    (28, 4, 128, 150, (150, 784, 703)),               # pairs first, then single row tiles (the last one ragged)
-    (32, 8, 64, 300, (300, 600, 641)),                # the same with d = 64; more single tiles than pairs
-    (16, 16, 64, 1400, (1400, 154, 33)),              # compress clusters of six, where seven would not all fit the GPU
-    (24, 24, 64, 1300, (1300, 60)),                   # five for six
+def launch_shape(kvc, n, n_c):
+    x = [ctypes.c_int() for _ in range(3)]
+    assert kvc._lib.kvc_attention_shape(kvc._h, n, n_c, 1, *(ctypes.byref(v) for v in x)) == 0
+    return tuple(v.value for v in x)
+
+
+@pytest.mark.parametrize("hq,hkv,d,B,chunks,shape", [
+    (1, 1, 64, 40, (1, 40, 9), (1, 1, 0)),                # one row; one key tile, then two
+    (32, 32, 128, 140, (140, 129, 128), (1, 1, 0)),       # two row tiles per kv-head, the second with 12 rows / one row
+    (28, 4, 128, 260, (260, 577), (1, 1, 0)),             # G = 7: 126 rows per tile; 577 tokens
+    (4, 1, 128, 2000, (2000, 40, 33), (1, 8, 0)),         # clusters of 8
+    (4, 2, 64, 2500, (2500, 40, 1), (1, 8, 0)),           # the same with d = 64
+    (4, 1, 128, 1100, (1100, 40, 33), (1, 4, 0)),         # clusters of 4
+    (8, 2, 64, 700, (700, 256, 255), (1, 4, 0)),
+    (32, 8, 128, 900, (900, 196, 197), (1, 2, 0)),        # clusters of 2
+    (16, 16, 128, 130, (130, 1200), (2, 1, 5)),           # two row tiles per CTA
+    (16, 16, 128, 130, (130, 1660), (2, 1, 6)),           # two row tiles per CTA, odd count: the last CTA has one
+    (12, 4, 64, 140, (140, 1100), (1, 1, 0)),             # G = 3, long block after a short cache
+    (28, 4, 128, 150, (150, 784, 703), (2, 1, 7)),        # pairs first, then single row tiles (the last one ragged)
+    (32, 8, 64, 300, (300, 600, 641), (2, 1, 7)),         # the same with d = 64; more single tiles than pairs
+    (16, 16, 64, 1400, (1400, 154, 33), (1, 4, 0)),       # compress clusters of six, where seven would not all fit the GPU
+    (24, 24, 64, 1300, (1300, 60), (1, 4, 0)),            # five for six
 ])
-def test_launch_shapes(hq, hkv, d, B, chunks):
+def test_launch_shapes(hq, hkv, d, B, chunks, shape):
     torch.manual_seed(B + hq)
     kvc = Kvc(1, hq, hkv, d, torch.bfloat16, B, max(chunks))
     orc = KVCOracle(1, hq, hkv, d, B, 32)
     pos = 0
     for n in chunks:
+        last = launch_shape(kvc, n, min(pos, B))
         q, k, v = (torch.randn(n, h, d).to(torch.bfloat16) for h in (hq, hkv, hkv))
         compare_chunk(kvc, orc, 0, q, k, v, pos)        # output within 2e-2 (or one bf16 ulp of the rounded oracle value)
         pos += n
+    assert last == shape                                # (row tiles per CTA, key split, pairs) of the last block
 
 
 @pytest.mark.parametrize("hq,hkv,d,B,chunks,window,flags", [

@@ -280,10 +280,11 @@ def test_inputs_may_be_reused_behind_a_call(dtype, policy, flags):
     for reuse in (False, True):
         kvc = Kvc(layers, hq, hkv, d, dtype, B, n, policy=policy, flags=flags)
         buf = [[torch.empty_like(t) for t in data[0]] for _ in range(layers)]
-        outs = []
+        outs, kept = [], []
         for i, qkv in enumerate(data):
             layer = i % layers
             ins = buf[layer] if reuse else [t.clone() for t in qkv]
+            kept.append(ins)                    # (the allocator must not hand a clone's memory on before the side stream is done)
             if reuse:
                 for b, t in zip(ins, qkv):
                     b.copy_(t)
