@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
       }
       const uint32_t tO0 = tmem + 256 + lane_addr + t * H, tO1 = tO0 + 128;    // this group's columns of both chains' O
       const bool both = n_it1 > 0;                             // (one key tile: chain 1 has no O)
-      if (S == 1) {
+      if (R == 2 || S == 1) {                                  // (a key split always has one row tile per CTA)
         if (ok) {
           const float inv = 1.f / L, a0 = w0 * inv, a1 = w1 * inv;
 #pragma unroll
@@ -571,7 +571,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
             tma_store_wait_read();
           }
         }
-      } else {
+      } else if constexpr (R == 1) {
         // Combine the partials of the cluster (S is a power of two; rank s owns rows [s*rows_per, (s+1)*rows_per)).
         // A thread has its row's merged columns in registers.  The owner's threads keep them (up to S = 4; clusters of two
         // 15.6 -> 15.0 us, 16.6 -> 15.9; with eight 12.5 -> 13.0, hence not there); the others write theirs into
