@@ -26,8 +26,9 @@
 
 namespace kvc {
 
-// 512 threads and at most ~108 KB of shared memory per CTA: two CTAs share an SM, so that one scores
-// (TMA / tensor-core bound) while the other selects (barrier bound) when many kv-heads are in flight.
+// 512 threads and, with up to 128 observer rows, at most 97 KB of shared memory per CTA: two CTAs share an SM, so that one
+// scores (TMA / tensor-core bound) while the other selects (barrier bound) when many kv-heads are in flight.  With more
+// rows a CTA asks for up to 129 KB and is alone on its SM.
 static constexpr int kCompressThreads = 512;
 static constexpr int kDigitBits = 11;
 static constexpr int kSelBins = 1 << kDigitBits;

@@ -63,7 +63,9 @@ __global__ void __launch_bounds__(kCcThreads, 1) attn_cc_kernel(const T* __restr
   using L = AttnCc<D, BM>;
   constexpr int KT = L::KT, KS = L::KS, PS = L::PS, RT = BM / 4, JT = KT / 8, CT = D / 32;
   constexpr int EPC = 16 / (int)sizeof(T), CPR = D / EPC;  // elements per 16-byte piece, pieces per row
-  constexpr int kUnrollS = D == 128 ? 8 : 4, kUnrollV = D == 128 ? 4 : 2;   // (d = 128: 3 % faster than 4 and 2; d = 64: slower)
+  constexpr int kUnrollS = D == 128 ? 8 : 4, kUnrollV = D == 128 ? 4 : 2;
+  // (d = 128: 3 % faster than 4 and 2, although 32 rows per CTA then take all 255 registers and spill 8 bytes, bf16 inputs
+  // 44; d = 64: slower)
   extern __shared__ __align__(16) float smem_f[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rg = lane >> 3, kg = lane & 7;
   float* sQ = smem_f;                                       // [BM][KS]; at the end this CTA's merged rows

@@ -94,8 +94,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
 
   // Without a key split the row tiles that see the most keys, the last ones, start first, and the kv-heads take turns: in
   // a launch of several waves the short CTAs then fill the end (2048 tokens in one pass, 28 / 4 heads, 4 layers with five
-  // short blocks behind it: 316 -> 241 us), and in one wave the longest CTAs are not the last to get an SM (long video
-  // with compress on a side stream: 1121 -> 1060 us per request).
+  // short blocks behind it: 316 -> 241 us), and in one wave the longest CTAs are not the last to get an SM (requests: tiled
+  // image 2735 -> 2661 us, hybrid long video 3144 -> 3108, long video no difference).
   const int lin = blockIdx.y * gridDim.x + blockIdx.x;
   const bool ordered = S == 1;
   const int layer = blockIdx.z, g = ordered ? lin % gridDim.y : blockIdx.y;
@@ -539,8 +539,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
 #pragma unroll
             for (int i = 0; i < 16; ++i) pk[i] = pack_bf16x2(f[2 * i], f[2 * i + 1]);
             if constexpr (R == 1) {
-              // Straight from the registers, a sector per store: no barrier, no wait for a copy to leave (32 CTAs of three
-              // key tiles 7.2 -> 6.7 us, 128 CTAs of thirteen 17.2 -> 16.9; with 16-byte stores 6.8 and 17.7).
+              // Straight from the registers, a sector per store: no barrier, no wait for a copy to leave (requests: image
+              // 2897 -> 2842 us, image from a graph 1552 -> 1514, tiled image 2831 -> 2736).
               if (row_valid) {
                 __nv_bfloat16* dst = out + layer * p.out_ls + (static_cast<long long>(tok) * p.Hq + head_row + hh) * D + t * H + c * 32;
                 if ((reinterpret_cast<uintptr_t>(dst) & 31) == 0) {
