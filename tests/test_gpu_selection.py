@@ -3,7 +3,7 @@ import pytest
 import torch
 
 from oracle.kvc_oracle import KVCOracle
-from paper_2604_16734_b200.binding import Kvc
+from paper_2604_16734_b200.binding import KVC_SCORE_KEYDIFF, Kvc
 from parity_util import compare_chunk
 
 pytestmark = pytest.mark.gpu
@@ -69,3 +69,26 @@ def test_equal_keys_at_the_cutoff(dtype):
     rows = {tuple(x[0].tolist()) for v in vs for x in v.cpu()}
     assert all(tuple(x) in rows for x in V[0, :B].cpu().tolist())
     assert len({tuple(x) for x in V[0, :B].cpu().tolist()}) == B
+
+
+@pytest.mark.parametrize("hq,hkv,d,dtype,n,B", [
+    (16, 4, 64, torch.bfloat16, 333, 1500),             # the compress kernel runs beside the attention
+    (4, 4, 128, torch.bfloat16, 65, 90),                # candidates ranked directly
+    (2, 1, 64, torch.bfloat16, 2300, 7000),             # keys re-read from the workspace, move lists in global memory
+    (4, 1, 64, torch.float32, 64, 128),
+])
+def test_query_agnostic_selection_ahead_of_the_attention(hq, hkv, d, dtype, n, B):
+    # calls enqueued back to back, so that a selection runs while its block's attention does, against plain stream order
+    # (flag 8), bit for bit: everything that is compared is copied or selected, and the sums are taken in the same order
+    layers, blocks = 2, B // n + 4
+    torch.manual_seed(n)
+    qkv = [[torch.randn(blocks * n, h, d, device="cuda").to(dtype) for h in (hq, hkv, hkv)] for _ in range(layers)]
+    held = []
+    for flags in (0, 8):
+        kvc = Kvc(layers, hq, hkv, d, dtype, B, n, 32, flags=flags, policy=KVC_SCORE_KEYDIFF)
+        for p in range(0, blocks * n, n):
+            for l in range(layers):
+                kvc.prefill_chunk(l, *(x[p:p + n] for x in qkv[l]), p)
+        assert kvc.status() == 0
+        held.append([t[:, :B].clone() for l in range(layers) for t in kvc.cache_view(l)[:3]])
+    assert all(torch.equal(a, b) for a, b in zip(*held))
