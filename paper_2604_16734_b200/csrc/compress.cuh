@@ -576,8 +576,8 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
   const int total_holes = sh.s_remaining;
   if (rank == 0 && tid == 0) mcount[g] = total_holes;
   // The query-agnostic score, selection and listing need nothing of the attention kernel and are done in front of the wait;
-  // the moves write rows that it reads.  (Behind the wait, 4 kv-heads x 1833 candidates, d = 64: 6.4 -> 1.6 us, 16.9 -> 13.8
-  // us per call with the attention beside it.)
+  // the moves write rows that it reads.  (Behind the wait, 4 kv-heads x 1833 candidates, d = 64: 6.4 -> 1.7 us; requests
+  // 1584 -> 1281 us, 16.5 -> 13.3 per call with the attention beside it.)
   if constexpr (MODE == kScoreKeyDiff) {
     pdl_wait();
     if (tid == 0) stamp_begin(p);
