@@ -64,9 +64,10 @@ typedef enum {
                                   the call's q must stay unchanged, and the layer's cache must not be read by the
                                   caller, until the next kvc call on that layer, kvc_reset of it, kvc_status or
                                   kvc_join has been enqueued on the stream that does so; every kvc call orders
-                                  itself after the pending work of the layers it touches.  Inside a stream
-                                  capture, call kvc_join before ending the capture.  All calls of one context must
-                                  come from one host thread. */
+                                  itself after the pending work of the layers it touches and of the workspace
+                                  slots it uses (kvc_prefill_chunk_layers and _host use the first ones).  Before
+                                  another context uses the same workspace, and before a stream capture begins or
+                                  ends, call kvc_join.  All calls of one context must come from one host thread. */
 
 typedef struct {
   int n_layers;        /* L >= 1                                                                 */

@@ -215,13 +215,14 @@ struct ProfScope {
   ~ProfScope() { if (on) cudaEventRecord(b, st); }
 };
 
-// Makes `st` wait for the compress kernels of layers [l0, l1) that still run on the side stream.
-static int wait_pending(kvc_ctx* c, int l0, int l1, cudaStream_t st) {
+// Makes `st` wait for the compress kernels of layers [l0, l1) that still run on the side stream.  `keep`: they stay pending
+// (a later call or kvc_join, perhaps on another stream, waits for them too).
+static int wait_pending(kvc_ctx* c, int l0, int l1, cudaStream_t st, bool keep = false) {
   for (int l = l0; l < l1; ++l) {
     if (!c->pending[l]) continue;
     cudaError_t e = cudaStreamWaitEvent(st, c->ev_comp[l], 0);
     if (e != cudaSuccess) return fail(c, KVC_ECUDA, "cudaStreamWaitEvent: %s", cudaGetErrorString(e));
-    c->pending[l] = 0;
+    if (!keep) c->pending[l] = 0;
   }
   return KVC_OK;
 }
@@ -793,6 +794,10 @@ static int run_chunk(kvc_ctx* c, int layer0, int nl, const void* q, long long q_
   const bool pdl = pdl_main;
   cudaError_t e = cudaSuccess;
   if (int rc = wait_pending(c, layer0, layer0 + nl, st)) return rc;    // a compress kernel of an earlier block may still run
+  // ... and one of another layer in a workspace slot of this call: a single-layer call with compress on the side stream works
+  // in its layer's slot, a batched call and kvc_prefill_chunk_host in the first ones (the built-in scratch is not shared so)
+  if (!clear_status)
+    if (int rc = wait_pending(c, g.slot0, g.slot0 + nl, st, true)) return rc;
   // every host check has passed: from here on work is enqueued.  A workspace that keeps an earlier user's contents
   // (the built-in scratch array) gets its status word cleared first.
   if (clear_status)

@@ -1,13 +1,15 @@
 """GPU tests of the corners around the hot path: the query-agnostic score on degenerate keys (Sec. 3.2: keys
 parallel to the anchor, identical keys, a zero key), the bounded device-side wait running out, and the guard
 regions that the parity helper keeps around every buffer."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
 
 from oracle.kvc_oracle import KVCOracle
 from paper_2604_16734_b200 import binding
-from paper_2604_16734_b200.binding import Kvc, KVC_ETIMEOUT
+from paper_2604_16734_b200.binding import Kvc, KVC_ETIMEOUT, KVC_FLAG_ASYNC_COMPRESS
 
 from parity_util import check_guards, compare_chunk, guarded_copy, install_guards
 
@@ -300,3 +302,71 @@ def test_inputs_may_be_reused_behind_a_call(dtype, policy, flags):
         res.append((outs, [kvc.cache_view(l)[2][:, :B].clone() for l in range(layers)]))
     assert all(torch.equal(a, b) for a, b in zip(res[0][0], res[1][0]))
     assert all(torch.equal(a, b) for a, b in zip(res[0][1], res[1][1]))
+
+
+# ------------------------------------------------------------------------------------------------
+# workspace slots while a compress kernel is pending on a side stream
+
+def _longest_chain(graph):
+    """Nodes on the longest path of a captured graph."""
+    rt, handle, n = ctypes.CDLL("libcudart.so.12"), ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t()
+    assert rt.cudaGraphGetEdges(handle, None, None, ctypes.byref(n)) == 0
+    src, dst = (ctypes.c_void_p * n.value)(), (ctypes.c_void_p * n.value)()
+    assert rt.cudaGraphGetEdges(handle, src, dst, ctypes.byref(n)) == 0
+    after = {}
+    for a, b in zip(src, dst):
+        after.setdefault(a, []).append(b)
+
+    def depth(node):
+        return 1 + max((depth(x) for x in after.get(node, ())), default=0)
+
+    return max(depth(node) for node in after)
+
+
+@pytest.mark.parametrize("single,batched,chain", [(0, 2, 4), (1, 2, 4), (3, 0, 3)])
+def test_a_batched_call_waits_for_the_workspace_slots_it_uses(single, batched, chain):
+    # a batched call works in the first slots: behind the compress kernel of a layer that has one of them as its own, beside
+    # that of any other.  The calls are captured and never run: attention, compress, attention, compress in one chain or two
+    n, B = 64, 128
+    kvc = Kvc(4, 4, 2, 64, torch.bfloat16, B, n, flags=KVC_FLAG_ASYNC_COMPRESS | 8)      # 8: plain edges
+    q, k, v = (torch.randn(2, n, h, 64, device="cuda", dtype=torch.bfloat16) for h in (4, 2, 2))
+    out = torch.empty_like(q)
+    for p in (0, n, 2 * n):                                       # every layer evicts from here on; kernels are loaded
+        for l in range(4):
+            kvc.prefill_chunk(l, q[0], k[0], v[0], p)
+    kvc.prefill_chunk_layers(0, q, k, v, 3 * n, out)
+    kvc.prefill_chunk_layers(2, q, k, v, 3 * n, out)
+    assert kvc.status() == 0
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        kvc.prefill_chunk(single, q[0], k[0], v[0], 4 * n, out[0])
+        kvc.prefill_chunk_layers(batched, q, k, v, 4 * n, out)
+        kvc.join()
+    assert _longest_chain(graph) == chain
+
+
+def test_batched_and_host_calls_beside_a_pending_compress():
+    # the same calls on a context without the flag give the same bits
+    layers, hq, hkv, d, B, n = 4, 8, 8, 64, 3000, 200
+    N = B + 6 * n
+    torch.manual_seed(11)
+    Q, K, V = (torch.randn(layers, N, h, d, device="cuda", dtype=torch.bfloat16) for h in (hq, hkv, hkv))
+    host = [x[1].cpu().pin_memory() for x in (Q, K, V)]
+    held = []
+    for flags in (0, KVC_FLAG_ASYNC_COMPRESS):
+        kvc = Kvc(layers, hq, hkv, d, torch.bfloat16, B, n, flags=flags)
+        out, out_host = torch.zeros_like(Q), torch.zeros_like(host[0]).pin_memory()
+        for l in range(layers):                                   # the cache is full, nothing evicted yet
+            kvc.prefill_chunk(l, Q[l, :B], K[l, :B], V[l, :B], 0, out[l, :B])
+        for i, p in enumerate(range(B, N, n)):
+            s = slice(p, p + n)
+            kvc.prefill_chunk(0, Q[0, s], K[0, s], V[0, s], p, out[0, s])
+            if i % 2:
+                kvc.prefill_chunk_host(1, *(x[s] for x in host), p, out_host[s])
+            kvc.prefill_chunk_layers(2, Q[2:, s], K[2:, s], V[2:, s], p, out[2:, s])
+            if i % 2 == 0:
+                kvc.prefill_chunk_host(1, *(x[s] for x in host), p, out_host[s])
+        kvc.host_flush()
+        assert kvc.status() == 0
+        held.append([out, out_host] + [t[:, :B] for l in range(layers) for t in kvc.cache_view(l)[:3]])
+    assert all(torch.equal(a, b) for a, b in zip(*held))
