@@ -19,8 +19,9 @@
  *   a2  score    if tot > B: importance of every cached key = attention probability it receives
  *                from the observer queries (the block's last w rows), summed over those rows and
  *                over the G query heads sharing the kv-head                   (Eq. 4)
- *   a3  select   evict the tot - B lowest-scoring entries; ties keep the older entry; the
- *                observers' own w keys are never evicted                      (Alg. 1, Evict)
+ *   a3  select   evict the tot - B lowest-scoring entries; ties keep the older entry (which one, if
+ *                a caller repeats positions, is unspecified); the observers' own w keys are never
+ *                evicted                                                      (Alg. 1, Evict)
  *   a4  compact  retained entries are moved into rows [0, B); length becomes B (Sec. 3.1)
  */
 #ifndef KVC_H_

@@ -71,6 +71,38 @@ def test_equal_keys_at_the_cutoff(dtype):
     assert len({tuple(x) for x in V[0, :B].cpu().tolist()}) == B
 
 
+@pytest.mark.parametrize("dtype,d,n,B", [
+    (torch.float32, 64, 16, 21),                        # ranked directly, one of two equal keys stays
+    (torch.float32, 64, 100, 150),                      # the keys of the cut-off bin ranked; equal keys end at the cut-off
+    (torch.bfloat16, 128, 100, 151),                    # ... or lie across it
+    (torch.float32, 128, 200, 300),                     # decided bit by bit
+    (torch.bfloat16, 64, 200, 301),
+    (torch.bfloat16, 64, 3200, 5001),                   # keys re-read from the workspace, move lists in global memory
+])
+def test_equal_keys_across_the_cutoff(dtype, d, n, B):
+    # two blocks with the same positions behind one far ahead of them, all scores equal: exactly B - w candidates stay, the
+    # oldest first, and the last block's window with them
+    w, starts = 4, (1 << 20, 0, 0)
+    torch.manual_seed(n)
+    k = torch.randn(1, 1, d, device="cuda").expand(n, 1, d).to(dtype).contiguous()
+    q = torch.randn(1, 1, d, device="cuda").expand(n, 1, d).to(dtype).contiguous()
+    vs = [torch.randn(n, 1, d, device="cuda").to(dtype) for _ in starts]
+    kvc = Kvc(1, 1, 1, d, dtype, B, n, w)
+    held = []
+    for p, v in zip(starts, vs):
+        kvc.prefill_chunk(0, q, k, v, p)
+        cand, new = held + list(range(p, p + n - w)), list(range(p + n - w, p + n))
+        held = (sorted(cand)[:B - w] if len(cand) + w > B else cand) + new
+    assert kvc.status() == 0
+    _, V, pos, length = kvc.cache_view(0)
+    pos = pos[0, :B].cpu().tolist()
+    assert length == B and sorted(pos) == sorted(held)
+    where = {tuple(row): (b, p + i) for b, (p, v) in enumerate(zip(starts, vs)) for i, row in enumerate(v[:, 0].cpu().tolist())}
+    rows = [where[tuple(row)] for row in V[0, :B].cpu().tolist()]
+    assert [p for _, p in rows] == pos and len(set(rows)) == B
+    assert all((2, n - w + i) in rows for i in range(w))
+
+
 @pytest.mark.parametrize("hq,hkv,d,dtype,n,B", [
     (16, 4, 64, torch.bfloat16, 333, 1500),             # the compress kernel runs beside the attention
     (4, 4, 128, torch.bfloat16, 65, 90),                # candidates ranked directly
