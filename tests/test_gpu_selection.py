@@ -5,6 +5,7 @@ import torch
 from oracle.kvc_oracle import KVCOracle
 from paper_2604_16734_b200.binding import KVC_SCORE_KEYDIFF, Kvc
 from parity_util import compare_chunk
+from test_gpu_attention_shapes import launch_shape
 
 pytestmark = pytest.mark.gpu
 
@@ -103,24 +104,53 @@ def test_equal_keys_across_the_cutoff(dtype, d, n, B):
     assert all((2, n - w + i) in rows for i in range(w))
 
 
-@pytest.mark.parametrize("hq,hkv,d,dtype,n,B", [
-    (16, 4, 64, torch.bfloat16, 333, 1500),             # the compress kernel runs beside the attention
-    (4, 4, 128, torch.bfloat16, 65, 90),                # candidates ranked directly
-    (2, 1, 64, torch.bfloat16, 2300, 7000),             # keys re-read from the workspace, move lists in global memory
-    (4, 1, 64, torch.float32, 64, 128),
+@pytest.mark.parametrize("hq,hkv,d,dtype,n,B,form", [
+    (16, 4, 64, torch.bfloat16, 333, 1500, "beside"),   # the compress kernel runs beside the attention
+    (4, 4, 128, torch.bfloat16, 65, 90, "ranked"),      # candidates ranked directly
+    (2, 1, 64, torch.bfloat16, 2300, 7000, "global"),   # keys re-read from the workspace, move lists in global memory
+    (4, 1, 64, torch.float32, 64, 128, "cuda cores"),
 ])
-def test_query_agnostic_selection_ahead_of_the_attention(hq, hkv, d, dtype, n, B):
+def test_query_agnostic_selection_ahead_of_the_attention(hq, hkv, d, dtype, n, B, form):
     # calls enqueued back to back, so that a selection runs while its block's attention does, against plain stream order
-    # (flag 8), bit for bit: everything that is compared is copied or selected, and the sums are taken in the same order
-    layers, blocks = 2, B // n + 4
+    # (flag 8), bit for bit: everything that is compared is copied or selected, and the sums are taken in the same order.
+    # The outputs would show a move that overwrites a row the attention still reads.
+    layers, blocks, w = 2, B // n + 4, 32
+    n_cand = B + n - w
     torch.manual_seed(n)
     qkv = [[torch.randn(blocks * n, h, d, device="cuda").to(dtype) for h in (hq, hkv, hkv)] for _ in range(layers)]
     held = []
-    for flags in (0, 8):
-        kvc = Kvc(layers, hq, hkv, d, dtype, B, n, 32, flags=flags, policy=KVC_SCORE_KEYDIFF)
-        for p in range(0, blocks * n, n):
-            for l in range(layers):
-                kvc.prefill_chunk(l, *(x[p:p + n] for x in qkv[l]), p)
+    for flags in (8, 0, 0, 0, 0):
+        kvc = Kvc(layers, hq, hkv, d, dtype, B, n, w, flags=flags, policy=KVC_SCORE_KEYDIFF)
+        if form == "beside":                             # (the rule: all CTAs of both kernels fit the GPU)
+            row_tiles, split, pairs = launch_shape(kvc, n, B)
+            tiles = -(-n // (128 // (hq // hkv)))
+            assert hkv * (tiles * split if row_tiles == 1 else tiles - pairs) + hkv * min(16, 148 // hkv, -(-n_cand // 256)) <= 148
+        assert (n_cand <= 128) == (form == "ranked") and (n_cand > 6144 and n > 2048) == (form == "global")
+        outs = [kvc.prefill_chunk(l, *(x[p:p + n] for x in qkv[l]), p) for p in range(0, blocks * n, n) for l in range(layers)]
         assert kvc.status() == 0
-        held.append([t[:, :B].clone() for l in range(layers) for t in kvc.cache_view(l)[:3]])
-    assert all(torch.equal(a, b) for a, b in zip(*held))
+        held.append(outs + [t[:, :B].clone() for l in range(layers) for t in kvc.cache_view(l)[:3]])
+    for got in held[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(held[0], got))
+
+
+@pytest.mark.parametrize("dtype,d,n,B", [(torch.bfloat16, 64, 30, 50), (torch.float32, 128, 30, 50), (torch.bfloat16, 128, 300, 500),
+                                         (torch.float32, 64, 300, 500)])
+def test_query_agnostic_ties_between_cached_and_new_entries(dtype, d, n, B):
+    # all keys equal, so age alone decides, and the last block's positions lie between those of the blocks before it: the
+    # cut-off falls inside it, with cached entries (positions read from the cache) and new ones (computed) on either side
+    hq = hkv = 2
+    w, starts = 4, (1000, 2000, 1500)
+    torch.manual_seed(d)
+    k = torch.randn(1, hkv, d, device="cuda").expand(n, hkv, d).to(dtype).contiguous()
+    kvc = Kvc(1, hq, hkv, d, dtype, B, n, w, policy=KVC_SCORE_KEYDIFF)
+    held = []
+    for p in starts:
+        q, v = (torch.randn(n, h, d, device="cuda").to(dtype) for h in (hq, hkv))
+        kvc.prefill_chunk(0, q, k, v, p)
+        cand, new = held + list(range(p, p + n - w)), list(range(p + n - w, p + n))
+        kept = sorted(cand)[:B - w] if len(cand) + w > B else cand
+        dropped, held = set(cand) - set(kept), kept + new
+    assert {x // 500 for x in kept} == {2, 3} and {x // 500 for x in dropped} == {3, 4}
+    assert kvc.status() == 0
+    _, _, pos, length = kvc.cache_view(0)
+    assert length == B and all(sorted(row) == sorted(held) for row in pos[:, :B].cpu().tolist())

@@ -133,6 +133,8 @@ def test_loads_in_front_of_the_dependency_wait_bypass_l1():
     stage = re.search(r"void stage16\(.*?\n}", open(os.path.join(csrc, "kernels_cc.cuh")).read(), re.S).group()
     for body in (fetch, stage):
         assert "__ldcg(reinterpret_cast<const uint4*>" in body and "*reinterpret_cast<const uint4*>" not in body
+    pos_of = re.search(r"auto pos_of = .*?\n  };", open(os.path.join(csrc, "compress.cuh")).read(), re.S).group()
+    assert re.search(r"kScoreKeyDiff\) return j < p.n_sc \? __ldcg\(pos \+ j\)", pos_of)
 
 
 def test_kernels_hold_their_tensor_memory_before_a_dependent_may_start():
