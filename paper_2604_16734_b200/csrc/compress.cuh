@@ -361,7 +361,6 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
       const float den = sqrtf(nm) * mu_norm;
       if (piece < kRowsInFlight && i0 + piece < n_steps && r < p.n_cand) score[r] = den > 0.f ? fmaxf(0.f, 1.f - dt / den) : 1.f;
     }
-    __syncthreads();
   } else {
     if (tid == 0) { pdl_wait(); stamp_begin(p); }
     __syncthreads();
