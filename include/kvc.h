@@ -274,10 +274,12 @@ int kvc_profile_read(kvc_ctx* ctx, double* ms, long long* launches);
  * calls stamps the nanosecond global timer when a CTA begins its work and when it ends, and the launch's record keeps
  * the earliest begin and the latest end; launches beyond `capacity` are not recorded.  Where a launch may overlap its
  * predecessor, the begin is past the wait for it: what the score and compress kernels load and multiply in front of that
- * wait is outside the record.  In plain stream order (KVC_FLAG_NO_PDL) and on the side stream of
- * KVC_FLAG_ASYNC_COMPRESS all of a kernel's work is inside.  records = NULL switches it off.  kvc_profile_device_read takes a HOST copy of the records (made by
- * the caller after synchronising) and ADDS, per kernel index as in kvc_profile_read, the durations in milliseconds
- * and the launch counts; *span_ms (may be NULL) receives the time from the first begin to the last end. */
+ * wait is outside the record, and with the query-agnostic policy score, selection and move lists are too, so that such a
+ * record holds the moves alone.  In plain stream order (KVC_FLAG_NO_PDL) and on the side stream of
+ * KVC_FLAG_ASYNC_COMPRESS all of a kernel's work is inside.  records = NULL switches it off.  kvc_profile_device_read
+ * takes a HOST copy of the records (made by the caller after synchronising) and ADDS, per kernel index as in
+ * kvc_profile_read, the durations in milliseconds and the launch counts; *span_ms (may be NULL) receives the time from
+ * the first begin to the last end. */
 int kvc_profile_device(kvc_ctx* ctx, void* records, long long capacity, void* stream);
 int kvc_profile_device_read(kvc_ctx* ctx, const void* records_host, double* ms, long long* launches, double* span_ms);
 

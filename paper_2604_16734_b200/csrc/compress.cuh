@@ -113,9 +113,11 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
   // its work: the call's inputs and the cache rows below n_c = n_sc (on a side stream, where the caller may reuse k by now,
   // n_sc covers all rows and there is nothing to wait for).  The attention kernel allows this launch only after its own
   // wait, so everything that precedes it in the stream has finished and is in L2; these reads go there (TMA, ld.global.cg)
-  // and never through L1, which is only known to be current behind this kernel's own wait.  (Loads, products and, for the
-  // query-agnostic score, the whole phase then overlap the attention's end: 32 kv-heads x 288 candidates 7.0 -> 6.4 us
-  // behind the wait, 4 x 2300 x 224 observer rows 11.6 -> 10.6, 4 x 1833 query-agnostic 10.3 -> 5.8.)
+  // and never through L1, which is only known to be current behind this kernel's own wait.  What it writes before the wait
+  // are the scores, move lists and counts of its workspace slot: the attention touches none of them, and the kernels that
+  // used the slot before had finished when the attention was past its own wait.  Cache rows are written behind the wait only.
+  // (Loads and products then overlap the attention's end: 32 kv-heads x 288 candidates 7.0 -> 6.4 us behind the wait,
+  // 4 x 2300 x 224 observer rows 11.6 -> 10.6.  The query-agnostic policy has all but the moves there, see below.)
 
   // ------------------------------------------------------------------------------------ phase 1: scores
   if constexpr (MODE == kScoreAttention) {
@@ -609,8 +611,8 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
   const int total_holes = sh.s_remaining;
   if (rank == 0 && tid == 0) mcount[g] = total_holes;
   // The query-agnostic score, selection and listing need nothing of the attention kernel and are done in front of the wait;
-  // the moves write rows that it reads.  (Behind the wait, 4 kv-heads x 1833 candidates, d = 64: 6.4 -> 1.7 us; requests
-  // 1584 -> 1281 us, 16.5 -> 13.3 per call with the attention beside it.)
+  // the moves write rows that it reads.  (Behind the wait, mean of the 72 evicting calls of a request with up to 4 kv-heads x
+  // 1801 candidates, d = 64: 6.4 us with the score alone in front of it, 1.6 with all three; the request 1577 -> 1278 us.)
   if constexpr (MODE == kScoreKeyDiff) {
     pdl_wait();
     if (tid == 0) stamp_begin(p);

@@ -810,9 +810,12 @@ static int run_chunk(kvc_ctx* c, int layer0, int nl, const void* q, long long q_
   if (c->use_tc) {
     const AttnShape sh = attn_launch_shape(g, !(cf.flags & 4u), evict);
     attn_ctas = sh.ctas;
-    // The query-agnostic score needs nothing of the attention: its kernel starts at once if it fits beside it (4 kv-heads,
-    // 88 + 32 CTAs: 1519 us per request against 1594; 112 + 72 CTAs: 2909 against 2888).  The query-aware one has only
-    // loads and products to do early, for which the end of the key loop is soon enough.
+    // The query-agnostic kernel needs nothing of the attention up to its moves: it starts at once if it fits beside it.  Us
+    // per request, started at once / at the end of the key loop (CTAs of attention + compress): 88 + 32 1281 / 1672, 32 + 64
+    // 2381 / 2962, 112 + 20 2112 / 2641, 72 + 16 677 / 892.  Without room it costs beside an attention that is short or splits its
+    // keys (112 + 40 3258 / 3191, 112 + 72 4855 / 4787, 88 + 64 2388 / 2379, 64 + 128 1346 / 1338); beside a long one that does
+    // not it would gain (128 + 28 1124 / 1171 with the blocks that fit started at once, 128 + 128 2718 / 2812, 132 + 44 1367 /
+    // 1577).  The query-aware kernel has only loads and products to do early, for which the end of the key loop is soon enough.
     const long long heads = (long long)g.Hkv * g.nl;
     const long long cluster = std::min<long long>({kvc::kMaxClusterWide, kvc::kNumSMs / heads, (g.n_cand + 255) / 256});
     g.early = evict && !async_compress && cf.policy == KVC_SCORE_KEYDIFF && cluster > 0 && attn_ctas + heads * cluster <= kvc::kNumSMs;
