@@ -215,14 +215,36 @@ struct ProfScope {
   ~ProfScope() { if (on) cudaEventRecord(b, st); }
 };
 
-// Makes `st` wait for the compress kernels of layers [l0, l1) that still run on the side stream.  `keep`: they stay pending
-// (a later call or kvc_join, perhaps on another stream, waits for them too).
-static int wait_pending(kvc_ctx* c, int l0, int l1, cudaStream_t st, bool keep = false) {
+// Makes `st` wait for the compress kernels of layers [l0, l1) that still run on the side stream.
+static int wait_pending(kvc_ctx* c, int l0, int l1, cudaStream_t st) {
   for (int l = l0; l < l1; ++l) {
     if (!c->pending[l]) continue;
     cudaError_t e = cudaStreamWaitEvent(st, c->ev_comp[l], 0);
     if (e != cudaSuccess) return fail(c, KVC_ECUDA, "cudaStreamWaitEvent: %s", cudaGetErrorString(e));
-    if (!keep) c->pending[l] = 0;
+    c->pending[l] = 0;
+  }
+  return KVC_OK;
+}
+
+// Makes `st` wait for the compress kernels that still use workspace slots [s0, s1) (slot l: layer l's).  They stay pending: a
+// later call or kvc_join, perhaps on another stream, waits for them too.  One left over from before a capture of `st` began
+// cannot be waited for inside it: the host does.
+static int wait_slots(kvc_ctx* c, int s0, int s1, cudaStream_t st) {
+  for (int l = s0; l < s1; ++l) {
+    if (!c->pending[l]) continue;
+    cudaStreamCaptureStatus here = cudaStreamCaptureStatusNone, there = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(st, &here);
+    if (e == cudaSuccess) e = cudaStreamIsCapturing(c->side[l % kvc_ctx::kSideStreams], &there);
+    if (e == cudaSuccess && here != cudaStreamCaptureStatusNone && there == cudaStreamCaptureStatusNone) {
+      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+      (void)cudaThreadExchangeStreamCaptureMode(&mode);
+      e = cudaEventSynchronize(c->ev_comp[l]);
+      (void)cudaThreadExchangeStreamCaptureMode(&mode);
+      if (e == cudaSuccess) c->pending[l] = 0;
+    } else if (e == cudaSuccess) {
+      e = cudaStreamWaitEvent(st, c->ev_comp[l], 0);
+    }
+    if (e != cudaSuccess) return fail(c, KVC_ECUDA, "wait for workspace slot %d: %s", l, cudaGetErrorString(e));
   }
   return KVC_OK;
 }
@@ -797,7 +819,7 @@ static int run_chunk(kvc_ctx* c, int layer0, int nl, const void* q, long long q_
   // ... and one of another layer in a workspace slot of this call: a single-layer call with compress on the side stream works
   // in its layer's slot, a batched call and kvc_prefill_chunk_host in the first ones (the built-in scratch is not shared so)
   if (!clear_status)
-    if (int rc = wait_pending(c, g.slot0, g.slot0 + nl, st, true)) return rc;
+    if (int rc = wait_slots(c, g.slot0, g.slot0 + nl, st)) return rc;
   // every host check has passed: from here on work is enqueued.  A workspace that keeps an earlier user's contents
   // (the built-in scratch array) gets its status word cleared first.
   if (clear_status)

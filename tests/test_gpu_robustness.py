@@ -345,6 +345,33 @@ def test_a_batched_call_waits_for_the_workspace_slots_it_uses(single, batched, c
     assert _longest_chain(graph) == chain
 
 
+def test_a_compress_left_pending_before_a_capture():
+    # a captured batched call cannot wait for work from outside the capture: the host has waited for it when the call returns
+    n, B = 64, 128
+    a, b = (Kvc(4, 4, 2, 64, torch.bfloat16, B, n, flags=KVC_FLAG_ASYNC_COMPRESS) for _ in range(2))
+    torch.manual_seed(3)
+    q, k, v = (torch.randn(2, n, h, 64, device="cuda", dtype=torch.bfloat16) for h in (4, 2, 2))
+    out = [torch.empty_like(q) for _ in range(2)]
+    for kvc, o in ((a, out[0]), (b, out[1])):
+        for p in (0, n, 2 * n):
+            for l in range(4):
+                kvc.prefill_chunk(l, q[0], k[0], v[0], p)
+        kvc.join()
+        kvc.prefill_chunk(0, q[0], k[0], v[0], 3 * n)                # left pending
+        if kvc is a:
+            kvc.prefill_chunk_layers(2, q, k, v, 3 * n, o)
+            continue
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            kvc.prefill_chunk_layers(2, q, k, v, 3 * n, o)
+            kvc.join()
+        graph.replay()
+    assert a.status() == 0 and b.status() == 0
+    assert torch.equal(*out)
+    for l in (0, 2, 3):
+        assert all(torch.equal(x[:, :B], y[:, :B]) for x, y in zip(a.cache_view(l)[:3], b.cache_view(l)[:3]))
+
+
 def test_batched_and_host_calls_beside_a_pending_compress():
     # the same calls on a context without the flag give the same bits
     layers, hq, hkv, d, B, n = 4, 8, 8, 64, 3000, 200
