@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(kCompressThreads, 2) compress_kernel(const __g
   int surplus = 0, row_cut = p.n_cand;                           // of the keys equal to thr, the last `surplus` rows do not survive
   // `ge` keys are at least as large as a thread's own, `rank` of them survive: the cut-off is the key with as many.  Nobody has
   // it if equal keys lie across the cut-off; then it is the largest key with more.
-  // (Requests cost up to 0.3 % for it: image 2731 -> 2741 us, proxies 1790 -> 1796, the others within their noise.  Counting
+  // (Requests cost up to 0.5 % for it: image 2731 -> 2741 us, proxies 1790 -> 1798, the others within their noise.  Counting
   // survivors against holes in the listing instead: 0.5 - 2.7 %, a matter of code size.)
   auto cut_at = [&](unsigned long long my, int ge, int rank) {
     if (ge == rank) sh.cutoff = my;
