@@ -16,8 +16,8 @@ static constexpr int kSubTileBytes = 128 * 128;   // 128 rows x 64 bf16 (one 128
 // kv-head.  A tile holds TOK = 128 / G tokens (TOK * G <= 128 rows).
 
 
-// K/V ring slots of the attention kernel: with one row tile per CTA the shared memory of the second Q tile and what is
-// left beside it hold two more, so that each of the two key chains has a key tile in flight beyond the one it works on.
+// K/V ring slots of the attention kernel, half of them for K: with one row tile per CTA the shared memory of the second Q tile
+// and what is left beside it hold two more.
 template <int R> __host__ __device__ constexpr int attn_stages() { return R == 1 ? 6 : 4; }
 
 // ------------------------------------------------------------------------------------------------
@@ -26,24 +26,25 @@ template <int R> __host__ __device__ constexpr int attn_stages() { return R == 1
 // [0, n_c) followed by the block's own tokens, which are read from the k/v inputs directly.
 //   warps 0-3   softmax of tile A     (thread = one row = one TMEM lane), 216 registers
 //   warps 4-7   softmax of tile B
-//   warp  8     TMA producer: Q tiles once, then K_j, V_j, K_j+1, ... through a ring of kStages 32 KB slots
-//   warp  9     MMA issuer of tile A, warp 10 of tile B (one lane each).  Per key tile j an issuer
-//               queues O_t += P_t V_j, then S_t = Q_t K_{j+1}^T.  P is handed over in two halves
-//               (64 keys each) so the first PV MMAs start while the second half of the exponentials
-//               is still being computed.  P -> P V -> next S -> softmax is the row tile's critical chain:
-//               with two row tiles the next S is issued directly behind the second half of P V, and the
-//               commits that free ring slots and publish O follow it.
-//   warp  11    only gives its registers away (setmaxnreg works on groups of four warps)
-// a0: the block's key / value tiles are stored into the cache from their ring slots (TMA stores issued by warp 9).
+//   warp  8     TMA producer: Q tiles once, then K_j and V_j through a ring of 32 KB slots, one half of it for each kind
+//   warp  9     issues S_t = Q_t K_j^T (one lane), warp 10 O_t += P_t V_j.  P is handed over in two halves (64 keys each) so
+//               the first PV MMAs start while the second half of the exponentials is still being computed.
+//   warp  11    a0: stores the block's key / value tiles into the cache from their ring slots (TMA stores)
 // The two softmax groups take turns on the exponentials (named barriers): while one tile's exponentials
-// occupy the CUDA cores the tensor pipe runs the other tile's MMAs; without the hand-over both tiles fall
-// into lockstep and the two pipes idle alternately.  Loading S and finding the maxima is outside the turn.
+// occupy the CUDA cores the other group loads its S and finds its maxima.
+// TMEM columns: S [0,128)  P_A [128,192)  P_B [192,256)  O_A [256,384)  O_B [384,512).  S is not kept under P: it is free
+// again as soon as a softmax group has it in registers, and the other group's next S is computed during the exponentials.
+// What binds the key loop is then the way from one S to the next (cycles, with one row tile per CTA): 240 for the load, 220
+// until the issuer sees all four warps past it, 630 of MMAs (Q and K both come from shared memory, 128 B a cycle), 300 - 450 until
+// the warps see the result; the exponentials of an item take 1400, and TMEM has no columns for a second S.  With P over S, as it
+// was before, the way was S -> maxima -> exponentials -> P V -> next S, with two row tiles in turns.  Requests before / after:
+// tiled image 2670 -> 2535 us, video 8370 -> 7966, long video 11869 -> 11368, image 2731 -> 2650, proxies 1796 -> 1735; the
+// results are the same bits.
 // (Measured and dropped: eight softmax warps per row tile, two threads per row, also in the form where a CTA
 // with a single row tile lends it the other tile's warps -- no faster; a polynomial 2^x on the FMA pipe for part
-// of the columns -- slower; S in two halves of 64 keys with the first issued early -- slower, MMAs with N = 64
-// read Q twice as often; exponentials against the running maximum with the tile's maximum found afterwards --
-// slower, the period is then bound by the two exponential phases, which that form lengthens.)
-// TMEM columns: S_A/P_A [0,128)  S_B/P_B [128,256)  O_A [256,384)  O_B [384,512).
+// of the columns -- slower; S in two halves of 64 keys -- an MMA with N = 64 takes as long as one with 128, long video 13250 us;
+// one thread for both kinds of MMA -- four commits an item, 14540; exponentials against the running maximum with the tile's
+// maximum found afterwards -- slower, the period is then bound by the two exponential phases, which that form lengthens.)
 // The running output is rescaled lazily: a row keeps its reference maximum until the true maximum
 // has grown by more than 2^8, so P stays below 256 and O rarely needs touching.
 //
@@ -51,12 +52,12 @@ template <int R> __host__ __device__ constexpr int attn_stages() { return R == 1
 // its row tile (one per CTA then) and ends with a partial (O, m, l).  The partials are exchanged through distributed
 // shared memory: rank s owns rows [s*128/S, (s+1)*128/S), every CTA sends the rows of another owner, (m, l) behind
 // them, in one bulk copy, and each rank combines and writes its rows.  Nothing but the final result goes to HBM.
-// Row tiles per CTA: R = 2 as described, or R = 1.  A CTA with one row tile runs it twice over: softmax group and
-// issuer t take its key tiles t, t+2, ... with S, P, O, maximum and row sum of their own (tile B's TMEM columns), and
+// Row tiles per CTA: R = 2 as described, or R = 1.  A CTA with one row tile runs it twice over: softmax group t takes its
+// key tiles t, t+2, ... with P, O, maximum and row sum of its own (tile B's TMEM columns), and
 // the two partial results are merged at the end, column half by column half straight from TMEM.  That doubles the CTA
 // count at about 1.06 times the cost per row tile and key tile.
-// What bounds a launch (device stamps, us): 1.3 until the first S (dependency wait, TMA, MMA), then 0.94 per key tile
-// with one row tile or 1.78 with two, 1.5 for the epilogue, 2.7 for the combine of a key split.  With the output through
+// What bounds a launch (device stamps, us): 1.3 until the first S (dependency wait, TMA, MMA), then 0.80 per key tile
+// with one row tile or 1.66 with two, 1.5 for the epilogue, 2.7 for the combine of a key split.  With the output through
 // shared memory, the merge from TMEM, the six-slot ring and cluster barriers that order no memory: tiled image (13 key
 // tiles, 128 CTAs) 16.4 -> 14.5, video (18 key tiles split over two, 112 CTAs) 17.5 -> 15.3; two row tiles (long video)
 // 73.3 -> 73.1.
@@ -65,9 +66,10 @@ template <int R> __host__ __device__ constexpr int attn_stages() { return R == 1
 static constexpr int kAttnThreads = 384;
 
 struct TcSmemAttn {
-  uint64_t q_full[2], kv_full[6], kv_empty[6], s_full[2], p_half[2][2], pv_done[2];
+  uint64_t q_full[2], kv_full[6], kv_empty[6], s_full[2], s_free, p_half[2][2], pv_done[2];
   uint64_t comb_full;        // key split: the other ranks' partial rows have landed in this CTA's shared memory
   uint32_t tmem_base;
+  int s_issued;              // two row tiles: the last item whose S has been issued
   int wait_ctl[2];           // [0] abort flag, [1] wait limit in units of 1024 cycles (see mbar_wait)
 };
 
@@ -86,6 +88,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
   constexpr int TILE_BYTES = NSUB * kSubTileBytes;
   constexpr uint32_t TMEM_COLS = 512;
   constexpr float kRescaleThreshold = 8.f;      // log2 units
+  // The turn is handed over when this quarter of P has been stored (2: tiled image 2540 -> 2560 us, video 7945 -> 7965).
+  constexpr int kTellAt = 3;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sQ = smem;                            // R tiles; after the key loop: the output tiles
@@ -115,20 +119,24 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
   const int T = Tc + (last_tok + 128) / 128;
   const int t_begin = split * T / S, t_end = (split + 1) * T / S;
   const int Tl = t_end - t_begin;                // key tiles of this CTA (0 is possible when S > T)
-  // A CTA with one row tile runs it twice over: softmax group and issuer t take the key tiles t, t+2, ... with
-  // accumulators, maxima and sums of their own (the TMEM columns of tile B are free), two key tiles are in flight as
+  // A CTA with one row tile runs it twice over: softmax group t takes the key tiles t, t+2, ... with accumulators, maxima and sums of their own (the TMEM columns of tile B are free), two key tiles are in flight as
   // with two row tiles, and the two partial results are merged at the end.  (With Tl = 1 group 1 has none; Tl = 0
   // happens with a key split, for the first rows of a block that see less of it than the last ones.)
   const bool alt = !has_B;
   const int n_it0 = alt ? (Tl + 1) / 2 : Tl, n_it1 = alt ? Tl / 2 : Tl;   // key tiles of group 0 / 1
+
+  // block tiles [u_lo, u_hi) of this CTA that it appends to the cache (see warp 11): those that begin in its rows
+  const int u_lo = max(max(t_begin - Tc, 0), (tokA + 127) / 128), u_hi = min(t_end - Tc, (tok_end + 127) / 128);
+  const bool appends = u_hi > u_lo;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) {
       mbar_init(&sh.q_full[i], 1); mbar_init(&sh.s_full[i], 1); mbar_init(&sh.pv_done[i], 1);
       mbar_init(&sh.p_half[i][0], 4); mbar_init(&sh.p_half[i][1], 4);     // one arrival per softmax warp
     }
-    // a ring slot is free again once the issuer of every active row tile has committed its MMAs on it
-    for (int i = 0; i < kStages; ++i) { mbar_init(&sh.kv_full[i], 1); mbar_init(&sh.kv_empty[i], has_B ? 2 : 1); }
+    mbar_init(&sh.s_free, 4);                                             // (likewise)
+    for (int i = 0; i < kStages; ++i) { mbar_init(&sh.kv_full[i], 1); mbar_init(&sh.kv_empty[i], appends ? 2 : 1); }
+    sh.s_issued = -1;
     sh.wait_ctl[0] = 0; sh.wait_ctl[1] = p.wait_limit_k;
     mbar_init(&sh.comb_full, 1);
     // key split: every other rank of the cluster will copy its partial of this rank's rows here
@@ -154,8 +162,26 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
   const uint32_t tmem = sh.tmem_base;
   volatile int* abort_flag = sh.wait_ctl;
 
+  // The items of this CTA, in the order in which everything below takes them: item i is softmax group i & 1's next key tile.
+  // Two row tiles: items 2j and 2j + 1 are key tile j of row tile A and B; one row tile: item i is key tile i.
+  const int n_items = has_B ? 2 * Tl : Tl;
+
   if (warp >= 8) {
     reg_dec<56>();                               // (with 64 or 72 the compiler spills in the softmax groups of some forms: 2 - 8 % slower)
+    // Ring: K tiles go round the first kSlots slots, V tiles round the others.
+    constexpr int kSlots = kStages / 2;
+    auto load_tile = [&](int j, int v) {           // K (v = 0) or V (1) of local key tile j; false: gave up
+      const int slot = v * kSlots + j % kSlots, round = j / kSlots, kt = t_begin + j;
+      if (round > 0 && !mbar_wait(&sh.kv_empty[slot], (round - 1) & 1, abort_flag)) return false;
+      mbar_expect_tx(&sh.kv_full[slot], TILE_BYTES);
+      uint8_t* dst = ring + slot * TILE_BYTES;
+      if (kt < Tc) {                             // cache rows kt*128 .. (rows past n_c are masked by the softmax)
+        for (int sub = 0; sub < NSUB; ++sub) tma_load_4d(dst + sub * kSubTileBytes, v ? &tm_v : &tm_k, &sh.kv_full[slot], sub * 64, kt * 128, g, layer);
+      } else {                                   // block tokens (kt - Tc)*128 .. (tokens past n are zero-filled)
+        for (int sub = 0; sub < NSUB; ++sub) tma_load_4d(dst + sub * kSubTileBytes, v ? &tm_vin : &tm_kin, &sh.kv_full[slot], sub * 64, g, (kt - Tc) * 128, layer);
+      }
+      return true;
+    };
     if (warp == 8) {
       // ---------------------------------------------------------------- TMA producer
       if (lane == 0) {
@@ -169,7 +195,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
           if (lane == 0 || has_B)
             for (int sub = 0; sub < NSUB; ++sub) tma_prefetch_l2_4d(&tm_q, sub * 64, g * p.G, lane ? tokB : tokA, layer);
         } else {
-          const int i = (lane - 2) / NSUB, sub = (lane - 2) % NSUB;      // ring item i: K or V of key tile t_begin + i/2
+          const int i = (lane - 2) / NSUB, sub = (lane - 2) % NSUB;      // K or V of key tile t_begin + i/2
           const int kt = t_begin + (i >> 1);
           if (kt < Tc) tma_prefetch_l2_4d((i & 1) ? &tm_v : &tm_k, sub * 64, kt * 128, g, layer);
           else tma_prefetch_l2_4d((i & 1) ? &tm_vin : &tm_kin, sub * 64, g, (kt - Tc) * 128, layer);
@@ -185,152 +211,110 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
         mbar_expect_tx(&sh.q_full[0], NSUB * rows * 128);
         for (int sub = 0; sub < NSUB; ++sub)
           tma_load_4d(sQ + sub * kSubTileBytes, &tm_q, &sh.q_full[0], sub * 64, g * p.G, tokA, layer);
-        for (int i = 0; i < 2 * Tl; ++i) {         // item 2j = K of tile t_begin + j, item 2j+1 = V of it
-          const int slot = i % kStages, round = i / kStages;
-          if (round > 0 && !mbar_wait(&sh.kv_empty[slot], (round - 1) & 1, abort_flag)) break;
-          mbar_expect_tx(&sh.kv_full[slot], TILE_BYTES);
-          const int kt = t_begin + (i >> 1);
-          if (kt < Tc) {                           // cache rows kt*128 .. (rows past n_c are masked by the softmax)
-            const CUtensorMap* tm = (i & 1) ? &tm_v : &tm_k;
-            for (int sub = 0; sub < NSUB; ++sub)
-              tma_load_4d(ring + slot * TILE_BYTES + sub * kSubTileBytes, tm, &sh.kv_full[slot], sub * 64, kt * 128, g, layer);
-          } else {                                 // block tokens (kt - Tc)*128 .. (tokens past n are zero-filled)
-            const CUtensorMap* tm = (i & 1) ? &tm_vin : &tm_kin;
-            for (int sub = 0; sub < NSUB; ++sub)
-              tma_load_4d(ring + slot * TILE_BYTES + sub * kSubTileBytes, tm, &sh.kv_full[slot], sub * 64, g, (kt - Tc) * 128, layer);
-          }
-          if (i == 0 && has_B) {                   // (row tile A can start on Q_A and the first K tile)
+        // In the order in which they are needed: an SM takes in 64 bytes a cycle, and V tiles asked for beside the first K tile
+        // hold it up (three key tiles: 0.5 us of a call of 8).  Behind the first fill K runs a tile ahead of V, as S does.
+        const int fill = min(Tl, kSlots);
+        for (int j = 0; j < fill; ++j) {
+          load_tile(j, 0);
+          if (j == 0 && has_B) {                   // (row tile A can start on Q_A and the first K tile)
             mbar_expect_tx(&sh.q_full[1], NSUB * rows * 128);
             for (int sub = 0; sub < NSUB; ++sub)
               tma_load_4d(sQ + TILE_BYTES + sub * kSubTileBytes, &tm_q, &sh.q_full[1], sub * 64, g * p.G, tokB, layer);
           }
+          load_tile(j, 1);
+        }
+        for (int j = fill; j < Tl + 1; ++j) {
+          if (j < Tl && !load_tile(j, 0)) break;
+          if (j > fill && !load_tile(j - 1, 1)) break;
         }
       }
-    } else if (warp == 9 || warp == 10) {
-      // ---------------------------------------------------------------- MMA issuer of tile t
-      // a0 append (Alg. 1: C <- C u (K_i, V_i)).  The block's keys and values pass through the ring as key tiles
-      // anyway: the issuer of tile A stores such a tile from its ring slot into cache rows n_c + 128u .. with one
-      // TMA store per 64 columns (rows past the block are zero in the tile and land in unused cache rows or are
-      // clipped at cap).  Among the CTAs that load block tile u, the one whose rows contain token 128u owns it.
-      // Nobody in this kernel reads the appended rows.  The lanes of the warp write the positions.
-      const int u_lo = max(t_begin, Tc) - Tc, u_hi = t_end - Tc;            // block tiles of this CTA: [u_lo, u_hi)
-      auto owns = [&](int u) { return u * 128 >= tokA && u * 128 < tok_end; };
-      if (warp == 9 && u_hi > u_lo) {
-        bool waited = false;
-        for (int u = u_lo; u < u_hi; ++u) {
-          if (!owns(u)) continue;
-          if (!waited) { pdl_wait(); waited = true; }                       // the previous block's compaction is done with the cache
-          int* pos = reinterpret_cast<int*>(cache + layer * p.cache_ls + p.pos_off) + static_cast<long long>(g) * p.cap + p.n_c;
+    } else if (warp == 11) {
+      // ---------------------------------------------------------------- a0 append (Alg. 1: C <- C u (K_i, V_i))
+      // The block's keys and values pass through the ring as key tiles anyway: such a tile is stored from its ring slot into
+      // cache rows n_c + 128u .. with one TMA store per 64 columns (rows past the block are zero in the tile and land in unused
+      // cache rows or are clipped at cap).  Among the CTAs that load block tile u, the one whose rows contain token 128u owns
+      // it.  Nobody in this kernel reads the appended rows.  In a CTA that owns tiles every slot is handed back by this warp,
+      // too, once a store has read it.
+      if (appends) {
+        pdl_wait();                                // the previous block's compaction is done with the cache
+        int* pos = reinterpret_cast<int*>(cache + layer * p.cache_ls + p.pos_off) + static_cast<long long>(g) * p.cap + p.n_c;
+        for (int u = u_lo; u < u_hi; ++u)
           for (int i = u * 128 + lane; i < min(p.n, u * 128 + 128); i += 32) pos[i] = static_cast<int>(p.pos0 + i);
+        if (lane == 0) {
+          for (int i = 0; i < 2 * Tl; ++i) {       // K and V of local key tile i / 2
+            const int j = i >> 1, slot = (i & 1) * kSlots + j % kSlots, u = t_begin + j - Tc;
+            if (!mbar_wait(&sh.kv_full[slot], (j / kSlots) & 1, abort_flag)) break;
+            if (u >= u_lo && u < u_hi) {
+              for (int sub = 0; sub < NSUB; ++sub)
+                tma_store_4d((i & 1) ? &tm_v : &tm_k, ring + slot * TILE_BYTES + sub * kSubTileBytes, sub * 64, p.n_c + u * 128, g, layer);
+              tma_store_commit();
+              tma_store_wait_read();
+            }
+            mbar_arrive(&sh.kv_empty[slot]);
+          }
         }
       }
-      if (lane == 0 && (warp == 9 ? n_it0 : n_it1) > 0) {
-        const int t = warp - 9;
-        bool stored = false, store_waited = false;
-        // item i of the ring (2j = K, 2j+1 = V of local key tile j) has landed in `slot`: store it if it is ours
-        // (with two row tiles the issuer of tile A stores, else the issuer that consumes the item);
-        // true if the slot must not be handed back before the store has read it
-        auto append_item = [&](int i, int slot) {
-          const int u = t_begin + (i >> 1) - Tc;
-          if ((t != 0 && !alt) || u < 0 || !owns(u)) return false;
-          if (!store_waited) { pdl_wait(); store_waited = true; }
-          const CUtensorMap* tm = (i & 1) ? &tm_v : &tm_k;
-          for (int sub = 0; sub < NSUB; ++sub)
-            tma_store_4d(tm, ring + slot * TILE_BYTES + sub * kSubTileBytes, sub * 64, p.n_c + u * 128, g, layer);
-          tma_store_commit();
-          stored = true;
-          return i + kStages < 2 * Tl;
-        };
+    } else if (warp == 9) {
+      // ---------------------------------------------------------------- issuer of S = Q K^T, item by item
+      // S has one buffer of 128 columns: the next item's S is issued as soon as a group has this one in its registers, and is
+      // there by the time the other group comes for it.  (One thread for both kinds of MMA is too slow: four commits an item.)
+      if (lane == 0 && n_items > 0) {
         constexpr uint32_t idesc_qk = idesc_bf16_f32(128, 128, 0, 0);
+        constexpr uint32_t hi = smem_desc_hi_sw128(1024);
+        const uint32_t q_lo0 = smem_desc_lo(smem_u32(sQ), 16), k_lo0 = smem_desc_lo(smem_u32(ring), 16);   // K-major operands
+        bool ok = mbar_wait(&sh.q_full[0], 0, abort_flag);
+        for (int i = 0; i < n_items && ok; ++i) {
+          const int t = i & 1, j = has_B ? i >> 1 : i, slot = j % kSlots;
+          if (!has_B || t == 0) ok = mbar_wait(&sh.kv_full[slot], (j / kSlots) & 1, abort_flag);
+          if (ok && has_B && i == 1) ok = mbar_wait(&sh.q_full[1], 0, abort_flag);
+          if (ok && i > 0) ok = mbar_wait_spin(&sh.s_free, (i - 1) & 1, abort_flag);
+          if (!ok) break;
+          tc_fence_after_sync();
+          const uint32_t q_lo = q_lo0 + (has_B ? t : 0) * (TILE_BYTES >> 4), k_lo = k_lo0 + slot * (TILE_BYTES >> 4);
+#pragma unroll
+          for (int kk = 0; kk < D / 16; ++kk) {      // 16 of the d columns per MMA
+            const uint32_t off = ((kk / 4) * kSubTileBytes + (kk % 4) * 32) >> 4;
+            mma_ss_lh(tmem, q_lo + off, hi, k_lo + off, hi, idesc_qk, kk > 0);
+          }
+          mma_commit(&sh.s_full[t]);
+          if (has_B) *static_cast<volatile int*>(&sh.s_issued) = i;
+          if (!has_B || t == 1) mma_commit(&sh.kv_empty[slot]);
+        }
+      }
+    } else {
+      // ---------------------------------------------------------------- issuer of O_t += P_t V, item by item, half by half
+      // With two row tiles per CTA it lets the S of the item after next go first: that one is wanted soon, while P V of this
+      // item has time until the group's next P (long video 11675 -> 11457 us per request, hybrid 3083 -> 3049; with one row
+      // tile per CTA 1 % slower).
+      if (lane == 0 && n_items > 0) {
         constexpr uint32_t idesc_pv = idesc_bf16_f32(128, D, 0, 1);
         constexpr uint32_t hi = smem_desc_hi_sw128(1024);
-        const uint32_t q_lo = smem_desc_lo(smem_u32(sQ) + (alt ? 0 : t) * TILE_BYTES, 16);   // K-major operand
-        const uint32_t k_lo0 = smem_desc_lo(smem_u32(ring), 16);                        // K-major operand
-        const uint32_t v_lo0 = smem_desc_lo(smem_u32(ring), kSubTileBytes);             // MN-major operand
-        const uint32_t tS = tmem + t * 128, tO = tmem + 256 + t * 128;
-        const int first = alt ? t : 0, step = alt ? 2 : 1;   // local key tiles of this issuer: first, first + step, ...
-        auto issue_S = [&](int slot) {               // S_t = Q_t K^T, 16 of the d columns per MMA
-          const uint32_t k_lo = k_lo0 + slot * (TILE_BYTES >> 4);
+        const uint32_t v_lo0 = smem_desc_lo(smem_u32(ring) + kSlots * TILE_BYTES, kSubTileBytes);   // MN-major operand
+        bool ok = true;
+        for (int i = 0; i < n_items && ok; ++i) {
+          const int t = i & 1, it = i >> 1, j = has_B ? it : i, slot = j % kSlots;
+          if (!has_B || t == 0) ok = mbar_wait(&sh.kv_full[kSlots + slot], (j / kSlots) & 1, abort_flag);
+          const uint32_t v_lo = v_lo0 + slot * (TILE_BYTES >> 4), tP = tmem + 128 + t * 64, tO = tmem + 256 + t * 128;
 #pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) {
-            const uint32_t off = ((kk / 4) * kSubTileBytes + (kk % 4) * 32) >> 4;
-            mma_ss_lh(tS, q_lo + off, hi, k_lo + off, hi, idesc_qk, kk > 0);
-          }
-        };
-        auto issue_PV = [&](int slot, int half, bool acc) {   // O_t += P_t V, 16 keys per MMA, 64 keys per half
-          const uint32_t v_lo = v_lo0 + slot * (TILE_BYTES >> 4);
-#pragma unroll
-          for (int kk = 4 * half; kk < 4 * half + 4; ++kk)
-            mma_ts_lh(tO, tS + kk * 8, v_lo + kk * (2048 >> 4), hi, idesc_pv, acc || kk > 0);
-        };
-        const int i0 = 2 * first;                    // ring item of this issuer's first K tile (slot i0, first round)
-        bool ok = mbar_wait(&sh.q_full[alt ? 0 : t], 0, abort_flag) && mbar_wait(&sh.kv_full[i0], 0, abort_flag);
-        if (ok) {
-          tc_fence_after_sync();
-          issue_S(i0);
-          mma_commit(&sh.s_full[t]);
-          if (append_item(i0, i0)) tma_store_wait_read();
-          mma_commit(&sh.kv_empty[i0]);
-        }
-        for (int jj = first, it = 0; jj < Tl && ok; jj += step, ++it) {
-          const int jn = jj + step;                  // the key tile whose S is queued behind P V of this one
-          const int iv = 2 * jj + 1, ik = 2 * jn;
-          const int slotV = iv % kStages, slotK = ik % kStages;
-          ok = mbar_wait_spin(&sh.p_half[t][0], it & 1, abort_flag) && mbar_wait(&sh.kv_full[slotV], (iv / kStages) & 1, abort_flag);
-          if (!ok) break;
-          tc_fence_after_sync();
-          issue_PV(slotV, 0, it > 0);
-          const bool hold_v = append_item(iv, slotV);
-          // What follows the second half of P is the row tile's critical chain (P -> P V -> next S -> softmax).  With
-          // two row tiles nothing else sits between the two groups of MMAs: the next K tile (landed long ago) is
-          // waited for here, and the commits that free the slots and publish O come after the next S has been issued
-          // (they then complete with it, which nobody minds: O is read after the next S at the earliest).  In-kernel
-          // stamps put the commits and the wait at 380 of the chain's 4000 cycles.  A CTA with one row tile in a
-          // launch of two (ring of four slots) has two key chains, every ring item feeds one of them only, and the
-          // ring holds one key tile per chain: there the V slot goes back to the producer first, and the K tile is
-          // waited for when it is needed (measured: the deferred order starves the other chain and costs 13 %; with
-          // the six slots of a one-row-tile launch it gains 3 %).
-          const bool defer = !alt || R == 1;
-          if (defer && jn < Tl) {
-            ok = mbar_wait(&sh.kv_full[slotK], (ik / kStages) & 1, abort_flag);
+          for (int half = 0; half < 2; ++half) {
+            ok = ok && mbar_wait_spin(&sh.p_half[t][half], it & 1, abort_flag);
+            if (has_B && half == 0) ok = ok && word_wait_spin(&sh.s_issued, min(i + 2, n_items - 1), abort_flag);
             if (!ok) break;
+            tc_fence_after_sync();
+#pragma unroll
+            for (int kk = 4 * half; kk < 4 * half + 4; ++kk)   // 16 keys per MMA, 64 keys per half
+              mma_ts_lh(tO, tP + kk * 8, v_lo + kk * (2048 >> 4), hi, idesc_pv, it > 0 || kk > 0);
           }
-          ok = mbar_wait_spin(&sh.p_half[t][1], it & 1, abort_flag);
           if (!ok) break;
-          tc_fence_after_sync();
-          issue_PV(slotV, 1, true);
-          if (!defer) {
-            mma_commit(&sh.pv_done[t]);
-            if (hold_v) tma_store_wait_read();
-            mma_commit(&sh.kv_empty[slotV]);
-            if (jn < Tl) {
-              ok = mbar_wait(&sh.kv_full[slotK], (ik / kStages) & 1, abort_flag);
-              if (!ok) break;
-              tc_fence_after_sync();
-            }
-          }
-          if (jn < Tl) {
-            issue_S(slotK);
-            mma_commit(&sh.s_full[t]);
-          }
-          if (defer) {
-            mma_commit(&sh.pv_done[t]);
-            if (hold_v) tma_store_wait_read();
-            mma_commit(&sh.kv_empty[slotV]);
-          }
-          if (jn < Tl) {
-            if (append_item(ik, slotK)) tma_store_wait_read();
-            mma_commit(&sh.kv_empty[slotK]);
-          }
+          mma_commit(&sh.pv_done[t]);
+          if (!has_B || t == 1) mma_commit(&sh.kv_empty[kSlots + slot]);
         }
-        // the stores have read their ring slots (the combine of a key split reuses the ring) ...
-        if (stored) tma_store_wait_read();
       }
     }
     __syncwarp();
     // One row tile: the epilogue writes over the ring and the Q tile once both key chains are complete, which says
-    // nothing about the stores above; warps 9 and 10 tell it here that no store reads the ring any more.
-    if (alt && (warp == 9 || warp == 10)) named_barrier_arrive(5, 256 + 64);
+    // nothing about the stores above; warp 11 tells it here that no store reads the ring any more.
+    if (alt && warp == 11) named_barrier_arrive(5, 256 + 32);
     if (S > 1) {                                             // the cluster barriers of the combine below
       cluster_arrive_relaxed(); cluster_wait();
       cluster_arrive_relaxed(); cluster_wait();
@@ -345,7 +329,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
     const int tok = tok0 + r / p.G, hh = r % p.G;
     const bool row_valid = r < rows && tok < p.n;
     const uint32_t lane_addr = static_cast<uint32_t>((warp & 3) * 32) << 16;
-    const uint32_t tmem_S = tmem + t * 128 + lane_addr, tmem_O = tmem + 256 + t * 128 + lane_addr;
+    const uint32_t tmem_S = tmem + lane_addr, tmem_P = tmem + 128 + t * 64 + lane_addr, tmem_O = tmem + 256 + t * 128 + lane_addr;
     float m_ref = -INFINITY, l = 0.f;                        // reference maximum (log2 units) and row sum
     bool ok = true;
     const int first = alt ? t : 0, step = alt ? 2 : 1;       // local key tiles of this group: first, first + step, ...
@@ -358,13 +342,19 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
         // Waits that gave up only skip the arithmetic: the turn barrier is passed on every path, once per key
         // tile and warp, so the other row tile never waits for a turn that is not handed over.
         if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&sh.s_full[t], it & 1, abort_flag));
-        bool took_turn = false;
+        bool took_turn = false, told = false;
+        const bool hand_over = t == 0 ? it < n_it1 : it + 1 < n_it0;   // the other group has a key tile left: its it-th (group 0 asks) or (it+1)-th
         if (ok) do {
         tc_fence_after_sync();
         uint32_t sr[128];
 #pragma unroll
         for (int c = 0; c < 4; ++c) tmem_ld32(tmem_S + c * 32, sr + c * 32);
+        // O_t holds every earlier tile, and the columns of P are free?  (asked while S is on its way; long so as a rule)
+        const bool pv_ready = it > 0 && mbar_test_wait(&sh.pv_done[t], (it - 1) & 1);
         tmem_wait_ld();
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sh.s_free);               // the other group's next S may be computed
         // columns [0, lim) of this tile are visible: a cache tile ends at row n_c, a block tile at the row's
         // own token (causal inside the block); only the last cache tile and diagonal tiles need the mask
         const int u = kt - Tc;                                // >= 0: tile of the block's own tokens
@@ -384,27 +374,30 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
         }
         const float mx = fmaxf(fmax3(mx4[0], mx4[1], mx4[2]), fmaxf(fmax3(mx4[3], mx4[4], mx4[5]), fmaxf(mx4[6], mx4[7])));
         const float m_new = mx * p.scale_log2;                // scale > 0
-        if (it == 0) {
-          m_ref = m_new == -INFINITY ? 0.f : m_new;
-        } else {
-          const bool grow = m_new > m_ref + kRescaleThreshold;
-          if (__any_sync(0xffffffffu, grow)) {
-            const float f = grow ? fast_exp2(m_ref - m_new) : 1.f;
-            if (grow) { m_ref = m_new; l *= f; }
-            ok = __all_sync(0xffffffffu, mbar_wait(&sh.pv_done[t], (it - 1) & 1, abort_flag));  // O_t holds every earlier tile
+        const bool grow = m_new > m_ref + kRescaleThreshold;  // (first tile: m_ref is -infinity)
+        if (__any_sync(0xffffffffu, grow || !pv_ready)) {
+          if (it == 0) {
+            m_ref = m_new == -INFINITY ? 0.f : m_new;
+          } else {
+            ok = __all_sync(0xffffffffu, mbar_wait(&sh.pv_done[t], (it - 1) & 1, abort_flag));
             if (!ok) break;
-            tc_fence_after_sync();
+            if (__any_sync(0xffffffffu, grow)) {
+              tc_fence_after_sync();
+              const float f = grow ? fast_exp2(m_ref - m_new) : 1.f;
+              if (grow) { m_ref = m_new; l *= f; }
 #pragma unroll
-            for (int c = 0; c < D / 32; ++c) {
-              uint32_t o[32];
-              tmem_ld32(tmem_O + c * 32, o);
-              tmem_wait_ld();
+              for (int c = 0; c < D / 32; ++c) {
+                uint32_t o[32];
+                tmem_ld32(tmem_O + c * 32, o);
+                tmem_wait_ld();
 #pragma unroll
-              for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
-              tmem_st32(tmem_O + c * 32, o);
+                for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
+                tmem_st32(tmem_O + c * 32, o);
+              }
             }
           }
         }
+        tc_fence_after_sync();
         // Only the exponentials are taken in turns: loading S and finding the row maxima overlap the other
         // tile's exponentials.
         if (turns) { named_barrier(2 + t, 256); took_turn = true; }
@@ -422,15 +415,16 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
             ps2[i & 1] = add_f32x2(ps2[i & 1], f32x2(p0, p1));
             pk[i] = pack_bf16x2(p0, p1);
           }
-          tmem_st16(tmem_S + c * 16, pk);
-          if (c & 1) {                                        // 64 keys of P are in TMEM: release them to the MMA warp
+          if (c == 2) {                                       // the first 64 keys of P have landed: the MMA warp may take them
             tmem_wait_st();
             tc_fence_before_sync();
             // one arrival per warp: 128 arrivals on one shared-memory word are served one after the other, and the
             // issuer saw the barrier complete some 300 cycles after the first of them (in-kernel stamps)
             __syncwarp();
-            if (lane == 0) mbar_arrive(&sh.p_half[t][c >> 1]);
+            if (lane == 0) mbar_arrive(&sh.p_half[t][0]);
           }
+          tmem_st16(tmem_P + c * 16, pk);
+          if (c == kTellAt) { if (turns && hand_over) named_barrier_arrive(3 - t, 256); told = true; }
         }
         {
           float ps[4];
@@ -438,10 +432,13 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
           f32x2_split(ps2[1], ps[2], ps[3]);
           l += (ps[0] + ps[1]) + (ps[2] + ps[3]);
         }
+        tmem_wait_st();
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sh.p_half[t][1]);
         } while (0);
         if (turns && !took_turn) named_barrier(2 + t, 256);   // a wait gave up before the turn was taken: take it now
-        // hand the turn over if the other group has a key tile left: its it-th (group 0 asks) or (it+1)-th (group 1)
-        if (turns && (t == 0 ? it < n_it1 : it + 1 < n_it0)) named_barrier_arrive(3 - t, 256);
+        if (turns && !told && hand_over) named_barrier_arrive(3 - t, 256);
       }
       // The key loop is over: the next kernel of the stream may be scheduled and set itself up while this one
       // writes its results.  (Triggered at the start instead, the waiting CTAs of the next attention launch take the
@@ -492,18 +489,18 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
       }
     } else {
       // One row tile, two key chains.  Both accumulators sit in TMEM on the same lanes, so no thread has to hand rows
-      // over: group t takes half the columns of both, and only (m, l) are exchanged (through the TMEM columns of S).
+      // over: group t takes half the columns of both, and only (m, l) are exchanged (through the TMEM columns of P).
       constexpr int H = D / 2;
       if (ok && n_it0 > 0) ok = mbar_wait(&sh.pv_done[0], (n_it0 - 1) & 1, abort_flag);
       if (ok && n_it1 > 0) ok = mbar_wait(&sh.pv_done[1], (n_it1 - 1) & 1, abort_flag);
       ok = __all_sync(0xffffffffu, ok);
       if (ok) {
         tc_fence_after_sync();
-        tmem_st2(tmem_S, __float_as_uint(l > 0.f ? m_ref : -INFINITY), __float_as_uint(l));   // -inf: no key of the row seen
+        tmem_st2(tmem_P, __float_as_uint(l > 0.f ? m_ref : -INFINITY), __float_as_uint(l));   // -inf: no key of the row seen
         tmem_wait_st();
         tc_fence_before_sync();
       }
-      named_barrier(5, 256 + 64);                              // both groups are here, and no store reads the ring
+      named_barrier(5, 256 + 32);                              // both groups are here, and no store reads the ring
       // This CTA's shared memory may be written by the cluster: everything that used it is complete and nothing was
       // written there through the generic proxy, so the arrival need not order memory (a release costs 0.4 us here).
       if (S > 1) cluster_arrive_relaxed();
@@ -511,7 +508,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
       if (ok) {
         tc_fence_after_sync();
         uint32_t mb, lb;
-        tmem_ld2(tmem + (1 - t) * 128 + lane_addr, mb, lb);
+        tmem_ld2(tmem + 128 + (1 - t) * 64 + lane_addr, mb, lb);
         tmem_wait_ld();
         const float m_own = l > 0.f ? m_ref : -INFINITY, m_oth = __uint_as_float(mb), l_oth = __uint_as_float(lb);
         m_all = fmaxf(m_own, m_oth);

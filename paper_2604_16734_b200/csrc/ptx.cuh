@@ -85,6 +85,22 @@ __device__ __forceinline__ bool mbar_wait_spin(uint64_t* bar, uint32_t parity, v
   }
 }
 
+// The same bounded spin until a counter in shared memory has reached `want`.
+__device__ __forceinline__ bool word_wait_spin(volatile int* word, int want, volatile int* wait_ctl) {
+  if (*word >= want) return true;
+  const long long t0 = clock64();
+  while (true) {
+#pragma unroll 1
+    for (int i = 0; i < 64; ++i)
+      if (*word >= want) return true;
+    if (wait_ctl[0]) return false;
+    if (((clock64() - t0) >> 10) > static_cast<long long>(wait_ctl[1])) {
+      wait_ctl[0] = 1;
+      return false;
+    }
+  }
+}
+
 // ---------------------------------------------------------------- proxies / fences
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

@@ -106,3 +106,19 @@ def test_compress_on_a_side_stream_gives_the_same_bits(hq, hkv, d, n, B, window)
     assert all(torch.equal(a, b) for a, b in zip(outs_a, outs_b))
     assert all(torch.equal(a[:, :B], b[:, :B]) for a, b in zip(cache_a, cache_b))
     assert torch.equal(score_a, score_b)
+
+
+@pytest.mark.parametrize("hq,hkv,d,n,blocks,row_tiles", [
+    (4, 2, 128, 128, 9, 1),                           # one to nine key tiles: below, at and around a ring of three per kind,
+    (4, 2, 64, 100, 9, 1),                            # the appended tile in each of its slots
+    (32, 32, 64, 640, 3, 2),                          # two row tiles per CTA: a ring of two, blocks of five tiles
+    (28, 4, 128, 784, 2, 2),                          # pairs and single row tiles on the same ring
+])
+def test_key_tiles_around_the_ring(hq, hkv, d, n, blocks, row_tiles):
+    torch.manual_seed(n)
+    kvc = Kvc(1, hq, hkv, d, torch.bfloat16, n * blocks, n, flags=4)     # KVC_FLAG_NO_KEY_SPLIT
+    orc = KVCOracle(1, hq, hkv, d, n * blocks, 32)
+    for i in range(blocks):
+        q, k, v = (torch.randn(n, h, d).to(torch.bfloat16) for h in (hq, hkv, hkv))
+        compare_chunk(kvc, orc, 0, q, k, v, i * n)    # (and the cached rows, bit for bit)
+    assert launch_shape(kvc, n, n * (blocks - 1))[0] == row_tiles
