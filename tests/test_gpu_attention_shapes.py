@@ -122,3 +122,15 @@ def test_key_tiles_around_the_ring(hq, hkv, d, n, blocks, row_tiles):
         q, k, v = (torch.randn(n, h, d).to(torch.bfloat16) for h in (hq, hkv, hkv))
         compare_chunk(kvc, orc, 0, q, k, v, i * n)    # (and the cached rows, bit for bit)
     assert launch_shape(kvc, n, n * (blocks - 1))[0] == row_tiles
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(2, 2, 64), (6, 2, 128)])
+@pytest.mark.parametrize("n_c", [1, 31, 32, 33, 64, 95, 96, 97, 127, 129])
+def test_mask_at_the_quarters_of_a_tile(hq, hkv, d, n_c):
+    # the last cache tile ends at row n_c, the block's own tile at every row's token: limits around multiples of 32 columns
+    torch.manual_seed(n_c)
+    kvc = Kvc(1, hq, hkv, d, torch.bfloat16, n_c, 130, 1)
+    orc = KVCOracle(1, hq, hkv, d, n_c, 1)
+    for pos, n in ((0, n_c), (n_c, 130)):
+        q, k, v = (torch.randn(n, h, d).to(torch.bfloat16) for h in (hq, hkv, hkv))
+        compare_chunk(kvc, orc, 0, q, k, v, pos)
