@@ -554,6 +554,9 @@ static cudaError_t launch_cc_score(const Geom& g, int dev, const void* q, const 
 // 17.0 / 27.3 / 45.9 / 92.9;  784 x 7, 4, 2832 keys 46.6 / 46.9 / 52.7;  1000 x 1, 32, 1500 keys 29.3 / 33.7 / 51.4;
 // 256 x 4, 2, 1280 keys 21.3 / 12.9 / 10.9 / 9.3 / 18.1;  100 x 3, 4, 4100 keys 61.4 / 33.2 / 21.5 / 14.9 / 12.6;
 // 128 x 1, 32, 320 keys 7.2 / 7.2 / 9.2 / 7.8 / 25.7.  On all sixteen the model picks the fastest or is within 1 %.
+// (Fitted, and the figures taken, while S still lay under P; since then a key tile costs 0.80 and 1.66.  The rule stays: the shape
+// groups a row's keys, which decides the last bits of its log-sum-exp and, between candidates whose scores agree to seven
+// digits, which of them is retained.)
 // (An exchange of the partials through an L2-resident global buffer instead of distributed shared memory was measured
 // too: slower, the release / acquire round trip costs more than the narrow SM-to-SM path.)
 struct AttnShape { int R, S, n_pairs; long long ctas; };
