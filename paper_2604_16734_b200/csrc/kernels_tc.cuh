@@ -67,6 +67,7 @@ static constexpr int kAttnThreads = 384;
 
 struct TcSmemAttn {
   uint64_t q_full[2], kv_full[6], kv_empty[6], s_full[2], s_free, p_half[2][2], pv_done[2];
+  uint64_t mma_done[2];      // a wait ran out: every MMA that this issuer issued is complete
   uint64_t comb_full;        // key split: the other ranks' partial rows have landed in this CTA's shared memory
   uint32_t tmem_base;
   int s_issued;              // two row tiles: the last item whose S has been issued
@@ -138,6 +139,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
     for (int i = 0; i < kStages; ++i) { mbar_init(&sh.kv_full[i], 1); mbar_init(&sh.kv_empty[i], appends ? 2 : 1); }
     sh.s_issued = -1;
     sh.wait_ctl[0] = 0; sh.wait_ctl[1] = p.wait_limit_k;
+    mbar_init(&sh.mma_done[0], 1); mbar_init(&sh.mma_done[1], 1);
     mbar_init(&sh.comb_full, 1);
     // key split: every other rank of the cluster will copy its partial of this rank's rows here
     if (S > 1) mbar_expect_tx(&sh.comb_full, (S - 1) * (128 / S) * (D + 4) * 4);
@@ -318,8 +320,20 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
     if (S > 1) { cluster_arrive_relaxed(); cluster_wait(); }  // the cluster barriers of the combine below
     // No barrier of the whole block at the end: TMEM is given back as soon as the softmax warps have read it for the last time,
     // and every warp leaves when it is done (requests: video 7944 -> 7855 us, query-agnostic 1268 -> 1261, image 2652 -> 2643).
+    // The softmax warps may be here without their results, when a wait ran out.  Then an issuer can have MMAs under way, or a
+    // tile can have landed for it that it issued some on: it comes here behind its loop and sees them to their end.
+    // (Requests: video 7852 -> 7864 us, tiled image 2532 -> 2538, image from a graph no difference.)
+    if (warp == 9 || warp == 10) {
+      named_barrier(6, 256 + 64);
+      if (__builtin_expect(abort_flag[0] != 0, 0) && lane == 0) {
+        mma_commit(&sh.mma_done[warp - 9]);
+        mbar_drain(&sh.mma_done[warp - 9], 0);
+      }
+      __syncwarp();
+      named_barrier_arrive(7, 96);
+    }
     if (warp == 8) {
-      named_barrier(6, 256 + 32);
+      named_barrier(7, 96);
       tc_fence_after_sync();
       tmem_dealloc(tmem, TMEM_COLS);
     }
@@ -471,7 +485,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
       return reinterpret_cast<uint4*>(sQ + tile * TILE_BYTES + (c16 >> 3) * kSubTileBytes + r * 128 + (((c16 & 7) ^ (r & 7)) << 4));
     };
     // the last read of TMEM is done: it may be given back
-    auto tmem_done = [&]() { tc_fence_before_sync(); named_barrier_arrive(6, 256 + 32); };
+    auto tmem_done = [&]() { tc_fence_before_sync(); named_barrier_arrive(6, 256 + 64); };
     if (has_B) {
       // Two row tiles: a group owns its rows.  Normalise, round, store the tile over its Q tile (read for the last time
       // by the MMAs that pv_done covers) and let TMA write it out (tokens past n are clipped).

@@ -85,7 +85,16 @@ __device__ __forceinline__ bool mbar_wait_spin(uint64_t* bar, uint32_t parity, v
   }
 }
 
-// The same bounded spin until a counter in shared memory has reached `want`.
+// Wait before memory is given up that copies or MMAs in flight may still use, for exits after a wait that ran out.  Not ended by the
+// abort flag, since what was issued completes whether or not somebody has given up, nor by the context's limit, which may be too
+// short for it.  Bounded by a number of polls (each suspends the thread for a while): the fewest instructions, since what they cost
+// is the place that they take among the code of the ordinary path (with mbar_wait's clock: video 7850 -> 7900 us).
+__device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity) {
+#pragma unroll 1
+  for (int i = 0; i < (1 << 22) && !mbar_try_wait(bar, parity); ++i) {}
+}
+
+// The same bounded spin as mbar_wait_spin until a counter in shared memory has reached `want`.
 __device__ __forceinline__ bool word_wait_spin(volatile int* word, int want, volatile int* wait_ctl) {
   if (*word >= want) return true;
   const long long t0 = clock64();
