@@ -4,6 +4,7 @@
 // cores; softmax, masking and the score reduction run on the CUDA cores in fp32.
 #pragma once
 #include <cuda.h>
+#include <stddef.h>
 #include "geom.cuh"
 #include "ptx.cuh"
 
@@ -73,6 +74,7 @@ struct TcSmemAttn {
   int s_issued;              // two row tiles: the last item whose S has been issued
   int wait_ctl[2];           // [0] abort flag, [1] wait limit in units of 1024 cycles (see mbar_wait)
 };
+static_assert(offsetof(TcSmemAttn, kv_full) == offsetof(TcSmemAttn, q_full) + 2 * sizeof(uint64_t));   // (walked as one array)
 
 template <int D, int R>
 __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
@@ -172,10 +174,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
     reg_dec<56>();                               // (with 64 or 72 the compiler spills in the softmax groups of some forms: 2 - 8 % slower)
     // Ring: K tiles go round the first kSlots slots, V tiles round the others.
     constexpr int kSlots = kStages / 2;
+    uint32_t loads = ~3u;                          // per barrier, q_full and kv_full: the parity of the last phase that loads complete
     auto load_tile = [&](int j, int v) {           // K (v = 0) or V (1) of local key tile j; false: gave up
       const int slot = v * kSlots + j % kSlots, round = j / kSlots, kt = t_begin + j;
       if (round > 0 && !mbar_wait(&sh.kv_empty[slot], (round - 1) & 1, abort_flag)) return false;
       mbar_expect_tx(&sh.kv_full[slot], TILE_BYTES);
+      loads ^= 4u << slot;
       uint8_t* dst = ring + slot * TILE_BYTES;
       if (kt < Tc) {                             // cache rows kt*128 .. (rows past n_c are masked by the softmax)
         for (int sub = 0; sub < NSUB; ++sub) tma_load_4d(dst + sub * kSubTileBytes, v ? &tm_v : &tm_k, &sh.kv_full[slot], sub * 64, kt * 128, g, layer);
@@ -229,6 +233,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
           if (j < Tl && !load_tile(j, 0)) break;
           if (j > fill && !load_tile(j - 1, 1)) break;
         }
+        // The block keeps its shared memory until they have landed, whoever has given up waiting for them.  (Barriers without a
+        // load are in their first phase, and the one before counts as complete.  Requests: no difference beyond their spread.)
+        if (!has_B) loads |= 2u;
+#pragma unroll 1
+        for (int i = 0; i < 2 + kStages; ++i) mbar_drain(&sh.q_full[0] + i, loads >> i & 1);
       }
     } else if (warp == 11) {
       // ---------------------------------------------------------------- a0 append (Alg. 1: C <- C u (K_i, V_i))

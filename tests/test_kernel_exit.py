@@ -61,3 +61,13 @@ def test_attention_keeps_tensor_memory_until_its_mmas_are_done(emulator, shape):
     # MMAs that outlast the limit
     faults, status = emulator(kernel="attention", limit_ms=20, mma_us=40000, **shape)
     assert status == KVC_ETIMEOUT and not [f for f in faults if "TMEM" in f or "MMA" in f]
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_attention_waits_for_its_loads(emulator, shape):
+    # loads that land long after everybody has given up: Q and the first tiles, or the last key tile's
+    key_tiles = ((shape["n"] + 127) // 128 + (shape["n_c"] + 127) // 128) // shape.get("split", 1)
+    loads = shape["row_tiles"] + 2 * key_tiles
+    for late in ((0, 1, 2, 3), (loads - 2, loads - 1)):
+        faults, status = emulator(kernel="attention", limit_ms=20, load_ms=",".join(f"{i}:150" for i in late), **shape)
+        assert (faults, status) == ([], KVC_ETIMEOUT), late
