@@ -659,7 +659,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
                                  rows_per * RS * 4, dsmem_addr(smem_u32(&sh.comb_full), owner));
           }
         }
-        ok = mbar_wait(&sh.comb_full, 0, abort_flag) && ok;    // the other ranks' rows have landed
+        // The other ranks' rows have landed.  They are sent whoever has given up, so they are waited for in any case: this CTA's
+        // shared memory must not go while they are on their way.
+        if (__builtin_expect(!mbar_wait(&sh.comb_full, 0, abort_flag), 0)) mbar_drain(&sh.comb_full, 0);
         if (S == 8) {
           // (16 rows per owner: two warps with a row per thread would be alone; every thread takes a piece of a row)
           constexpr int CW = 16;                                 // columns per work item: (row, piece)

@@ -71,3 +71,12 @@ def test_attention_waits_for_its_loads(emulator, shape):
     for late in ((0, 1, 2, 3), (loads - 2, loads - 1)):
         faults, status = emulator(kernel="attention", limit_ms=20, load_ms=",".join(f"{i}:150" for i in late), **shape)
         assert (faults, status) == ([], KVC_ETIMEOUT), late
+
+
+def test_attention_waits_for_the_copies_of_its_cluster(emulator):
+    # its own key tiles are late, so that it has given up when the other CTAs' partial rows are still on their way to it
+    faults, status = emulator(kernel="attention", limit_ms=20, load_ms="1:60", copy_ms=200, **SHAPES[2])
+    assert (faults, status) == ([], KVC_ETIMEOUT)
+    # nothing but those copies is late
+    faults, status = emulator(kernel="attention", limit_ms=30, copy_ms=200, **SHAPES[2])
+    assert (faults, status) == ([], KVC_ETIMEOUT)
