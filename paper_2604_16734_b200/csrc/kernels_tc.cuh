@@ -331,7 +331,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
     // and every warp leaves when it is done (requests: video 7944 -> 7855 us, query-agnostic 1268 -> 1261, image 2652 -> 2643).
     // The softmax warps may be here without their results, when a wait ran out.  Then an issuer can have MMAs under way, or a
     // tile can have landed for it that it issued some on: it comes here behind its loop and sees them to their end.
-    // (Requests: video 7852 -> 7864 us, tiled image 2532 -> 2538, image from a graph no difference.)
+    // (The price is the room of this code among the other: image 2627 -> 2643 us, video 7852 -> 7864, tiled image and image from a
+    // graph within their spread.  With a flag of its own, so that warp 8 need not come behind the issuers: video 7935.)
     if (warp == 9 || warp == 10) {
       named_barrier(6, 256 + 64);
       if (__builtin_expect(abort_flag[0] != 0, 0) && lane == 0) {
