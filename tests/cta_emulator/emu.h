@@ -76,6 +76,7 @@ inline void engine() {
       b.tx -= bytes;
       advance(b);
       if (bar == copies_bar) --copies_flying; else --loads_flying;
+      if (bar != copies_bar && !tmem_held) fault("a load lands when TMEM has been given back");   // (what the block does by then)
       cv.notify_all();
     }
     while (!pipe.empty() && (pipe.front().commit || mma_at + std::chrono::microseconds(mma_us) <= now)) {

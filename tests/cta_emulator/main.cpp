@@ -53,6 +53,8 @@ int main(int argc, char** argv) {
     if (R == 2) emu::block_idx.x = emu::grid_dim.x - 1;
     rc = R == 1 ? call(kvc::attn_tc_kernel<64, 1>) : call(kvc::attn_tc_kernel<64, 2>);
   }
+  if (args["kernel"] == "compress")
+    rc = emu::run(kvc::kCompressThreads, [&] { kvc::compress_kernel<64, kvc::kScoreAttention, 128>(tm, tm, tm, nullptr, cache.data(), ws.data(), g, 1, 2); });
   printf("status %d\n", *reinterpret_cast<int*>(ws.data()));
   return rc;
 }

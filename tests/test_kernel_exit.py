@@ -80,3 +80,14 @@ def test_attention_waits_for_the_copies_of_its_cluster(emulator):
     # nothing but those copies is late
     faults, status = emulator(kernel="attention", limit_ms=30, copy_ms=200, **SHAPES[2])
     assert (faults, status) == ([], KVC_ETIMEOUT)
+
+
+def test_compress_that_nothing_holds_up(emulator):
+    assert emulator(kernel="compress", limit_ms=5000, n_c=900, budget=900) == ([], 0)
+
+
+@pytest.mark.parametrize("late", [dict(load_ms="0:150,1:150,2:150"), dict(load_ms="3:150,4:150"), dict(mma_us=40000)])
+def test_compress_waits_for_its_loads_and_mmas(emulator, late):
+    # the selection lays its tables over the tiles, and tensor memory goes back before it
+    faults, status = emulator(kernel="compress", limit_ms=20, n_c=900, budget=900, **late)
+    assert (faults, status) == ([], KVC_ETIMEOUT)
