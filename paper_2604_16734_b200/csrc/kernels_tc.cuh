@@ -822,14 +822,15 @@ __global__ void __launch_bounds__(128) score_tc_kernel(const __grid_constant__ C
   float acc[2] = {0.f, 0.f};
   bool ok = true;
   const int n_groups = (p.w + tok_per_group - 1) / tok_per_group;
-  for (int grp = 0; grp < n_groups && ok; ++grp) {
+  int grp = 0, issued = 0;                                             // (thread 0: groups whose products have been issued)
+  for (; grp < n_groups; ++grp) {
     const int t_first = p.n - p.w + grp * tok_per_group;               // first observer token of the group
     const int t_cnt = min(tok_per_group, p.n - t_first);
     const int cols = t_cnt * p.G;                                      // real observer columns
     const int n_mma = (cols + 15) & ~15;                               // MMA N: multiple of 16, <= 256
-    // everyone is past the previous group's TMEM reads and smem reads
+    // everyone is past the previous group's TMEM reads and smem reads, and all go on or, if a wait ran out, none
     tc_fence_before_sync();
-    __syncthreads();
+    if (!__syncthreads_and(ok)) { ok = false; break; }
     for (int c = threadIdx.x; c < 256; c += blockDim.x) {
       float lv = INFINITY;                                             // padding column: 2^-inf = 0
       if (c < cols) lv = lse[static_cast<long long>(t_first + c / p.G) * p.Hq + g * p.G + c % p.G] * 1.4426950408889634f;
@@ -851,12 +852,13 @@ __global__ void __launch_bounds__(128) score_tc_kernel(const __grid_constant__ C
           mma_ss(tmem, smem_desc_sw128(aK + (kk / 4) * kSubTileBytes + (kk % 4) * 32, 16, 1024),
                  smem_desc_sw128(aQ + (kk / 4) * kQSubBytes + (kk % 4) * 32, 16, 1024), idesc, kk > 0);
         mma_commit(&sh.bar_s);
+        ++issued;
       }
     }
     __syncwarp();
     __syncthreads();                                                   // lse2 visible
-    ok = mbar_wait(&sh.bar_s, grp & 1, abort_flag);
-    if (!ok) break;
+    ok = __all_sync(0xffffffffu, mbar_wait(&sh.bar_s, grp & 1, abort_flag));   // (a warp reads TMEM as one)
+    if (!ok) continue;
     tc_fence_after_sync();
     for (int c0 = 0; c0 < n_mma; c0 += 32) {                           // the second half may be absent
       uint32_t sr[32];
@@ -874,6 +876,13 @@ __global__ void __launch_bounds__(128) score_tc_kernel(const __grid_constant__ C
   }
   const int key = key0 + threadIdx.x;
   if (ok && key < p.n_cand) score[key] = acc[0] + acc[1];
+  // Thread 0 has given up: not before its loads and MMAs are complete does the block give up what they use.  (Asked without need
+  // they cost 0.4 - 0.9 of the 36 - 41 us of a call with 384 or 448 observer rows.)
+  if (threadIdx.x == 0 && __builtin_expect(!ok, 0)) {
+    mbar_drain(&sh.bar_k, 0);
+    mbar_drain(&sh.bar_q, (grp - 1) & 1);                              // (groups 0 .. grp - 1 have been loaded)
+    if (issued > 0) mbar_drain(&sh.bar_s, (issued - 1) & 1);
+  }
   tc_fence_before_sync();
   __syncthreads();
   if (warp == 0) {

@@ -55,6 +55,8 @@ int main(int argc, char** argv) {
   }
   if (args["kernel"] == "compress")
     rc = emu::run(kvc::kCompressThreads, [&] { kvc::compress_kernel<64, kvc::kScoreAttention, 128>(tm, tm, tm, nullptr, cache.data(), ws.data(), g, 1, 2); });
+  if (args["kernel"] == "score")
+    rc = emu::run(128, [&] { kvc::score_tc_kernel<64>(tm, tm, ws.data(), g, 256); });
   printf("status %d\n", *reinterpret_cast<int*>(ws.data()));
   return rc;
 }

@@ -37,7 +37,8 @@ def emulator(tmp_path_factory):
                     os.path.join(HERE, "cta_emulator", "main.cpp"), "-o", exe], check=True)
 
     def run(**kw):
-        r = subprocess.run([exe] + [f"{k}={v}" for k, v in kw.items()], capture_output=True, text=True, timeout=60)
+        r = subprocess.run(["timeout", "20", exe] + [f"{k}={v}" for k, v in kw.items()], capture_output=True, text=True)
+        assert r.returncode != 124, "the kernel does not end"
         lines = r.stdout.splitlines()
         assert lines and lines[-1].startswith("status"), r.stdout + r.stderr
         return [x[len("FAULT "):] for x in lines[:-1]], int(lines[-1].split()[1])
@@ -90,4 +91,16 @@ def test_compress_that_nothing_holds_up(emulator):
 def test_compress_waits_for_its_loads_and_mmas(emulator, late):
     # the selection lays its tables over the tiles, and tensor memory goes back before it
     faults, status = emulator(kernel="compress", limit_ms=20, n_c=900, budget=900, **late)
+    assert (faults, status) == ([], KVC_ETIMEOUT)
+
+
+def test_score_that_nothing_holds_up(emulator):
+    assert emulator(kernel="score", limit_ms=5000, n=512, w=512) == ([], 0)
+
+
+@pytest.mark.parametrize("late", [dict(load_ms="0:150,1:150"), dict(load_ms="2:150"), dict(mma_us=40000),
+                                  dict(mma_us=20000, suspend_ms="3:400")])
+def test_score_waits_for_its_loads_and_mmas(emulator, late):
+    # (the last one: a warp still sees the first group's products, and those that have given up leave with it)
+    faults, status = emulator(kernel="score", limit_ms=20, n=512, w=512, **late)
     assert (faults, status) == ([], KVC_ETIMEOUT)
