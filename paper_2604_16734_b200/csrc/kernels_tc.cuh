@@ -56,12 +56,12 @@ template <int R> __host__ __device__ constexpr int attn_stages() { return R == 1
 // Row tiles per CTA: R = 2 as described, or R = 1.  A CTA with one row tile runs it twice over: softmax group t takes its
 // key tiles t, t+2, ... with P, O, maximum and row sum of its own (tile B's TMEM columns), and
 // the two partial results are merged at the end, column half by column half straight from TMEM.  That doubles the CTA
-// count at about 1.06 times the cost per row tile and key tile.
-// What bounds a launch (device stamps, us): 1.3 until the first S (dependency wait, TMA, MMA), then 0.80 per key tile
-// with one row tile or 1.66 with two, 1.5 for the epilogue, 2.7 for the combine of a key split.  With the output through
-// shared memory, the merge from TMEM, the six-slot ring and cluster barriers that order no memory: tiled image (13 key
-// tiles, 128 CTAs) 16.4 -> 14.5, video (18 key tiles split over two, 112 CTAs) 17.5 -> 15.3; two row tiles (long video)
-// 73.3 -> 73.1.
+// count at 0.80 per row tile and key tile, against half of 1.66 in a pair.
+// What bounds a launch (device stamps, us): 1.3 - 1.4 until the first S (dependency wait, TMA, MMA), then 0.80 per key tile
+// with one row tile or 1.66 with two, 1.5 - 1.7 for the epilogue, about 3.5 for the combine of a key split.
+// (While S lay under P, 0.94 and 1.78 a key tile: with the output through shared memory, the merge from TMEM, the six-slot ring
+// and cluster barriers that order no memory, tiled image (13 key tiles, 128 CTAs) 16.4 -> 14.5, video (18 key tiles split over
+// two, 112 CTAs) 17.5 -> 15.3; two row tiles (long video) 73.3 -> 73.1.)
 // grid (R == 1 ? tiles * S : tiles - n_pairs, Hkv, nl) with tiles = ceil(n/TOK), cluster (S,1,1), block 384,
 // dynamic smem (R + attn_stages<R>()) * (D/64) * 16 KB + 1 KB.
 static constexpr int kAttnThreads = 384;
@@ -122,9 +122,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
   const int T = Tc + (last_tok + 128) / 128;
   const int t_begin = split * T / S, t_end = (split + 1) * T / S;
   const int Tl = t_end - t_begin;                // key tiles of this CTA (0 is possible when S > T)
-  // A CTA with one row tile runs it twice over: softmax group t takes the key tiles t, t+2, ... with accumulators, maxima and sums of their own (the TMEM columns of tile B are free), two key tiles are in flight as
-  // with two row tiles, and the two partial results are merged at the end.  (With Tl = 1 group 1 has none; Tl = 0
-  // happens with a key split, for the first rows of a block that see less of it than the last ones.)
+  // A CTA with one row tile runs it twice over: softmax group t takes the key tiles t, t+2, ... with accumulators, maxima and sums
+  // of their own (the TMEM columns of tile B are free), two key tiles are in flight as with two row tiles, and the two partial
+  // results are merged at the end.  (With Tl = 1 group 1 has none; Tl = 0 happens with a key split, for the first rows of a block
+  // that see less of it than the last ones.)
   const bool alt = !has_B;
   const int n_it0 = alt ? (Tl + 1) / 2 : Tl, n_it1 = alt ? Tl / 2 : Tl;   // key tiles of group 0 / 1
 
@@ -497,8 +498,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_tc_kernel(const __grid_c
     // the last read of TMEM is done: it may be given back
     auto tmem_done = [&]() { tc_fence_before_sync(); named_barrier_arrive(6, 256 + 64); };
     if (has_B) {
-      // Two row tiles: a group owns its rows.  Normalise, round, store the tile over its Q tile (read for the last time
-      // by the MMAs that pv_done covers) and let TMA write it out (tokens past n are clipped).
+      // Two row tiles: a group owns its rows.  Normalise, round, store the tile over its Q tile and let TMA write it out (tokens
+      // past n are clipped).  Nothing reads that Q tile any more: this group has had its last S (s_full), which is what its last P
+      // was made from, and only the S of its own row tile are made from it.
       ok = ok && mbar_wait(&sh.pv_done[t], (Tl - 1) & 1, abort_flag);
       ok = __all_sync(0xffffffffu, ok);                       // the TMEM accesses below are warp-wide
       if (ok) {

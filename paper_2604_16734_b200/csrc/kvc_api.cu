@@ -546,17 +546,19 @@ static cudaError_t launch_cc_score(const Geom& g, int dev, const void* q, const 
 }
 
 // Launch shape of the tensor-core attention: R row tiles per CTA (1 or 2) and, with one, the key split S over a cluster.
-// The shapes are compared with a model of the kernel's duration fitted to device stamps of all five shapes on sixteen
-// configurations (us): a key tile costs 1.78 per pair of row tiles taking turns and 0.94 for a single tile (whose two
-// softmax groups take alternate key tiles), a CTA 4.3 around them, the combine 2.7 (3.7 over eight CTAs); CTAs beyond
-// what is resident at a time (one per SM; 32 clusters of four, 14 of eight) run as further waves.  Measured, R=2 / R=1 S=1 /
+// The shapes are compared with a model of the kernel's duration.  It was fitted to device stamps of all five shapes on sixteen
+// configurations while S still lay under P (us): a key tile cost 1.78 per pair of row tiles taking turns and 0.94 for a
+// single tile (whose two softmax groups take alternate key tiles), a CTA 4.3 around them, the combine 2.7 (3.7 over eight CTAs); CTAs beyond
+// what is resident at a time (one per SM; 32 clusters of four, 14 of eight) run as further waves.  Measured then, R=2 / R=1 S=1 /
 // S=2 / S=4 / S=8:  196 x 4 rows, 8 kv-heads, 2244 keys 35.3 / 20.6 / 15.7 / 25.2 / 46.2;  576 x 7, 4, 1600 keys 28.2 /
 // 17.0 / 27.3 / 45.9 / 92.9;  784 x 7, 4, 2832 keys 46.6 / 46.9 / 52.7;  1000 x 1, 32, 1500 keys 29.3 / 33.7 / 51.4;
 // 256 x 4, 2, 1280 keys 21.3 / 12.9 / 10.9 / 9.3 / 18.1;  100 x 3, 4, 4100 keys 61.4 / 33.2 / 21.5 / 14.9 / 12.6;
-// 128 x 1, 32, 320 keys 7.2 / 7.2 / 9.2 / 7.8 / 25.7.  On all sixteen the model picks the fastest or is within 1 %.
-// (Fitted, and the figures taken, while S still lay under P; since then a key tile costs 0.80 and 1.66.  The rule stays: the shape
-// groups a row's keys, which decides the last bits of its log-sum-exp and, between candidates whose scores agree to seven
-// digits, which of them is retained.)
+// 128 x 1, 32, 320 keys 7.2 / 7.2 / 9.2 / 7.8 / 25.7.
+// Since S has columns of its own a key tile costs 1.66 and 0.80, and the combine about 3.5.  Neither the figures above nor the
+// constants have been taken again: with them some launches of three to six key tiles would not be split over four CTAs, and a
+// last wave that is not full is charged as a full one.  (A changed shape groups a row's keys differently: the last bits of its
+// log-sum-exp, and which of two candidates with scores that agree to seven digits is retained, may change with it.  Both are
+// right; what has to be the same bits is a call with compress on a side stream and in stream order.)
 // (An exchange of the partials through an L2-resident global buffer instead of distributed shared memory was measured
 // too: slower, the release / acquire round trip costs more than the narrow SM-to-SM path.)
 struct AttnShape { int R, S, n_pairs; long long ctas; };
@@ -576,9 +578,9 @@ static AttnShape attn_launch_shape(const Geom& g, bool allow_split, bool evict) 
   AttnShape best = {2, 1, tiles / 2, (tiles - tiles / 2) * heads};
   double best_us = tiles == 1 ? INFINITY : waves(best.ctas, kvc::kNumSMs) * (T * 1.78 + 4.3);   // a single row tile never fills a pair
   // Pairs that would leave SMs idle: the row tiles with the most keys, the last ones, get a CTA each instead (1.2 us per
-  // key tile there: their ring has four slots).  784 x 7 rows, 4 kv-heads, 2832 keys: 46.5 -> 38.2 us; 640 x 4, 8, d = 64
-  // 31.5 -> 25.7; 1024 x 4, 8, 5120 keys 78.4 -> 76.6, all without the reserve.  With it, requests with compress on a side
-  // stream take, against none: 700 x 1 rows, 32 kv-heads 469 -> 411 us, 640 x 4, 8, d = 64 620 -> 604, 1024 x 4,
+  // key tile there, measured with K and V tiles going round all four slots of their ring; now each kind has two).
+  // 784 x 7 rows, 4 kv-heads, 2832 keys: 46.5 -> 38.2 us; 640 x 4, 8, d = 64 31.5 -> 25.7; 1024 x 4, 8, 5120 keys
+  // 78.4 -> 76.6, all without the reserve.  With it, requests with compress on a side stream take, against none: 700 x 1 rows, 32 kv-heads 469 -> 411 us, 640 x 4, 8, d = 64 620 -> 604, 1024 x 4,
   // 8 2654 -> 2589, 784 x 7, 4 891 -> 898.
   const long long per_head = (kvc::kNumSMs - reserve) / heads;
   if (per_head > tiles - tiles / 2 && per_head < tiles) {
